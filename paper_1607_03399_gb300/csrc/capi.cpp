@@ -274,6 +274,16 @@ void fill_ops(const RefElems& R, std::vector<unsigned char>& out) {
     for (int m = 0; m < Nq; ++m) o.tab.edge[e][m] = int8_t(R.edge_nodes[e][m]);
   for (int f = 0; f < 4; ++f)
     for (int k = 0; k < Nt; ++k) o.tab.tet_face[f][k] = int8_t(R.tet_face_nodes[f][k]);
+  // Cholesky factor of the line mass as the device holds it, C[j][m] = L[m][j] (m >= j)
+  for (int j = 0; j < Nq; ++j)
+    for (int m = j; m < Nq; ++m) {
+      double v = double(o.w.M1[m * Nq + j]);
+      for (int k = 0; k < j; ++k) v -= o.M1C[k * Nq + j] * o.M1C[k * Nq + m];
+      o.M1C[j * Nq + m] = m == j ? std::sqrt(v) : v / o.M1C[j * Nq + j];
+    }
+  for (int a = 0; a < 3; ++a)
+    for (int i = 0; i < Nt; ++i)
+      for (int l = 0; l <= i; ++l) o.MaL[a][i * (i + 1) / 2 + l] = double(o.w.Ma[a][i * Nt + l]) * (l == i ? 0.5 : 1.0);
   out.resize(sizeof(o));
   std::memcpy(out.data(), &o, sizeof(o));
 }
@@ -393,7 +403,7 @@ int64_t nsrc_dev(const dg_ctx* c) {
 BlobLayout blob_layout(const dg_ctx* c) {
   const size_t rs = c->prec == DG_F64 ? 8 : 4;
   const int64_t Kwp = nblk(vKw(c)) * kB, Ktp = nblk(vKt(c)) * kB;
-  const int64_t nparts = (nblk(vKw(c)) + 3) / 4 + (nblk(vKt(c)) + 3) / 4 + 1;
+  const int64_t nparts = nblk(vKw(c)) + nblk(vKt(c)) + 1;
   BlobLayout L;
   size_t o = 0;
   auto take = [&](size_t bytes) {

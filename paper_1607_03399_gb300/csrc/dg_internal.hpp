@@ -69,6 +69,10 @@ template <int N, typename real>
 struct AllOps {
   WedgeOps<N, real> w;
   Tables<N> tab;
+  // energy: upper triangular C with M^1D = C^T C, and the packed lower
+  // triangles of the three M_a with half their diagonals
+  alignas(8) double M1C[(N + 1) * (N + 1)];
+  double MaL[3][nt_of(N) * (nt_of(N) + 1) / 2];
 };
 
 // Point source in the pressure equation: rhs_p += amp R(f0, t - t0) g, with
@@ -116,7 +120,7 @@ struct DevMesh {
   int64_t tet_off = 0;               // first real of the tet region in a field buffer
   int64_t total_nodes = 0;           // canonical nodes
   int* err = nullptr;                // device error word
-  double* partials = nullptr;        // per-block energy partial sums
+  double* partials = nullptr;        // energy sums, one per 32-element block
   double* energy = nullptr;          // final energy
   const real* tet_mass = nullptr;    // reference tet mass matrix (energy only)
   const SourceDev* src = nullptr;    // point sources

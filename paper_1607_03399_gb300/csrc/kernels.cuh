@@ -1560,102 +1560,172 @@ __global__ void __launch_bounds__(256) k_pack(const DevMesh<real> M, const real*
 // ---------------------------------------------------------------------------
 // discrete energy (Section 4.1), double accumulation, deterministic order
 // ---------------------------------------------------------------------------
+// One CTA per 32-element block (lane = element), warp f takes field f.
+// Bound by the FP64 pipe (2 multiply-adds per cycle and SM), so the layout
+// follows from the operation count: M^1D = C^T C turns the quadratic form of
+// M^{tri,k} (x) M^1D into sum_j y_j^T M^{tri,k} y_j with y = (C (x) I) q, each
+// of those a symmetric form on its lower triangle (Nt (Nt + 3) / 2 operations
+// instead of the Nq Nt^2 of every slice pair), and the block forms the entries
+// of M^{tri,k} once in shared memory for its four fields.  At N = 3: 1,605
+// FP64 multiply-adds per wedge against 25,600 (each slice pair re-forming the
+// mass entries in every thread).  FP32 state, 524,288 wedges, N = 3: 50.3 ms
+// -> 2.0 ms (0.63 T multiply-adds/s of FP64 allow 1.3 ms); 128 wedges, FP64: 1.25 ms
+// -> 22 us.
+template <int N>
+__host__ __device__ constexpr int energy_smem_bytes() {
+  return nt_of(N) * (nt_of(N) + 1) / 2 * kB * 8;
+}
+
 template <int N>
 __global__ void __launch_bounds__(128) k_energy(const DevMesh<real> M, const real* __restrict__ q) {
-  constexpr int Nt = nt_of(N), Nq = N + 1, Npw = npw_of(N), Npt = npt_of(N);
+  constexpr int Nt = nt_of(N), Nq = N + 1, Npt = npt_of(N);
   const AllOps<N, real>& O = OPS<N>();
-  const int nblk_cta_w = (M.nblk_w + 3) / 4;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  double* sM = reinterpret_cast<double*>(smem_raw);  // [Nt (Nt + 1) / 2][32]
+  __shared__ double red[4];
+  const int lane = threadIdx.x & 31, f = threadIdx.x >> 5;
   double E = 0.0;
-  const int gw = blockIdx.x * 4 + (threadIdx.x >> 5);  // 32-element block handled by this warp
-  const int lane = threadIdx.x & 31;
-  if (blockIdx.x < nblk_cta_w) {
-    const int e = gw * kB + lane;
-    if (gw < M.nblk_w && e < M.Kw) {
-      const int Kp = M.Kw_pad;
-      const int vb0 = M.w_vid[0 * Kp + e], vb1 = M.w_vid[1 * Kp + e], vb2 = M.w_vid[2 * Kp + e];
-      const double x0 = M.vx[vb0], x1 = M.vx[vb1], x2 = M.vx[vb2];
-      const double y0 = M.vy[vb0], y1 = M.vy[vb1], y2 = M.vy[vb2];
-      const double A = 0.25 * ((x1 - x0) * (y2 - y0) - (x2 - x0) * (y1 - y0));
-      double Ja[3];
-      for (int a = 0; a < 3; ++a) Ja[a] = 0.5 * A * (double(M.vz[M.w_vid[(3 + a) * Kp + e]]) - double(M.vz[M.w_vid[a * Kp + e]]));
-      const double wgt[4] = {1.0 / double(M.w_mat[0 * Kp + e]), 1.0 / double(M.w_mat[1 * Kp + e]),
-                             1.0 / double(M.w_mat[1 * Kp + e]), 1.0 / double(M.w_mat[1 * Kp + e])};
+  if (int(blockIdx.x) < M.nblk_w) {
+    const int blk = blockIdx.x, e = blk * kB + lane;
+    {
+      // J_a = A h_a / 2 at the three columns, from the block's vertex table
+      const real* X = M.w_xyz + int64_t(blk) * 12 * kB + lane;
+      auto x = [&](int i) { return double(X[i * kB]); };
+      const double A = 0.25 * ((x(1) - x(0)) * (x(5) - x(3)) - (x(2) - x(0)) * (x(4) - x(3)));
+      const double J0 = 0.5 * A * (x(9) - x(6)), J1 = 0.5 * A * (x(10) - x(7)), J2 = 0.5 * A * (x(11) - x(8));
+      // this warp's entries of the packed lower triangle (half the diagonal:
+      // the form is twice its lower triangle)
 #pragma unroll 1
-      for (int f = 0; f < 4; ++f) {
-        double ef = 0.0;
-#pragma unroll 1
-        for (int jp = 0; jp < Nq; ++jp)
-#pragma unroll 1
-          for (int jj = 0; jj < Nq; ++jj) {
-            const double m1 = double(O.w.M1[jj * Nq + jp]);
-            double d = 0.0;
-#pragma unroll 1
-            for (int i = 0; i < Nt; ++i) {
-              double s = 0.0;
-#pragma unroll 1
-              for (int l = 0; l < Nt; ++l) {
-                const double mt = Ja[0] * double(O.w.Ma[0][i * Nt + l]) + Ja[1] * double(O.w.Ma[1][i * Nt + l]) +
-                                  Ja[2] * double(O.w.Ma[2][i * Nt + l]);
-                s += mt * double(q[widx<N>(gw, jp * Nt + l, lane) + f]);
-              }
-              d += double(q[widx<N>(gw, jj * Nt + i, lane) + f]) * s;
-            }
-            ef += m1 * d;
+      for (int at = f; at < Nt * (Nt + 1) / 2; at += 4)
+        sM[at * kB + lane] = J0 * O.MaL[0][at] + J1 * O.MaL[1][at] + J2 * O.MaL[2][at];
+    }
+    __syncthreads();
+    if (e < M.Kw) {
+      const real* qf = q + widx<N>(blk, 0, lane) + f;
+      if constexpr (N <= 3) {
+        // all slices at once: a node value is converted to double once (a
+        // conversion takes the FP64 pipe as long as a multiply-add)
+        double y[Nq][Nt];
+#pragma unroll
+        for (int i = 0; i < Nt; ++i) {
+#pragma unroll
+          for (int j = 0; j < Nq; ++j) y[j][i] = 0.0;
+#pragma unroll
+          for (int m = 0; m < Nq; ++m) {
+            const double v = double(qf[(m * Nt + i) * (kB * 4)]);
+#pragma unroll
+            for (int j = 0; j <= m; ++j) y[j][i] += O.M1C[j * Nq + m] * v;
           }
-        E += wgt[f] * ef;
+        }
+#pragma unroll
+        for (int i = 0; i < Nt; ++i) {
+          double s[Nq];
+#pragma unroll
+          for (int j = 0; j < Nq; ++j) s[j] = 0.0;
+#pragma unroll
+          for (int l = 0; l <= i; ++l) {
+            const double m = sM[(i * (i + 1) / 2 + l) * kB + lane];
+#pragma unroll
+            for (int j = 0; j < Nq; ++j) s[j] += m * y[j][l];
+          }
+#pragma unroll
+          for (int j = 0; j < Nq; ++j) E += s[j] * y[j][i];
+        }
+      } else {
+        // slice by slice: y of all slices would not fit the registers
+#pragma unroll 1
+        for (int j = 0; j < Nq; ++j) {
+          double y[Nt];
+#pragma unroll
+          for (int i = 0; i < Nt; ++i) y[i] = 0.0;
+#pragma unroll 1
+          for (int m = j; m < Nq; ++m) {
+            const double cj = O.M1C[j * Nq + m];
+#pragma unroll
+            for (int i = 0; i < Nt; ++i) y[i] += cj * double(qf[(m * Nt + i) * (kB * 4)]);
+          }
+          // (the mass entries are read again for every slice: held in registers
+          // across the slices they would cost most of the warps in flight)
+          asm volatile("" ::: "memory");
+#pragma unroll
+          for (int i = 0; i < Nt; ++i) {
+            double s = 0.0;
+#pragma unroll
+            for (int l = 0; l <= i; ++l) s += sM[(i * (i + 1) / 2 + l) * kB + lane] * y[l];
+            E += s * y[i];
+          }
+        }
       }
+      E = 2.0 * E / double(M.w_mat[(f == 0 ? 0 : 1) * M.Kw_pad + e]);
     }
   } else {
-    const int gt = gw - nblk_cta_w * 4;
-    const int e = gt * kB + lane;
-    if (gt < M.nblk_t && e < M.Kt) {
-      const int Kp = M.Kt_pad;
+    const int blk = int(blockIdx.x) - M.nblk_w, e = blk * kB + lane;
+    if (e < M.Kt) {
       double X[4][3];
-      for (int v = 0; v < 4; ++v) {
-        const int id = M.t_vid[v * Kp + e];
-        X[v][0] = M.vx[id];
-        X[v][1] = M.vy[id];
-        X[v][2] = M.vz[id];
-      }
+#pragma unroll
+      for (int v = 0; v < 4; ++v)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) X[v][d] = double(M.t_xyz[(int64_t(blk) * 12 + v * 3 + d) * kB + lane]);
       double G[3][3];
+#pragma unroll
       for (int d = 0; d < 3; ++d)
+#pragma unroll
         for (int m = 0; m < 3; ++m) G[d][m] = 0.5 * (X[m + 1][d] - X[0][d]);
       const double J = G[0][0] * (G[1][1] * G[2][2] - G[1][2] * G[2][1]) - G[0][1] * (G[1][0] * G[2][2] - G[1][2] * G[2][0]) +
                        G[0][2] * (G[1][0] * G[2][1] - G[1][1] * G[2][0]);
-      const double wgt[4] = {1.0 / double(M.t_mat[0 * Kp + e]), 1.0 / double(M.t_mat[1 * Kp + e]),
-                             1.0 / double(M.t_mat[1 * Kp + e]), 1.0 / double(M.t_mat[1 * Kp + e])};
+      // the constant reference mass on its lower triangle, four rows at a time
+      const real* qf = q + tidx<N>(M.tet_off, blk, 0, lane) + f;
+      double d = 0.0, o = 0.0;
 #pragma unroll 1
-      for (int f = 0; f < 4; ++f) {
-        double ef = 0.0;
-#pragma unroll 1
-        for (int i = 0; i < Npt; ++i) {
-          double s = 0.0;
-#pragma unroll 1
-          for (int l = 0; l < Npt; ++l) s += double(M.tet_mass[i * Npt + l]) * double(q[tidx<N>(M.tet_off, gt, l, lane) + f]);
-          ef += s * double(q[tidx<N>(M.tet_off, gt, i, lane) + f]);
+      for (int i0 = 0; i0 < Npt; i0 += 4) {
+        double s[4] = {0.0, 0.0, 0.0, 0.0}, y[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) y[r] = i0 + r < Npt ? double(qf[(i0 + r) * (kB * 4)]) : 0.0;
+        const real* m0 = M.tet_mass + i0 * Npt;
+#pragma unroll 4
+        for (int l = 0; l < i0; ++l) {
+          const double ql = double(qf[l * (kB * 4)]);
+#pragma unroll
+          for (int r = 0; r < 4; ++r) s[r] += double(m0[(i0 + r < Npt ? r : 0) * Npt + l]) * ql;
         }
-        E += wgt[f] * J * ef;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          if (i0 + r < Npt) {
+#pragma unroll
+            for (int c = 0; c < r; ++c) s[r] += double(m0[r * Npt + i0 + c]) * y[c];
+            o += s[r] * y[r];
+            d += double(m0[r * Npt + i0 + r]) * (y[r] * y[r]);
+          }
+        }
       }
+      E = J * (d + 2.0 * o) / double(M.t_mat[(f == 0 ? 0 : 1) * M.Kt_pad + e]);
     }
   }
   // block reduction in a fixed order
-  __shared__ double red[128];
-  red[threadIdx.x] = E;
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) E += __shfl_down_sync(0xffffffffu, E, s);
+  if (lane == 0) red[f] = E;
   __syncthreads();
-  for (int s = 64; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) M.partials[blockIdx.x] = 0.5 * red[0];
-  (void)Npw;
+  if (threadIdx.x == 0) M.partials[blockIdx.x] = 0.5 * ((red[0] + red[1]) + (red[2] + red[3]));
 }
 
-__global__ void k_energy_final(const double* __restrict__ partials, int n, double* out, int* err) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < n; ++i) s += partials[i];
-    *out = s;
-    if (!isfinite(s)) atomicOr(err, kErrNonfinite);
+// the block sums in a fixed order: 1024 strided sums, then a tree
+__global__ void __launch_bounds__(1024) k_energy_final(const double* __restrict__ partials, int n, double* out, int* err) {
+  __shared__ double red[32];
+  double s = 0.0;
+  for (int i = threadIdx.x; i < n; i += 1024) s += partials[i];
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xffffffffu, s, d);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    s = red[threadIdx.x];
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xffffffffu, s, d);
+    if (threadIdx.x == 0) {
+      *out = s;
+      if (!isfinite(s)) atomicOr(err, kErrNonfinite);
+    }
   }
 }
 
@@ -1703,6 +1773,8 @@ int prepare_n() {
     err = cudaFuncSetAttribute(k_tet_stage<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, tet_smem_bytes<N>());
   if (err == cudaSuccess)
     err = cudaFuncSetAttribute(k_pack<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, pack_smem_bytes<N>());
+  if (err == cudaSuccess)
+    err = cudaFuncSetAttribute(k_energy<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, energy_smem_bytes<N>());
   // the gradient kernels where their shared memory fits one CTA (not FP64 at N = 5,
   // whose adjoint the library refuses)
   if constexpr (grad_smem_bytes<N>() <= 227 * 1024) {
@@ -1789,10 +1861,9 @@ int launch_pack_n(const DevMesh<real>& m, const real* canon, real* packed, bool 
 
 template <int N>
 int launch_energy_n(const DevMesh<real>& m, const real* q, cudaStream_t s) {
-  const int nw = (m.nblk_w + 3) / 4, nt = (m.nblk_t + 3) / 4;
-  const int grid = nw + nt;
-  if (grid > 0) k_energy<N><<<grid, 128, 0, s>>>(m, q);
-  k_energy_final<<<1, 32, 0, s>>>(m.partials, grid, m.energy, m.err);
+  const int grid = m.nblk_w + m.nblk_t;
+  if (grid > 0) k_energy<N><<<grid, 128, energy_smem_bytes<N>(), s>>>(m, q);
+  k_energy_final<<<1, 1024, 0, s>>>(m.partials, grid, m.energy, m.err);
   return int(cudaGetLastError());
 }
 
@@ -1822,13 +1893,13 @@ int DGW_CAT(launch_energy_, REALNS)(const DevMesh<REAL>& m, const REAL* q, void*
 }
 int DGW_CAT(launch_sample_, REALNS)(const DevMesh<REAL>& m, const REAL* q, REAL* out, int nshots, void* stream) {
   const int n = nshots * m.nrec;
-  if (n > 0) REALNS::k_sample<NORD><<<(n + 127) / 128, 128, 0, cudaStream_t(stream)>>>(m, q, out, nshots);
+  if (n > 0) REALNS::k_sample<NORD><<<(n + 3) / 4, 128, 0, cudaStream_t(stream)>>>(m, q, out, nshots);
   return int(cudaGetLastError());
 }
 int DGW_CAT(launch_inject_, REALNS)(const DevMesh<REAL>& m, REAL* muq, REAL* x, const REAL* resid, int nshots, REAL b5,
                                     void* stream) {
   const int n = nshots * m.nrgrp;
-  if (n > 0) REALNS::k_inject<NORD><<<(n + 127) / 128, 128, 0, cudaStream_t(stream)>>>(m, muq, x, resid, nshots, b5);
+  if (n > 0) REALNS::k_inject<NORD><<<(n + 3) / 4, 128, 0, cudaStream_t(stream)>>>(m, muq, x, resid, nshots, b5);
   return int(cudaGetLastError());
 }
 int DGW_CAT(launch_grad_, REALNS)(const DevMesh<REAL>& m, const REAL* x, const REAL* q, const REAL* r, double dt,
