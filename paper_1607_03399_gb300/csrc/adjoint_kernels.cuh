@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(128) k_inject(const DevMesh<real> M, real* __r
 template <int N>
 __host__ __device__ constexpr int grad_smem_bytes() {
   constexpr int Nt = nt_of(N), Nq = N + 1, Np = Nt * Nq;
-  return int(sizeof(real)) * (2 * 4 * Np * kB + G_COUNT * kB) + 8 * 3 * Nq * kB + 16;
+  return int(sizeof(real)) * (2 * 4 * Np * kB + (G_COUNT + 13) / 2 * 2 * kB) + 8 * 3 * Nq * kB + 16;
 }
 
 // the warp that owns triangle face fb (0 bottom, 1 top) in the gradient
@@ -110,7 +110,8 @@ __global__ void __launch_bounds__(32 * (N + 1), (sizeof(real) == 4) ? (N <= 3 ? 
   real* sX = reinterpret_cast<real*>(smem_raw);
   real* sQ = sX + 4 * Np * kB;
   real* sG = sQ + 4 * Np * kB;
-  double* red = reinterpret_cast<double*>(sG + G_COUNT * kB);  // [warp][3][32]
+  real* sC = sG + G_COUNT * kB;  // [12][32] vertex coordinates
+  double* red = reinterpret_cast<double*>(sG + (G_COUNT + 13) / 2 * 2 * kB);  // [warp][3][32]
   uint64_t* bar = reinterpret_cast<uint64_t*>(red + 3 * Nq * kB);  // slabs and coordinates
   int* failed = reinterpret_cast<int*>(bar + 1);
   const int lane = threadIdx.x & 31, j = threadIdx.x >> 5;
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(32 * (N + 1), (sizeof(real) == 4) ? (N <= 3 ? 
     mbar_expect_tx(bar, 2 * slab_bytes + xyz_bytes);
     bulk_g2s(sX, X + int64_t(blk) * 4 * Np * kB, slab_bytes, bar);
     bulk_g2s(sQ, Q + int64_t(blk) * 4 * Np * kB, slab_bytes, bar);
-    bulk_g2s(sG, M.w_xyz + int64_t(blk) * 12 * kB, xyz_bytes, bar);
+    bulk_g2s(sC, M.w_xyz + int64_t(blk) * 12 * kB, xyz_bytes, bar);
   }
   // this slice of the right-hand side, the material and the face neighbours
   // (ids, codes, impedances), in flight while the slabs arrive
@@ -155,7 +156,8 @@ __global__ void __launch_bounds__(32 * (N + 1), (sizeof(real) == 4) ? (N <= 3 ? 
     }
     return;
   }
-  if (j == 0) wedge_geometry(sG, lane);
+#pragma unroll 1
+  for (int p = j; p < kGeoParts; p += Nq) wedge_geometry_part<true>(p, sC, sG, lane);
   __syncthreads();
 #define GEO(item) sG[(item) * kB + lane]
   const real J0 = GEO(G_J0), J1 = GEO(G_J1), J2 = GEO(G_J2);

@@ -654,8 +654,8 @@ void fill_blob(const dg_ctx* c, const BlobLayout& L, std::vector<unsigned char>&
   }
   if (c->mass == DG_MASS_STORED) {
     // M^{tri,k} = sum_a J_a M_a with J_a = A h_a / 2 at the three columns
-    // (Lemma 3.1, bi-unit reference: A = x_r y_s - x_s y_r), factored L L^T in
-    // double; entry (i, l <= i) at i (i + 1) / 2 + l with 1 / L_ii on the diagonal
+    // (Lemma 3.1, bi-unit reference: A = x_r y_s - x_s y_r), factored L D L^T in
+    // double; entry (i, l < i) of -L at i (i + 1) / 2 + l, 1 / D_i on the diagonal
     const RefElems& R = *c->ref;
     const int nt = R.Nt, nl = nt * (nt + 1) / 2;
     real* fac = reinterpret_cast<real*>(blob.data() + L.wfac);
@@ -679,7 +679,12 @@ void fill_blob(const dg_ctx* c, const BlobLayout& L, std::vector<unsigned char>&
       }
       for (int i = 0; i < nt; ++i)
         for (int l = 0; l <= i; ++l)
-          one[size_t(w) * nl + i * (i + 1) / 2 + l] = real(l < i ? Lk[size_t(i) * nt + l] : 1.0 / Lk[size_t(i) * nt + i]);
+        {
+          // M = L L^T = (L S^-1) S^2 (L S^-1)^T with S = diag(L): the negated
+          // unit lower triangle and 1 / S_i^2, as the stage's sweeps use them
+          const double lii = Lk[size_t(i) * nt + i];
+          one[size_t(w) * nl + i * (i + 1) / 2 + l] = real(l < i ? -Lk[size_t(i) * nt + l] / Lk[size_t(l) * nt + l] : 1.0 / (lii * lii));
+        }
     }
     const int64_t nl4 = nl4_of(c->N);
     for (int64_t w = 0; w < Kwp; ++w) {
@@ -763,6 +768,7 @@ struct StageExtra {
   double g = 1.0;
   void* rhs_out = nullptr;
   bool no_sources = false;
+  bool res_store = true;
 };
 
 int launch_stage(dg_ctx* c, const void* q_in, void* q_out, void* res, double a, double b, double dt, bool rk,
@@ -782,7 +788,9 @@ int launch_stage(dg_ctx* c, const void* q_in, void* q_out, void* res, double a, 
     A.flux = c->flux;
     A.wedge_bpc = c->tuned_bpc;
     if (c->tuned_onthefly) A.m.w_fac = nullptr;
+    A.tri_far = c->tri_far ? 1 : 0;
     A.rk_g = x.g;
+    A.res_store = x.res_store ? 1 : 0;
     A.rhs_out = static_cast<double*>(x.rhs_out);
     if (x.no_sources) A.m.nsrc = 0;
     rc = stage_f64(c->N, A, rk, s, c->tet_stream, c->ev_fork, c->ev_join);
@@ -804,6 +812,7 @@ int launch_stage(dg_ctx* c, const void* q_in, void* q_out, void* res, double a, 
     A.split = c->tuned_split;
     A.tri_far = c->tri_far ? 1 : 0;
     A.rk_g = float(x.g);
+    A.res_store = x.res_store ? 1 : 0;
     A.rhs_out = static_cast<float*>(x.rhs_out);
     if (x.no_sources) A.m.nsrc = 0;
     rc = stage_f32(c->N, A, rk, s, c->tet_stream, c->ev_fork, c->ev_join);
@@ -1544,8 +1553,10 @@ int dg_step(dg_ctx* c, double dt, int64_t nsteps) {
       int src = p;
       int lrc = DG_OK;
       for (int s = 0; s < 5 && lrc == DG_OK; ++s) {
+        StageExtra x;
+        x.res_store = s < 4;  // the next step's first stage (a = 0) reads no residual
         lrc = launch_stage(c, c->d_q[src], c->d_q[1 - src], c->d_res, kLSRK_A[s], kLSRK_B[s], dt, true, c->cap_stream,
-                           kLSRK_C[s]);
+                           kLSRK_C[s], x);
         src = 1 - src;
       }
       if (lrc == DG_OK) {
@@ -1950,6 +1961,7 @@ int dg_adjoint_step(dg_ctx* c, double dt) {
     void* qout = adj_field(c, st < 4 ? kAdjQs + st : kAdjScr);
     StageExtra x;
     x.rhs_out = adj_field(c, kAdjRs + st);
+    x.res_store = st < 4;
     R[st] = x.rhs_out;
     rc = launch_stage(c, Q[st], qout, adj_field(c, kAdjRes), kLSRK_A[st], kLSRK_B[st], dt, true, c->stream, kLSRK_C[st], x);
   }
@@ -1988,6 +2000,7 @@ int dg_step_record_chain(dg_ctx* c, double dt, int64_t nsteps, void* const* d_re
     for (int st = 0; st < 5 && rc == DG_OK; ++st) {
       StageExtra x;
       x.rhs_out = rec + size_t(5 + st) * fb;
+      x.res_store = st < 4;
       void* qout = st < 4 ? static_cast<void*>(rec + size_t(st + 1) * fb)
                           : (i + 1 < nsteps ? d_recs[i + 1] : c->d_q[c->cur]);
       rc = launch_stage(c, rec + size_t(st) * fb, qout, c->d_res, kLSRK_A[st], kLSRK_B[st], dt, true, c->stream,

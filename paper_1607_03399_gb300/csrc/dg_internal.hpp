@@ -151,6 +151,7 @@ struct StageArgs {
   real* res = nullptr;          // RK residual (unused in RHS mode)
   real rk_a = 0, rk_b = 0, dt = 0;
   real rk_g = 1;                // RK: q_out = rk_g q_in + rk_b res' (1 in the forward method)
+  int res_store = 1;            // RK: store the residual (0: no later stage reads it)
   real* rhs_out = nullptr;      // RK: also store the stage right-hand side here (optional)
   double c_stage = 0;           // stage time = *clock + c_stage * dt
   int bc = 1, flux = 0;

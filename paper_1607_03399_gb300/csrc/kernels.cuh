@@ -35,7 +35,7 @@ __device__ __forceinline__ const AllOps<N, real>& OPS() {
 }
 
 __device__ __forceinline__ float rsqrt_r(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_r(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ double rsqrt_r(double x) { return rsqrt(x); }
 __device__ __forceinline__ float sqrt_r(float x) { return sqrtf(x); }
 __device__ __forceinline__ double sqrt_r(double x) { return sqrt(x); }
 
@@ -362,7 +362,7 @@ __device__ __forceinline__ void add_sources(const DevMesh<real>& M, int type, in
     const real* __restrict__ g = M.src_g + sd.goff + n0;
 #pragma unroll
     for (int c = 0; c < C; ++c)
-      if (n0 + c < np) acc[c] += w * g[c];
+      if (n0 + c < np) acc[c] = fmar(w, g[c], acc[c]);
   }
 }
 // the same on field-pair accumulators whose x component is the pressure
@@ -379,7 +379,7 @@ __device__ __forceinline__ void add_sources(const DevMesh<real>& M, int type, in
     const real* __restrict__ g = M.src_g + sd.goff + n0;
 #pragma unroll
     for (int c = 0; c < C; ++c)
-      if (n0 + c < np) acc[c].x += w * g[c];
+      if (n0 + c < np) acc[c].x = fmar(w, g[c], acc[c].x);
   }
 }
 
@@ -517,95 +517,331 @@ __host__ __device__ constexpr int wedge_min_ctas() {
 
 // Lemma 3.1 for one wedge: everything the stage needs, from the six vertices
 // (bi-unit reference, x = sum_a lambda_a(r,s) [(1-t)/2 X_a + (1+t)/2 X_{a+3}]),
-// X = [x_a][y_a][zb_a][zt_a] (a = 0..2, bottom x and y; bottom and top z).
-__device__ __forceinline__ void wedge_geometry_vals(const real (&X)[12], real (&G)[G_COUNT]) {
-  const real x0 = X[0], x1 = X[1], x2 = X[2], y0 = X[3], y1 = X[4], y2 = X[5];
-  const real zb0 = X[6], zb1 = X[7], zb2 = X[8], zt0 = X[9], zt1 = X[10], zt2 = X[11];
-  const real xr = real(0.5) * (x1 - x0), xs = real(0.5) * (x2 - x0);
-  const real yr = real(0.5) * (y1 - y0), ys = real(0.5) * (y2 - y0);
-  const real A = xr * ys - xs * yr;  // t_z J (constant)
-  const real iA = real(1) / A;
-  G[G_RX] = ys * iA;
-  G[G_RY] = -xs * iA;
-  G[G_SX] = -yr * iA;
-  G[G_SY] = xr * iA;
-  G[G_A] = A;
-  const real h0 = zt0 - zb0, h1 = zt1 - zb1, h2 = zt2 - zb2;
-  G[G_J0] = real(0.5) * A * h0;  // J at the three columns (J linear in r, s)
-  G[G_J1] = real(0.5) * A * h1;
-  G[G_J2] = real(0.5) * A * h2;
-  // z_r, z_s are linear in t: z_r(t) = zr0 + t zr1 (likewise z_s), so
-  // t_x J = y_r z_s - z_r y_s and t_y J = z_r x_s - x_r z_s are linear in t
-  const real zr0 = real(0.25) * ((zb1 - zb0) + (zt1 - zt0)), zr1 = real(0.25) * ((zt1 - zt0) - (zb1 - zb0));
-  const real zs0 = real(0.25) * ((zb2 - zb0) + (zt2 - zt0)), zs1 = real(0.25) * ((zt2 - zt0) - (zb2 - zb0));
-  G[G_TX0] = yr * zs0 - zr0 * ys;
-  G[G_TX1] = yr * zs1 - zr1 * ys;
-  G[G_TY0] = zr0 * xs - xr * zs0;
-  G[G_TY1] = zr1 * xs - xr * zs1;
-  {
-    // triangle faces: n = c / |c| with c the edge cross product, J_f = |c| / 4
-    const real ax = x1 - x0, ay = y1 - y0, bx = x2 - x0, by = y2 - y0;
-    real az = zb1 - zb0, bz = zb2 - zb0;
-    real cx = ay * bz - az * by, cy = az * bx - ax * bz, cz = ax * by - ay * bx;
-    real cc = cx * cx + cy * cy + cz * cz, ic = rsqrt_r(cc);
-    G[G_JFB] = real(0.25) * cc * ic;
-    G[G_NB0] = -cx * ic;
-    G[G_NB1] = -cy * ic;
-    G[G_NB2] = -cz * ic;
-    az = zt1 - zt0;
-    bz = zt2 - zt0;
-    cx = ay * bz - az * by;
-    cy = az * bx - ax * bz;
-    cz = ax * by - ay * bx;
-    cc = cx * cx + cy * cy + cz * cz;
-    ic = rsqrt_r(cc);
-    G[G_JFT] = real(0.25) * cc * ic;
-    G[G_NT0] = cx * ic;
-    G[G_NT1] = cy * ic;
-    G[G_NT2] = cz * ic;
-  }
-  const real xx[3] = {x0, x1, x2}, yy[3] = {y0, y1, y2}, hh[3] = {h0, h1, h2};
-#pragma unroll
-  for (int ed = 0; ed < 3; ++ed) {
-    const int ia = ed, ib = (ed + 1) % 3;
-    const real dx = xx[ib] - xx[ia], dy = yy[ib] - yy[ia];
+// X = [x_a][y_a][zb_a][zt_a] (a = 0..2, bottom x and y; bottom and top z), in
+// six parts: 0 the metric terms (with JAC the column Jacobians too), 1 the
+// bottom and 2 the top triangle, 3..5 the quadrilateral faces.
+constexpr int kGeoParts = 6;
+template <bool JAC>
+__device__ __forceinline__ void wedge_geometry_part(int part, const real* sX, real* sG, int lane) {
+  auto X = [&](int i) { return sX[i * kB + lane]; };
+#define SETG(item, v) sG[(item) * kB + lane] = (v)
+  if (part == 0) {
+    const real x0 = X(0), y0 = X(3);
+    const real xr = real(0.5) * (X(1) - x0), xs = real(0.5) * (X(2) - x0);
+    const real yr = real(0.5) * (X(4) - y0), ys = real(0.5) * (X(5) - y0);
+    const real A = xr * ys - xs * yr;  // t_z J (constant)
+    const real iA = real(1) / A;
+    SETG(G_RX, ys * iA);
+    SETG(G_RY, -xs * iA);
+    SETG(G_SX, -yr * iA);
+    SETG(G_SY, xr * iA);
+    SETG(G_A, A);
+    const real zb0 = X(6), zb1 = X(7), zb2 = X(8), zt0 = X(9), zt1 = X(10), zt2 = X(11);
+    if (JAC) {
+      SETG(G_J0, real(0.5) * A * (zt0 - zb0));  // J at the three columns (J linear in r, s)
+      SETG(G_J1, real(0.5) * A * (zt1 - zb1));
+      SETG(G_J2, real(0.5) * A * (zt2 - zb2));
+    }
+    // z_r, z_s are linear in t: z_r(t) = zr0 + t zr1 (likewise z_s), so
+    // t_x J = y_r z_s - z_r y_s and t_y J = z_r x_s - x_r z_s are linear in t
+    const real zr0 = real(0.25) * ((zb1 - zb0) + (zt1 - zt0)), zr1 = real(0.25) * ((zt1 - zt0) - (zb1 - zb0));
+    const real zs0 = real(0.25) * ((zb2 - zb0) + (zt2 - zt0)), zs1 = real(0.25) * ((zt2 - zt0) - (zb2 - zb0));
+    SETG(G_TX0, yr * zs0 - zr0 * ys);
+    SETG(G_TX1, yr * zs1 - zr1 * ys);
+    SETG(G_TY0, zr0 * xs - xr * zs0);
+    SETG(G_TY1, zr1 * xs - xr * zs1);
+  } else if (part < 3) {
+    // triangle faces: n = c / |c| with c the edge cross product (outward), J_f = |c| / 4
+    const bool top = part == 2;
+    const real x0 = X(0), y0 = X(3), z0 = X(top ? 9 : 6);
+    const real ax = X(1) - x0, ay = X(4) - y0, bx = X(2) - x0, by = X(5) - y0;
+    const real az = X(top ? 10 : 7) - z0, bz = X(top ? 11 : 8) - z0;
+    const real cx = ay * bz - az * by, cy = az * bx - ax * bz, cz = ax * by - ay * bx;
+    const real cc = cx * cx + cy * cy + cz * cz, ic = rsqrt_r(cc), sc = top ? ic : -ic;
+    SETG(top ? G_JFT : G_JFB, real(0.25) * cc * ic);
+    const int n0 = top ? G_NT0 : G_NB0;
+    SETG(n0 + 0, cx * sc);
+    SETG(n0 + 1, cy * sc);
+    SETG(n0 + 2, cz * sc);
+  } else {
+    const int ed = part - 3, ia = ed, ib = ed == 2 ? 0 : ed + 1;
+    const real dx = X(ib) - X(ia), dy = X(3 + ib) - X(3 + ia);
     const real ll = dx * dx + dy * dy, il = rsqrt_r(ll);
     const real Le = ll * il;
-    G[G_QNX0 + ed] = dy * il;  // horizontal outward normal of the quad face
-    G[G_QNY0 + ed] = -dx * il;
-    G[G_QCA0 + ed] = real(0.25) * Le * hh[ia];  // M~_e = ca Mea + cb Meb
-    G[G_QCB0 + ed] = real(0.25) * Le * hh[ib];
+    SETG(G_QNX0 + ed, dy * il);  // horizontal outward normal of the quad face
+    SETG(G_QNY0 + ed, -dx * il);
+    SETG(G_QCA0 + ed, real(0.25) * Le * (X(9 + ia) - X(6 + ia)));  // M~_e = ca Mea + cb Meb
+    SETG(G_QCB0 + ed, real(0.25) * Le * (X(9 + ib) - X(6 + ib)));
+  }
+#undef SETG
+}
+
+// M^{tri,k} = sum_a J_a M_a with J_a = A h_a / 2 (Lemma 3.1) of wedge e from its
+// vertices; L D L^T factor row by row into the block's table, in the stored
+// factor's form (negated unit lower triangle, 1 / D_i on the diagonal).
+template <int N>
+__device__ __forceinline__ void factor_wedge(const AllOps<N, real>& O, const DevMesh<real>& M, int e, int lane, real* sL) {
+  constexpr int Nt = nt_of(N);
+  const int Kp = M.Kw_pad;
+#define LQ(q) sL[(((q) >> 2) * kB + lane) * 4 + ((q) & 3)]
+  const int v0 = M.w_vid[0 * Kp + e], v1 = M.w_vid[1 * Kp + e], v2 = M.w_vid[2 * Kp + e];
+  const int v3 = M.w_vid[3 * Kp + e], v4 = M.w_vid[4 * Kp + e], v5 = M.w_vid[5 * Kp + e];
+  const real x0 = M.vx[v0], y0 = M.vy[v0];
+  const real Ah = real(0.125) * ((M.vx[v1] - x0) * (M.vy[v2] - y0) - (M.vx[v2] - x0) * (M.vy[v1] - y0));
+  const real J0 = Ah * (M.vz[v3] - M.vz[v0]), J1 = Ah * (M.vz[v4] - M.vz[v1]), J2 = Ah * (M.vz[v5] - M.vz[v2]);
+#pragma unroll
+  for (int i = 0; i < Nt; ++i) {
+    real row[Nt];  // l_il D_l
+#pragma unroll
+    for (int l = 0; l < i; ++l) {
+      real s = J0 * O.w.Ma[0][i * Nt + l] + J1 * O.w.Ma[1][i * Nt + l] + J2 * O.w.Ma[2][i * Nt + l];
+#pragma unroll
+      for (int k = 0; k < l; ++k) s += row[k] * LQ(l * (l + 1) / 2 + k);
+      row[l] = s;
+    }
+    real d = J0 * O.w.Ma[0][i * Nt + i] + J1 * O.w.Ma[1][i * Nt + i] + J2 * O.w.Ma[2][i * Nt + i];
+#pragma unroll
+    for (int k = 0; k < i; ++k) {
+      const real nl = -(row[k] * LQ(k * (k + 1) / 2 + k));
+      d += row[k] * nl;
+      LQ(i * (i + 1) / 2 + k) = nl;
+    }
+    LQ(i * (i + 1) / 2 + i) = real(1) / d;
+  }
+#undef LQ
+}
+
+// X = (M^{tri,k})^{-1} W for the four right-hand sides of a slice (field pairs
+// W01, W23) with the L D L^T factor of the block's table sL: forward sweep row
+// by row, the diagonal, then the backward sweep in column-update form; four
+// entries per shared load.  The table holds the negated unit lower triangle
+// and 1 / D_i, so both sweeps are multiply-adds alone.
+template <int N>
+__device__ __forceinline__ void mass_solve(const real* sL, int lane, real2 (&W01)[nt_of(N)], real2 (&W23)[nt_of(N)]) {
+  constexpr int Nt = nt_of(N);
+  // row i of the factor, entries q = i (i + 1) / 2 + k, k = 0..i
+  auto load_row = [&](int i, real (&Lr)[Nt]) {
+    const int a0 = i * (i + 1) / 2;
+#pragma unroll
+    for (int c4 = a0 >> 2; c4 <= (a0 + i) >> 2; ++c4) {
+      const Q4 v = ldop4(sL + (c4 * kB + lane) * 4);
+      const real vv[4] = {v.p, v.u, v.v, v.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int k = c4 * 4 + q - a0;
+        if (k >= 0 && k <= i) Lr[k] = vv[q];
+      }
+    }
+  };
+  real d[Nt];
+#pragma unroll
+  for (int i = 0; i < Nt; ++i) {
+    real Lr[Nt];
+    load_row(i, Lr);
+#pragma unroll
+    for (int k = 0; k < i; ++k) {
+      const real2 nl = dup2(Lr[k]);
+      W01[i] = fma2(nl, W01[k], W01[i]);
+      W23[i] = fma2(nl, W23[k], W23[i]);
+    }
+    d[i] = Lr[i];
+  }
+#pragma unroll
+  for (int i = 0; i < Nt; ++i) {
+    W01[i] = mul2(W01[i], dup2(d[i]));
+    W23[i] = mul2(W23[i], dup2(d[i]));
+  }
+#pragma unroll
+  for (int i = Nt - 1; i > 0; --i) {
+    real Lr[Nt];
+    load_row(i, Lr);
+#pragma unroll
+    for (int k = 0; k < i; ++k) {
+      const real2 nl = dup2(Lr[k]);
+      W01[k] = fma2(nl, W01[i], W01[k]);
+      W23[k] = fma2(nl, W23[i], W23[k]);
+    }
   }
 }
 
-// The stage's geometry warp: coordinates arrive in the first 12 items of the
-// shared table (one column per lane) and are replaced by the first NG factors.
-template <int NG = G_COUNT>
-__device__ __forceinline__ void wedge_geometry(real* sG, int lane) {
-  real X[12];
-#pragma unroll
-  for (int i = 0; i < 12; ++i) X[i] = sG[i * kB + lane];
-  __syncwarp();
-  real G[G_COUNT];
-  wedge_geometry_vals(X, G);
-#pragma unroll
-  for (int i = 0; i < NG; ++i) sG[i * kB + lane] = G[i];
+// L2 prefetch for block pb, half a wave after the caller's: its neighbour, code
+// and material tables, so that the chain neighbour id -> neighbour trace starts
+// from L2 instead of DRAM, and its state slab (N <= 4 with the stored factor;
+// elsewhere the stage waits on arithmetic and it measured slower).
+// 524,288 wedges, us per stage of a step: N = 3 264 without, 249 with the
+// tables, 238 with the state too; N = 4 675, 662, 656; N = 2 119, 112, 109; a
+// whole wave ahead gains less, the residual slab or the factor nothing.
+template <int N>
+__device__ __forceinline__ void prefetch_ahead(const DevMesh<real>& M, const real* qin, int pb, int lane, bool state) {
+  if (pb >= M.nblk_w) return;
+  const int64_t Kp = M.Kw_pad, at = int64_t(pb) * kB;
+  if (lane < 13) {
+    const void* p = lane < 5    ? static_cast<const void*>(M.w_nbr + lane * Kp + at)
+                    : lane < 10 ? static_cast<const void*>(M.w_code + (lane - 5) * Kp + at)
+                                : static_cast<const void*>(M.w_mat + (lane - 10) * Kp + at);
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+  } else if (lane == 13 && state) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(qin + widx<N>(pb, 0, 0)),
+                 "r"(uint32_t(4 * npw_of(N) * kB * sizeof(real))));
+  }
 }
 
-// TF: the neighbour nodes of the triangle-face fluxes are requested before the
-// quadrilateral faces (one block per CTA: meshes where some of them are tets
-// or lie in another block, StageArgs::tri_far; two blocks per CTA: always);
-// otherwise each is read where its flux is formed
-template <int N, int BPC, int OP = kOpFFMA, bool TF = false>
-__global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>())
+// Fused low-storage Runge-Kutta update of a node: res <- a res + dt r, q_out <-
+// g q_in + b res, r = kappa X_p, X_u / rho; or the plain right-hand side.  The
+// residual is read only where a != 0 and stored only where a later stage reads
+// it (StageArgs::res_store): of the five stages of a step the first reads none
+// and the last stores none, a tenth of the step's traffic.
+struct UpdateCoef {
+  real2 s01, s23, d01, d23, a2, g2, b2;
+  __device__ __forceinline__ UpdateCoef(const StageArgs<real>& A, real kappa, real irho)
+      : s01(mk2(kappa, irho)), s23(dup2(irho)), d01(mul2(s01, dup2(A.dt))), d23(mul2(s23, dup2(A.dt))), a2(dup2(A.rk_a)),
+        g2(dup2(A.rk_g)), b2(dup2(A.rk_b)) {}
+  // g: packed index of the node; r0 its residual (0 where a = 0), q0 its state
+  __device__ __forceinline__ void node(const StageArgs<real>& A, bool rk, int64_t g, const real2 X01, const real2 X23,
+                                       const Q4& r0, const Q4& q0) const {
+    if (!rk || A.rhs_out != nullptr) {
+      const real2 r01 = mul2(X01, s01), r23 = mul2(X23, s23);
+      st4(rk ? A.rhs_out : A.q_out, g, Q4{r01.x, r01.y, r23.x, r23.y});
+      if (!rk) return;
+    }
+    const real2 r01 = fma2(X01, d01, mul2(a2, mk2(r0.p, r0.u)));
+    const real2 r23 = fma2(X23, d23, mul2(a2, mk2(r0.v, r0.w)));
+    const real2 q01 = fma2(b2, r01, mul2(g2, mk2(q0.p, q0.u)));
+    const real2 q23 = fma2(b2, r23, mul2(g2, mk2(q0.v, q0.w)));
+    if (A.res_store) st4(A.res, g, Q4{r01.x, r01.y, r23.x, r23.y});
+    st4(A.q_out, g, Q4{q01.x, q01.y, q23.x, q23.y});
+  }
+};
+template <int N, bool RES_SMEM>
+__device__ __forceinline__ void wedge_update(const StageArgs<real>& A, bool rk, const real* sq, const real* sr, int blk, int j,
+                                             int lane, int e, real kappa, real irho, const real2 (&W01)[nt_of(N)],
+                                             const real2 (&W23)[nt_of(N)]) {
+  constexpr int Nt = nt_of(N);
+  if (e >= A.m.Kw) return;
+  const UpdateCoef U(A, kappa, irho);
+#pragma unroll
+  for (int i = 0; i < Nt; ++i) {
+    const int n = j * Nt + i;
+    const int64_t g = widx<N>(blk, n, lane);
+    Q4 r0{0, 0, 0, 0};
+    if (rk && A.rk_a != real(0)) r0 = RES_SMEM ? lds4(sr, n, lane) : ld4(A.res, g);
+    U.node(A, rk, g, W01[i], W23[i], r0, lds4(sq, n, lane));
+  }
+}
+
+// ---------------------------------------------------------------------------
+// wedge stage on the CUDA cores
+// ---------------------------------------------------------------------------
+// Entry (m, code) of the neighbour's edge-node table, code = 2 * edge +
+// reversed, m-th node of this side: the six candidates packed five bits each
+// into one constant, so a lane with its own code extracts its node with a
+// shift and a mask instead of an indexed constant load (which is replayed for
+// every distinct index of the warp).
+template <int N>
+struct EdgeCandidates {
+  uint32_t c[N + 1];
+  __host__ __device__ constexpr EdgeCandidates() : c{} {
+    for (int m = 0; m <= N; ++m)
+      for (int code = 0; code < 6; ++code)
+        c[m] |= uint32_t(edge_node(N, code >> 1, (code & 1) ? N - m : m)) << (5 * code);
+  }
+};
+// D_r restricted to the edge b = 0 (rows a = 0..N) differentiates along the
+// edge: only its own N + 1 nodes enter; D_s likewise on the edge a = 0.
+__host__ __device__ constexpr bool dr_zero(int N, int i, int l) { return i <= N && l > N; }
+__host__ __device__ constexpr bool on_edge_a0(int N, int i) {
+  for (int b = 0; b <= N; ++b)
+    if (tri_idx(N, 0, b) == i) return true;
+  return false;
+}
+__host__ __device__ constexpr bool ds_zero(int N, int i, int l) { return on_edge_a0(N, i) && !on_edge_a0(N, l); }
+// acc += {X[2h][l], X[2h + 1][l]} * x, leaving out rows known to be zero
+// (FP32: the pair is one instruction and is left out when both rows are zero)
+template <int NT>
+__device__ __forceinline__ real2 fma_rows(const real* XP, int h, int l, real x, real2 acc, bool z0, bool z1) {
+  if constexpr (sizeof(real) == 4) {
+    if (z0 && (z1 || 2 * h + 1 >= NT)) return acc;
+    return fma2(cpair(XP, NT, h, l), dup2(x), acc);
+  } else {
+    const real2 c = cpair(XP, NT, h, l);
+    if (!z0) acc.x = fmar(c.x, x, acc.x);
+    if (!z1 && 2 * h + 1 < NT) acc.y = fmar(c.y, x, acc.y);
+    return acc;
+  }
+}
+// {-s_p, -s_u}: the ghost state of a boundary face is the own trace with the
+// pressure (Dirichlet) or the velocity (rigid) reversed; +1, +1 on interior
+// faces.  The negated jump is then own + (-s) * neighbour, one multiply-add
+// per component with no branch: rigid -2 u_n, Dirichlet -2 p as before.
+__device__ __forceinline__ real2 ghost_signs(bool bnd, int bc) {
+  return mk2(bnd && bc == 0 ? real(1) : real(-1), bnd && bc != 0 ? real(1) : real(-1));
+}
+
+// Flux pair (F_p, F_u), twice eq. (1)'s, of a triangle-face node with own
+// state o, neighbour state v, normal n, -tau_p and -tau_u.  Explicit
+// multiply-adds here and in the quadrilateral faces: every form of the stage
+// gives the same bits.
+__device__ __forceinline__ real2 tri_node_flux(const Q4& o, const Q4& v, real n0, real n1, real n2, const real2 s, real ntp,
+                                               real ntu) {
+  const real2 d01 = fma2(s, mk2(v.p, v.u), mk2(o.p, o.u));          // negated jumps of p, u_x
+  const real2 d23 = fma2(dup2(s.y), mk2(v.v, v.w), mk2(o.v, o.w));  // and of u_y, u_z
+  const real dn = fmar(n2, d23.y, fmar(n1, d23.x, n0 * d01.y));
+  return mk2(fmar(ntp, d01.x, dn), fmar(ntu, dn, d01.x));
+}
+// Quadrilateral face ed of slice j: the fluxes along the edge times M~_e =
+// (L_e / 4)(h_a Mea + h_b Meb) (ca, cb: half the two factors; identity in t),
+// F_p in gp2 and F_u in gu2 by output pairs.
+template <int N>
+__device__ __forceinline__ void quad_edge(const AllOps<N, real>& O, const real* sq, int j, int lane, int ed,
+                                          const Q4 (&tv)[N + 1], real nx, real ny, const real2 s, real tp, real tu, real ca,
+                                          real cb, real2 (&gp2)[(N + 2) / 2], real2 (&gu2)[(N + 2) / 2]) {
+  constexpr int Nt = nt_of(N), Nq = N + 1, NQH = (N + 2) / 2;
+  const real2 ca2 = dup2(ca), cb2 = dup2(cb);
+#pragma unroll
+  for (int h = 0; h < NQH; ++h) gp2[h] = gu2[h] = dup2(real(0));
+#pragma unroll
+  for (int m = 0; m < Nq; ++m) {
+    const Q4 o = lds4(sq, j * Nt + edge_node(N, ed, m), lane);
+    const real2 d01 = fma2(s, mk2(tv[m].p, tv[m].u), mk2(o.p, o.u));
+    const real d2 = fmar(s.y, tv[m].v, o.v);
+    const real dn = fmar(nx, d01.y, ny * d2);
+    const real2 Fp = dup2(fmar(-tp, d01.x, dn)), Fu = dup2(fmar(-tu, dn, d01.x));
+#pragma unroll
+    for (int h = 0; h < NQH; ++h) {
+      const real2 w = fma2(cpair(O.w.MebP, Nq, h, m), cb2, mul2(cpair(O.w.MeaP, Nq, h, m), ca2));
+      gp2[h] = fma2(w, Fp, gp2[h]);
+      gu2[h] = fma2(w, Fu, gu2[h]);
+    }
+  }
+}
+
+// One stage of a 32-wedge block per N + 1 warps (lane = element, warp j =
+// slice j), in the weak-in-t form
+//   W_p = M (-(t_xJ D_t u + t_yJ D_t v + A D_t w)) + lifts,  W_u = -t_cJ M D_t p + lifts
+// so M^tri is applied per slice to two vectors (the t-divergence and D_t p)
+// and, once per element instead of once per slice, to the four triangle-face
+// flux vectors: 2 + 4 / (N + 1) applications per slice where forming the four
+// right-hand sides first takes 4.  Every lane reads its quadrilateral-face
+// neighbours from global memory, also those in its own block (no per-lane
+// choice between two address spaces), and a boundary face reads its own trace.
+// Bound by memory latency and traffic at N <= 3 (a copy of the slabs and the
+// traces alone takes 218 us of the 240 at N = 3), by issue and registers at
+// N >= 4.  Warp instructions per warp, N = 3: 2,769 -> 2,140.  us per stage of
+// a step on 524,288 wedges, with the skipped residual traffic and the prefetch:
+// N = 3 298 -> 240, N = 4 769 -> 670; 30,118 wedges N = 5 326 -> 230.
+// TF: the neighbour nodes of the triangle-face fluxes come from global memory
+// and are requested before the slab arrives (meshes where some of them are
+// tets or lie in another block, StageArgs::tri_far; two blocks per CTA:
+// always); otherwise they are all in this block's slab.
+template <int N, int BPC, bool TF>
+__global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOpFFMA>())
     k_wedge_stage(const StageArgs<real> A, bool rk) {
-  constexpr int Nt = nt_of(N), Nq = N + 1, Np = Nt * Nq;
-  static_assert(OP == kOpFFMA || (sizeof(real) == 4 && BPC == 1 && Nt <= 16), "tensor-core applies: FP32, Nt <= 16");
-  using SM = WedgeSmem<N, OP>;
+  constexpr int Nt = nt_of(N), Nq = N + 1, Np = Nt * Nq, NH = (Nt + 1) / 2, NQH = (Nq + 1) / 2;
+  using SM = WedgeSmem<N, kOpFFMA>;
   const AllOps<N, real>& O = OPS<N>();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   // block sb of this CTA: warps sb (N+1) .. sb (N+1) + N, one per slice
-  const int sb = threadIdx.x / (32 * Nq);
+  const int sb = BPC == 1 ? 0 : threadIdx.x / (32 * Nq);
   const int j = (threadIdx.x >> 5) - sb * Nq;
   const bool leader = int(threadIdx.x) == sb * 32 * Nq;
   // [0] state slab (and stored factor), [1] residual slab, [2] vertex coordinates
@@ -615,35 +851,23 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
   real* sq = base + SM::q;
   real* sr = base + SM::r;
   real* sL = base + SM::L;
-  real* sF = base + SM::F;
+  real* sF = base + SM::F;  // [face][node][lane] pairs (F_p, F_u), then M^tri applied to each
   real* sG = base + SM::G;
-  real* sT = base + SM::T + j * Nt * kTP;  // this warp's operand tile (tensor cores)
   const DevMesh<real>& M = A.m;
   const real* __restrict__ qin = A.q_in;
-  real* __restrict__ qout = A.q_out;
-  real* __restrict__ resg = A.res;
   const int lane = threadIdx.x & 31;
   const int blk = blockIdx.x * BPC + sb;
-  const bool live = blk < M.nblk_w;  // false only for padding blocks of the last CTA
+  if (blk >= M.nblk_w) return;  // padding block of the last CTA
   const int e = blk * kB + lane;
   const int Kp = M.Kw_pad;
   constexpr uint32_t slab_bytes = uint32_t(4 * Np * kB * sizeof(real));
-  const bool res_async = rk && stage_res<N, OP>();
-  // the residual copy is issued with the state's (FP32 FMA applies) or after
-  // the weak-form accumulation, once the operand tiles in its space are free
-  const bool res_early = res_async && OP == kOpFFMA;
+  const bool res_async = rk && stage_res<N, kOpFFMA>() && A.rk_a != real(0);
 #define GEO(item) sG[(item) * kB + lane]
-#define LQ(q) sL[(((q) >> 2) * kB + lane) * 4 + ((q) & 3)]
-
-  if (!live) return;  // padding block of the last CTA
   // the warps of one block synchronise among themselves (named barrier 1 + sb)
-  // (immediate barrier ids, so that only BPC + 1 hardware barriers are reserved)
   auto block_sync = [&]() {
-    static_assert(BPC <= 4, "at most four blocks per CTA");
+    static_assert(BPC <= 2, "at most two blocks per CTA");
     if (sb == 0) asm volatile("bar.sync 1, %0;" ::"n"(32 * Nq) : "memory");
-    else if (BPC > 1 && sb == 1) asm volatile("bar.sync 2, %0;" ::"n"(32 * Nq) : "memory");
-    else if (BPC > 2 && sb == 2) asm volatile("bar.sync 3, %0;" ::"n"(32 * Nq) : "memory");
-    else if (BPC > 3) asm volatile("bar.sync 4, %0;" ::"n"(32 * Nq) : "memory");
+    else asm volatile("bar.sync 2, %0;" ::"n"(32 * Nq) : "memory");
   };
   // 0. bulk copies of the block's state (and residual) slabs; geometry meanwhile
   constexpr int NL4 = nl4_of(N);
@@ -654,24 +878,339 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
     mbar_init(&bar[2], 1);
-    mbar_init(&bar[3], 1);
     fence_mbar_init();
-    // the block's vertex coordinates first (the geometry warp waits on them alone)
+    // the block's vertex coordinates first (the geometry waits on them alone), in
+    // the flux table's place, which is written after the barrier below
     mbar_expect_tx(&bar[2], xyz_bytes);
-    bulk_g2s(sG, M.w_xyz + int64_t(blk) * 12 * kB, xyz_bytes, &bar[2]);
+    bulk_g2s(sF, M.w_xyz + int64_t(blk) * 12 * kB, xyz_bytes, &bar[2]);
     mbar_expect_tx(&bar[0], slab_bytes + (stored ? fac_bytes : 0u));
     bulk_g2s(sq, qin + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[0]);
     // stored mass factor: straight into the factor table with the state slab
     if (stored) bulk_g2s(sL, M.w_fac + int64_t(blk) * NL4 * 4 * kB, fac_bytes, &bar[0]);
-    if (res_early) {
+    if (res_async) {
       mbar_expect_tx(&bar[1], slab_bytes);
-      bulk_g2s(sr, resg + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[1]);
+      bulk_g2s(sr, A.res + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[1]);
     }
   }
+  if (j == N) prefetch_ahead<N>(M, qin, blk + 76 * wedge_min_ctas<N, BPC, kOpFFMA>() * BPC, lane, N <= 4 && stored);
+  // face neighbours, their impedances and the source flag, loaded while the
+  // slabs are in flight; so are (N <= 3) the neighbour traces
+  const real kappa = M.w_mat[0 * Kp + e], irho = M.w_mat[1 * Kp + e], zM = M.w_mat[2 * Kp + e];
+  int qnbr[3], qcode[3];
+#pragma unroll
+  for (int ed = 0; ed < 3; ++ed) {
+    qnbr[ed] = M.w_nbr[(2 + ed) * Kp + e];
+    qcode[ed] = M.w_code[(2 + ed) * Kp + e];
+  }
+  const int tnbr[2] = {M.w_nbr[0 * Kp + e], M.w_nbr[1 * Kp + e]};
+  const int tcode[2] = {M.w_code[0 * Kp + e], M.w_code[1 * Kp + e]};
+  // trace of quadrilateral face ed: nodes of slice j of the neighbour (or, on a boundary, of the element itself)
+  auto trace = [&](int ed, Q4 (&t)[Nq]) {
+    const bool bnd = qnbr[ed] < 0;
+    const int nbe = bnd ? e : qnbr[ed], sh = 5 * (bnd ? 2 * ed : qcode[ed]);
+    constexpr EdgeCandidates<N> cand;
+    const real* nb = qin + widx<N>(nbe >> 5, j * Nt, nbe & 31);
+#pragma unroll
+    for (int m = 0; m < Nq; ++m) t[m] = ldg4(nb, int((cand.c[m] >> sh) & 31u) * (kB * 4));
+  };
+  constexpr bool early = N <= 3;
+  Q4 nv[early ? 3 : 1][Nq];
+  if constexpr (early) {
+#pragma unroll
+    for (int ed = 0; ed < 3; ++ed) trace(ed, nv[ed]);
+  }
+  // the neighbour node of triangle-face flux node t of this warp (round-robin
+  // over the warps, bottom then top): a tet's face node, or a wedge's bottom or
+  // top node; a boundary face reads its own node
+  constexpr int NTT = (2 * Nt + Nq - 1) / Nq;
+  auto tri_nbr_node = [&](int t) {
+    const int idx = j + t * Nq;
+    const int fb = idx >= Nt ? 1 : 0;
+    const int k = idx - fb * Nt;
+    const int nbr = fb ? tnbr[1] : tnbr[0], code = fb ? tcode[1] : tcode[0];
+    const bool bnd = nbr < 0;
+    const int nbe = bnd ? e : nbr, nf = bnd ? fb : (code >> 4) & 3;
+    const int nk = bnd ? k : O.tab.tri_perm[code & 15][k];
+    if constexpr (TF) {
+      const bool ntet = !bnd && (code & kCodeTet) != 0;
+      const int node = ntet ? O.tab.tet_face[nf][nk] : (nf ? N * Nt : 0) + nk;
+      return ldg4(qin, ntet ? tidx<N>(M.tet_off, nbe >> 5, node, nbe & 31) : widx<N>(nbe >> 5, node, nbe & 31));
+    } else {
+      return lds4(sq, (nf ? N * Nt : 0) + nk, nbe & 31);
+    }
+  };
+  Q4 tnv[TF ? NTT : 1];
+  if constexpr (TF) {
+#pragma unroll
+    for (int t = 0; t < NTT; ++t)
+      if (j + t * Nq < 2 * Nt) tnv[t] = tri_nbr_node(t);
+  }
+  real zPq[3], zPt[2];
+#pragma unroll
+  for (int ed = 0; ed < 3; ++ed) zPq[ed] = qnbr[ed] < 0 ? zM : M.w_mat[2 * Kp + qnbr[ed]];
+#pragma unroll
+  for (int fb = 0; fb < 2; ++fb)
+    zPt[fb] = tnbr[fb] < 0 ? zM
+                           : ((tcode[fb] & kCodeTet) ? M.t_mat[2 * M.Kt_pad + tnbr[fb]] : M.w_mat[2 * Kp + tnbr[fb]]);
+  const bool src = M.nsrc > 0 && has_source(M, 6, e);
+  // the parts of the geometry, round-robin over the warps, each of which waits
+  // for the coordinates itself: the barrier's initialisation must be visible first
+  block_sync();
+  const bool geo_ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[2], 0));
+  if (geo_ok) {
+#pragma unroll 1
+    for (int p = j; p < kGeoParts; p += Nq) wedge_geometry_part<false>(p, sF, sG, lane);
+  } else if (lane == 0) {
+    atomicOr(M.err, kErrTimeout);
+  }
+  if (j == 1 && !stored) {
+    factor_wedge<N>(O, M, e, lane, sL);  // while the slabs are in flight
+  }
+  if (leader) *status = (mbar_wait_bounded(&bar[0], 0) && geo_ok) ? 1 : 0;
+  block_sync();
+  if (*reinterpret_cast<volatile int*>(status) == 0) {
+    // a copy never arrived: report, let any copy in flight drain, leave
+    if (leader) {
+      atomicOr(M.err, kErrTimeout);
+      if (res_async) mbar_wait_bounded(&bar[1], 0);
+      mbar_wait_bounded(&bar[0], 0);
+      mbar_wait_bounded(&bar[2], 0);
+    }
+    return;
+  }
+
+  // 1. triangle-face node fluxes (bottom then top), spread round-robin over
+  //    the warps, without the factor 1/2 (it enters with the lift)
+  {
+    real ntp[2], ntu[2];
+#pragma unroll
+    for (int fb = 0; fb < 2; ++fb) {
+      real tp, tu;
+      taus(A.flux, zM, zPt[fb], tp, tu);
+      ntp[fb] = -tp;
+      ntu[fb] = -tu;
+    }
+#pragma unroll
+    for (int t = 0; t < NTT; ++t) {
+      const int idx = j + t * Nq;
+      if (idx >= 2 * Nt) break;
+      const int fb = idx >= Nt ? 1 : 0;
+      const int k = idx - fb * Nt;
+      const real n0 = GEO(fb ? G_NT0 : G_NB0), n1 = GEO(fb ? G_NT1 : G_NB1), n2 = GEO(fb ? G_NT2 : G_NB2);
+      const Q4 o = lds4(sq, (fb ? N * Nt : 0) + k, lane);
+      Q4 v;
+      if constexpr (TF) v = tnv[t];
+      else v = tri_nbr_node(t);
+      const real2 F = tri_node_flux(o, v, n0, n1, n2, ghost_signs((fb ? tnbr[1] : tnbr[0]) < 0, A.bc), fb ? ntp[1] : ntp[0],
+                                    fb ? ntu[1] : ntu[0]);
+      *reinterpret_cast<real2*>(sF + ((fb * Nt + k) * kB + lane) * 2) = F;
+    }
+  }
+  block_sync();
+  // 2. M^tri applied in place to the four flux vectors (bottom F_p, F_u, top
+  //    F_p, F_u), one per warp
+#pragma unroll 1
+  for (int v = j; v < 4; v += Nq) {
+    real* f = sF + ((v >> 1) * Nt * kB + lane) * 2 + (v & 1);
+    real G[Nt];
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) G[i] = f[i * kB * 2];
+    real2 acc[NH];
+    apply_pairs<Nt, Nt>(O.w.MP, G, acc);
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) f[i * kB * 2] = pair_row(acc, i);
+  }
+
+  // 3. quadrilateral faces of slice j: M~_e F_p into W_p (by output pairs), M~_e F_u kept per edge
+  real2 Wp[NH];
+  real gu[3][Nq];
+#pragma unroll
+  for (int h = 0; h < NH; ++h) Wp[h] = dup2(real(0));
+#pragma unroll
+  for (int ed = 0; ed < 3; ++ed) {
+    Q4 tv[Nq];
+    if constexpr (early) {
+#pragma unroll
+      for (int m = 0; m < Nq; ++m) tv[m] = nv[ed][m];
+    } else {
+      trace(ed, tv);
+    }
+    const real nx = GEO(G_QNX0 + ed), ny = GEO(G_QNY0 + ed);
+    real tp, tu;
+    taus(A.flux, zM, zPq[ed], tp, tu);
+    real2 gp2[NQH], gu2[NQH];
+    quad_edge<N>(O, sq, j, lane, ed, tv, nx, ny, ghost_signs(qnbr[ed] < 0, A.bc), tp, tu, real(0.5) * GEO(G_QCA0 + ed),
+                 real(0.5) * GEO(G_QCB0 + ed), gp2, gu2);
+#pragma unroll
+    for (int m = 0; m < Nq; ++m) {
+      const int i = edge_node(N, ed, m);
+      if (i & 1) Wp[i >> 1].y += pair_row(gp2, m);
+      else Wp[i >> 1].x += pair_row(gp2, m);
+      gu[ed][m] = pair_row(gu2, m);
+    }
+  }
+
+  // 4. t-parts of slice j: the t-divergence dd = -(t_xJ D_t u_x + t_yJ D_t u_y
+  //    + A D_t u_z) and D_t p; W_p += M^tri dd, Mdp = M^tri D_t p
+  const real tj = O.w.gll[j];
+  const real ntx = -fmar(tj, GEO(G_TX1), GEO(G_TX0)), nty = -fmar(tj, GEO(G_TY1), GEO(G_TY0)), nA = -GEO(G_A);
+  real2 Mdp[NH];
+  {
+    real dp[Nt], dd[Nt];
+    real dtr[Nq];
+#pragma unroll
+    for (int m = 0; m < Nq; ++m) dtr[m] = O.w.Dt[j * Nq + m];
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) {
+      // D_t of the four fields as two packed pairs (p, u_x) and (u_y, u_z)
+      real2 dpu = dup2(real(0)), dvw = dup2(real(0));
+#pragma unroll
+      for (int m = 0; m < Nq; ++m) {
+        const Q4 v = lds4(sq, m * Nt + i, lane);
+        const real2 d2 = dup2(dtr[m]);
+        dpu = fma2(d2, mk2(v.p, v.u), dpu);
+        dvw = fma2(d2, mk2(v.v, v.w), dvw);
+      }
+      dp[i] = dpu.x;
+      dd[i] = fmar(ntx, dpu.y, fmar(nty, dvw.x, nA * dvw.y));
+    }
+#pragma unroll
+    for (int l = 0; l < Nt; ++l) {
+      const real2 xx = dup2(dd[l]);
+#pragma unroll
+      for (int h = 0; h < NH; ++h) Wp[h] = fma2(cpair(O.w.MP, Nt, h, l), xx, Wp[h]);
+    }
+    apply_pairs<Nt, Nt>(O.w.MP, dp, Mdp);
+  }
+  block_sync();  // M^tri has been applied to the flux vectors
+
+  // 5. right-hand sides of the mass solve by field pairs (p, u_x), (u_y, u_z):
+  //    the lifted triangle-face fluxes, -t_cJ M D_t p and the quadrilateral faces
+  real2 W01[Nt], W23[Nt];
+  {
+    const real cb = real(0.5) * GEO(G_JFB) * O.w.ell0[j], ct = real(0.5) * GEO(G_JFT) * O.w.ellN[j];
+    const real2 b01 = mk2(cb, cb * GEO(G_NB0)), t01 = mk2(ct, ct * GEO(G_NT0));
+    const real2 b23 = mk2(cb * GEO(G_NB1), cb * GEO(G_NB2)), t23 = mk2(ct * GEO(G_NT1), ct * GEO(G_NT2));
+    const real2 n23 = mk2(nty, nA);
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) {
+      const real2 fb = *reinterpret_cast<const real2*>(sF + ((0 * Nt + i) * kB + lane) * 2);
+      const real2 ft = *reinterpret_cast<const real2*>(sF + ((1 * Nt + i) * kB + lane) * 2);
+      const real md = pair_row(Mdp, i);
+      W01[i] = fma2(fb, b01, fma2(ft, t01, mk2(pair_row(Wp, i), ntx * md)));
+      W23[i] = fma2(dup2(fb.y), b23, fma2(dup2(ft.y), t23, mul2(dup2(md), n23)));
+    }
+#pragma unroll
+    for (int ed = 0; ed < 3; ++ed) {
+      const real nx = GEO(G_QNX0 + ed), ny = GEO(G_QNY0 + ed);
+#pragma unroll
+      for (int m = 0; m < Nq; ++m) {
+        const int i = edge_node(N, ed, m);
+        W01[i].y = fmar(nx, gu[ed][m], W01[i].y);
+        W23[i].x = fmar(ny, gu[ed][m], W23[i].x);
+      }
+    }
+  }
+  mass_solve<N>(sL, lane, W01, W23);
+  // 6. strong r, s parts of slice j (constant metric terms, Lemma 3.1), D_r and
+  //    D_s applied by output pairs, node l of the slice at a time
+  {
+    const real rx = GEO(G_RX), ry = GEO(G_RY), sx = GEO(G_SX), sy = GEO(G_SY);
+    real2 dv[NH], pr[NH], ps[NH];
+#pragma unroll
+    for (int h = 0; h < NH; ++h) dv[h] = pr[h] = ps[h] = dup2(real(0));
+#pragma unroll
+    for (int l = 0; l < Nt; ++l) {
+      const Q4 v = lds4(sq, j * Nt + l, lane);
+      const real2 ab = fma2(dup2(v.u), mk2(rx, sx), mul2(dup2(v.v), mk2(ry, sy)));
+#pragma unroll
+      for (int h = 0; h < NH; ++h) {
+        const bool r0 = dr_zero(N, 2 * h, l), r1 = dr_zero(N, 2 * h + 1, l);
+        const bool s0 = ds_zero(N, 2 * h, l), s1 = ds_zero(N, 2 * h + 1, l);
+        dv[h] = fma_rows<Nt>(O.w.DrP, h, l, ab.x, dv[h], r0, r1);
+        dv[h] = fma_rows<Nt>(O.w.DsP, h, l, ab.y, dv[h], s0, s1);
+        pr[h] = fma_rows<Nt>(O.w.DrP, h, l, v.p, pr[h], r0, r1);
+        ps[h] = fma_rows<Nt>(O.w.DsP, h, l, v.p, ps[h], s0, s1);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) {
+      const real pri = pair_row(pr, i), psi = pair_row(ps, i);
+      W01[i].x -= pair_row(dv, i);
+      W01[i].y = fmar(-rx, pri, fmar(-sx, psi, W01[i].y));
+      W23[i].x = fmar(-ry, pri, fmar(-sy, psi, W23[i].x));
+    }
+  }
+  // 7. fused low-storage Runge-Kutta update (or plain right-hand side)
+  if (res_async && !mbar_wait_bounded(&bar[1], 0)) {
+    if (lane == 0) atomicOr(M.err, kErrTimeout);
+    mbar_wait_bounded(&bar[1], 0);
+    return;
+  }
+  if (src) add_sources(M, 6, e, j * Nt, Np, *M.clock + A.c_stage * double(A.dt), W01);
+  wedge_update<N, stage_res<N, kOpFFMA>()>(A, rk, sq, sr, blk, j, lane, e, kappa, irho, W01, W23);
+#undef GEO
+}
+
+// The stage with M^tri applied on the tensor cores (precision variants): one
+// block per CTA, the four right-hand sides of a slice formed first and passed
+// through the warp's operand tile.
+template <int N, int OP>
+__global__ void __launch_bounds__(32 * (N + 1), wedge_min_ctas<N, 1, OP>())
+    k_wedge_stage_mma(const StageArgs<real> A, bool rk) {
+  constexpr int Nt = nt_of(N), Nq = N + 1, Np = Nt * Nq;
+  static_assert(sizeof(real) == 4 && Nt <= 16, "tensor-core applies: FP32, Nt <= 16");
+  using SM = WedgeSmem<N, OP>;
+  const AllOps<N, real>& O = OPS<N>();
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int j = threadIdx.x >> 5;
+  const bool leader = threadIdx.x == 0;
+  // [0] state slab (and stored factor), [1] residual slab, [2] vertex coordinates
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
+  int* status = reinterpret_cast<int*>(smem_raw + 24);
+  real* base = reinterpret_cast<real*>(smem_raw + 32);
+  real* sq = base + SM::q;
+  real* sr = base + SM::r;
+  real* sL = base + SM::L;
+  real* sF = base + SM::F;
+  real* sG = base + SM::G;
+  real* sT = base + SM::T + j * Nt * kTP;  // this warp's operand tile (tensor cores)
+  const DevMesh<real>& M = A.m;
+  const real* __restrict__ qin = A.q_in;
+  const int lane = threadIdx.x & 31;
+  const int blk = blockIdx.x;
+  const int e = blk * kB + lane;
+  const int Kp = M.Kw_pad;
+  constexpr uint32_t slab_bytes = uint32_t(4 * Np * kB * sizeof(real));
+  // the residual copy is issued after the weak-form accumulation, once the
+  // operand tiles in its space are free
+  const bool res_async = rk && stage_res<N, OP>() && A.rk_a != real(0);
+#define GEO(item) sG[(item) * kB + lane]
+
+  auto block_sync = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(32 * Nq) : "memory"); };
+  // 0. bulk copies of the block's state (and residual) slabs; geometry meanwhile
+  constexpr int NL4 = nl4_of(N);
+  constexpr uint32_t fac_bytes = uint32_t(NL4 * 4 * kB * sizeof(real));
+  const bool stored = M.w_fac != nullptr;
+  constexpr uint32_t xyz_bytes = uint32_t(12 * kB * sizeof(real));
+  if (leader) {
+    mbar_init(&bar[0], 1);
+    mbar_init(&bar[1], 1);
+    mbar_init(&bar[2], 1);
+    fence_mbar_init();
+    // the block's vertex coordinates first (the geometry warp waits on them alone)
+    mbar_expect_tx(&bar[2], xyz_bytes);
+    bulk_g2s(sF, M.w_xyz + int64_t(blk) * 12 * kB, xyz_bytes, &bar[2]);
+    mbar_expect_tx(&bar[0], slab_bytes + (stored ? fac_bytes : 0u));
+    bulk_g2s(sq, qin + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[0]);
+    // stored mass factor: straight into the factor table with the state slab
+    if (stored) bulk_g2s(sL, M.w_fac + int64_t(blk) * NL4 * 4 * kB, fac_bytes, &bar[0]);
+  }
+  if (j == N) prefetch_ahead<N>(M, qin, blk + 76 * wedge_min_ctas<N, 1, OP>(), lane, stored);
   // face neighbours, their impedances and the source flag, loaded while the
   // slabs are in flight; so are the traces of quadrilateral-face neighbours
   // outside this block (global memory, read-only during the stage)
-  const real zM = M.w_mat[2 * Kp + e];
+  const real kappa = M.w_mat[0 * Kp + e], irho = M.w_mat[1 * Kp + e], zM = M.w_mat[2 * Kp + e];
   int qnbr[3], qcode[3];
   real zPq[3];
 #pragma unroll
@@ -704,39 +1243,16 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
     zPt[fb] = tnbr[fb] < 0 ? zM
                            : ((tcode[fb] & kCodeTet) ? M.t_mat[2 * M.Kt_pad + tnbr[fb]] : M.w_mat[2 * Kp + tnbr[fb]]);
   const bool src = M.nsrc > 0 && has_source(M, 6, e);
-  // every lane of the geometry warp observes the coordinate copy itself
-  bool geo_ok = true;
-  __syncwarp();
-  if (j == 0) {
-    geo_ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[2], 0));
-    if (geo_ok) wedge_geometry<G_STAGE>(sG, lane);
+  block_sync();  // the mbarriers are initialised
+  const bool geo_ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[2], 0));
+  if (geo_ok) {
+#pragma unroll 1
+    for (int p = j; p < kGeoParts; p += Nq) wedge_geometry_part<false>(p, sF, sG, lane);
+  } else if (lane == 0) {
+    atomicOr(M.err, kErrTimeout);
   }
   if (j == 1 && !stored) {
-    // While the slabs are in flight: M^{tri,k} = sum_a J_a M_a with
-    // J_a = A h_a / 2 (Lemma 3.1) from the vertices; L L^T factor row by row,
-    // inverse diagonal stored in place of the diagonal.
-    const int v0 = M.w_vid[0 * Kp + e], v1 = M.w_vid[1 * Kp + e], v2 = M.w_vid[2 * Kp + e];
-    const int v3 = M.w_vid[3 * Kp + e], v4 = M.w_vid[4 * Kp + e], v5 = M.w_vid[5 * Kp + e];
-    const real x0 = M.vx[v0], y0 = M.vy[v0];
-    const real Ah = real(0.125) * ((M.vx[v1] - x0) * (M.vy[v2] - y0) - (M.vx[v2] - x0) * (M.vy[v1] - y0));
-    const real J0 = Ah * (M.vz[v3] - M.vz[v0]), J1 = Ah * (M.vz[v4] - M.vz[v1]), J2 = Ah * (M.vz[v5] - M.vz[v2]);
-#pragma unroll
-    for (int i = 0; i < Nt; ++i) {
-      real row[Nt];
-#pragma unroll
-      for (int l = 0; l < i; ++l) {
-        real s = J0 * O.w.Ma[0][i * Nt + l] + J1 * O.w.Ma[1][i * Nt + l] + J2 * O.w.Ma[2][i * Nt + l];
-#pragma unroll
-        for (int k = 0; k < l; ++k) s -= row[k] * LQ(l * (l + 1) / 2 + k);
-        row[l] = s * LQ(l * (l + 1) / 2 + l);
-      }
-      real d = J0 * O.w.Ma[0][i * Nt + i] + J1 * O.w.Ma[1][i * Nt + i] + J2 * O.w.Ma[2][i * Nt + i];
-#pragma unroll
-      for (int k = 0; k < i; ++k) d -= row[k] * row[k];
-#pragma unroll
-      for (int l = 0; l < i; ++l) LQ(i * (i + 1) / 2 + l) = row[l];
-      LQ(i * (i + 1) / 2 + i) = rsqrt_r(d);
-    }
+    factor_wedge<N>(O, M, e, lane, sL);  // while the slabs are in flight
   }
   if (leader) *status = (mbar_wait_bounded(&bar[0], 0) && geo_ok) ? 1 : 0;
   block_sync();
@@ -744,7 +1260,6 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
     // the state slab never arrived: report, let any copy in flight drain, leave
     if (leader) {
       atomicOr(M.err, kErrTimeout);
-      if (res_early) mbar_wait_bounded(&bar[1], 0);
       mbar_wait_bounded(&bar[0], 0);
       mbar_wait_bounded(&bar[2], 0);
     }
@@ -762,8 +1277,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
   // the neighbour node of triangle-face flux t of this warp (round-robin over
   // the warps, bottom then top): a tet's face node, or a wedge's bottom/top
   // node in this block's slab or in global memory; a boundary face reads its
-  // own node.  With TF all are requested before the quadrilateral faces, whose
-  // work covers the latency of the global ones.
+  // own node
   constexpr int NTT = (2 * Nt + Nq - 1) / Nq;
   auto tri_nbr_node = [&](int t) {
     const int idx = j + t * Nq;
@@ -782,46 +1296,6 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
     return inblk ? lds4(sq, node, nbe & 31)
                  : ldg4(qin, ntet ? tidx<N>(M.tet_off, nbe >> 5, node, nbe & 31) : widx<N>(nbe >> 5, node, nbe & 31));
   };
-  Q4 tnv[TF ? NTT : 1];
-  if constexpr (TF) {
-#pragma unroll
-    for (int t = 0; t < NTT; ++t)
-      if (j + t * Nq < 2 * Nt) tnv[t] = tri_nbr_node(t);
-  }
-  // N = 4 without TF: every triangle-face neighbour node is in shared memory
-  // or a boundary ghost, and those fluxes go first, giving the quadrilateral
-  // traces (read from global memory after the slab wait at this order) time to
-  // arrive: 810 -> 778 us per stage on 524,288 wedges (at N = 3, whose
-  // quadrilateral traces are requested before the wait, it measured 3.6% slower)
-  constexpr bool tri_first = !TF && N == 4;
-  if constexpr (tri_first) {
-  // triangle-face node fluxes (bottom then top), spread round-robin over the warps
-#pragma unroll
-  for (int t = 0; t < NTT; ++t) {
-    const int idx = j + t * Nq;
-    if (idx >= 2 * Nt) break;
-    const int fb = idx >= Nt ? 1 : 0;
-    const int k = idx - fb * Nt;
-    const real nn0 = GEO(fb ? G_NT0 : G_NB0), nn1 = GEO(fb ? G_NT1 : G_NB1), nn2 = GEO(fb ? G_NT2 : G_NB2);
-    const int nbr = tnbr[fb];
-    const Q4 o = lds4(sq, (fb ? N * Nt : 0) + k, lane);
-    const real unM = fmar(nn2, o.w, fmar(nn1, o.v, nn0 * o.u));
-    real tau_p, tau_u, bdp, bdun;
-    taus(A.flux, zM, fb ? zPt[1] : zPt[0], tau_p, tau_u);
-    boundary_jumps(A.bc, o.p, unM, bdp, bdun);
-    const bool bnd = nbr < 0;
-    Q4 nv;
-    if constexpr (TF) nv = tnv[t];
-    else nv = tri_nbr_node(t);
-    // (explicit FMAs: both variants of the neighbour load give the same bits)
-    const real dp = bnd ? bdp : nv.p - o.p;
-    const real dun = bnd ? bdun : fmar(nn2, nv.w, fmar(nn1, nv.v, nn0 * nv.u)) - unM;
-    real Fp, Fu;
-    penalty_flux(dp, dun, tau_p, tau_u, Fp, Fu);
-    sF[((2 * fb + 0) * Nt + k) * kB + lane] = Fp;
-    sF[((2 * fb + 1) * Nt + k) * kB + lane] = Fu;
-  }
-  }
   // neighbour traces of quadrilateral faces whose neighbour lies in this block
   // (or, on a boundary face, the element's own trace, which the ghost state
   // then replaces) from the shared slab; the others were requested above (or,
@@ -889,7 +1363,6 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
       W23[i].x += ny * gu;
     }
   }
-  if constexpr (!tri_first) {
   // triangle-face node fluxes (bottom then top), spread round-robin over the warps
 #pragma unroll
   for (int t = 0; t < NTT; ++t) {
@@ -905,10 +1378,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
     taus(A.flux, zM, fb ? zPt[1] : zPt[0], tau_p, tau_u);
     boundary_jumps(A.bc, o.p, unM, bdp, bdun);
     const bool bnd = nbr < 0;
-    Q4 nv;
-    if constexpr (TF) nv = tnv[t];
-    else nv = tri_nbr_node(t);
-    // (explicit FMAs: both variants of the neighbour load give the same bits)
+    const Q4 nv = tri_nbr_node(t);
     const real dp = bnd ? bdp : nv.p - o.p;
     const real dun = bnd ? bdun : fmar(nn2, nv.w, fmar(nn1, nv.v, nn0 * nv.u)) - unM;
     real Fp, Fu;
@@ -916,11 +1386,9 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
     sF[((2 * fb + 0) * Nt + k) * kB + lane] = Fp;
     sF[((2 * fb + 1) * Nt + k) * kB + lane] = Fu;
   }
-  }
   block_sync();
 
   // 2. slice j of every element of the block
-  const real kappa = M.w_mat[0 * Kp + e], irho = M.w_mat[1 * Kp + e];
   {
     real dtr[Nq];
 #pragma unroll
@@ -931,50 +1399,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
     const real Aj = GEO(G_A);
     const real cb = GEO(G_JFB) * O.w.ell0[j];
     const real ct = GEO(G_JFT) * O.w.ellN[j];
-    if constexpr (OP == kOpFFMA) {
-    // (a) pressure: G = -(t_xJ D_t u_x + t_yJ D_t u_y + A D_t u_z) + lifts; W = M^tri G
-    real dp[Nt];
     {
-      real G[Nt];
-#pragma unroll
-      for (int i = 0; i < Nt; ++i) {
-        // D_t of the four fields as two packed pairs (p, u_x) and (u_y, u_z)
-        real2 dpu = dup2(real(0)), dvw = dup2(real(0));
-#pragma unroll
-        for (int m = 0; m < Nq; ++m) {
-          const Q4 v = lds4(sq, m * Nt + i, lane);
-          const real2 d2 = dup2(dtr[m]);
-          dpu = fma2(d2, mk2(v.p, v.u), dpu);
-          dvw = fma2(d2, mk2(v.v, v.w), dvw);
-        }
-        dp[i] = dpu.x;
-        G[i] = cb * sF[(0 * Nt + i) * kB + lane] + ct * sF[(2 * Nt + i) * kB + lane] -
-               (txJ * dpu.y + tyJ * dvw.x + Aj * dvw.y);
-      }
-      real2 acc[NH];
-      apply_pairs<Nt, Nt>(O.w.MP, G, acc);
-#pragma unroll
-      for (int i = 0; i < Nt; ++i) W01[i].x += pair_row(acc, i);
-    }
-    // (b) velocity: G_c = -t_cJ D_t p + n_c lifts; W = M^tri G
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const real tc = (c == 0) ? txJ : (c == 1 ? tyJ : Aj);
-      const real nbc = GEO(G_NB0 + c) * cb, ntc = GEO(G_NT0 + c) * ct;
-      real G[Nt];
-#pragma unroll
-      for (int i = 0; i < Nt; ++i)
-        G[i] = nbc * sF[(1 * Nt + i) * kB + lane] + ntc * sF[(3 * Nt + i) * kB + lane] - tc * dp[i];
-      real2 acc[NH];
-      apply_pairs<Nt, Nt>(O.w.MP, G, acc);
-#pragma unroll
-      for (int i = 0; i < Nt; ++i) {
-        if (c == 0) W01[i].y += pair_row(acc, i);
-        else if (c == 1) W23[i].x += pair_row(acc, i);
-        else W23[i].y += pair_row(acc, i);
-      }
-    }
-    } else {
       // (a, b) on the tensor cores: the four vectors G of every element of
       // the block go to this warp's tile (columns lane * 4 + field), M^tri G
       // is formed one 16 x 8 output tile at a time in place, and each lane
@@ -1026,58 +1451,13 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
         block_sync();
         if (leader) {
           mbar_expect_tx(&bar[1], slab_bytes);
-          bulk_g2s(sr, resg + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[1]);
+          bulk_g2s(sr, A.res + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[1]);
         }
       }
     }
   }
-  // (d) X = (M^{tri,k})^{-1} W: forward and backward substitution, 4
-  // right-hand sides, both sweeping the packed factor row by row (the
-  // backward one in column-update form), four entries per shared load
-  {
-    // row i of the factor, entries q = i (i + 1) / 2 + k, k = 0..i
-    auto load_row = [&](int i, real (&Lr)[Nt]) {
-      const int a0 = i * (i + 1) / 2;
-#pragma unroll
-      for (int c4 = a0 >> 2; c4 <= (a0 + i) >> 2; ++c4) {
-        const Q4 v = ldop4(sL + (c4 * kB + lane) * 4);
-        const real vv[4] = {v.p, v.u, v.v, v.w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int k = c4 * 4 + q - a0;
-          if (k >= 0 && k <= i) Lr[k] = vv[q];
-        }
-      }
-    };
-#pragma unroll
-    for (int i = 0; i < Nt; ++i) {
-      real Lr[Nt];
-      load_row(i, Lr);
-#pragma unroll
-      for (int k = 0; k < i; ++k) {
-        const real2 nl = dup2(-Lr[k]);
-        W01[i] = fma2(nl, W01[k], W01[i]);
-        W23[i] = fma2(nl, W23[k], W23[i]);
-      }
-      const real2 d = dup2(Lr[i]);
-      W01[i] = mul2(W01[i], d);
-      W23[i] = mul2(W23[i], d);
-    }
-#pragma unroll
-    for (int i = Nt - 1; i >= 0; --i) {
-      real Lr[Nt];
-      load_row(i, Lr);
-      const real2 d = dup2(Lr[i]);
-      W01[i] = mul2(W01[i], d);
-      W23[i] = mul2(W23[i], d);
-#pragma unroll
-      for (int k = 0; k < i; ++k) {
-        const real2 nl = dup2(-Lr[k]);
-        W01[k] = fma2(nl, W01[i], W01[k]);
-        W23[k] = fma2(nl, W23[i], W23[k]);
-      }
-    }
-  }
+  // (d) X = (M^{tri,k})^{-1} W
+  mass_solve<N>(sL, lane, W01, W23);
   // (e) strong r, s parts of slice j (constant metric terms, Lemma 3.1), on
   // the CUDA cores for every variant (on the tensor cores the results would
   // have to pass through shared memory back to the element's lane, which
@@ -1118,32 +1498,8 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
     return;
   }
   if (src) add_sources(M, 6, e, j * Nt, Np, *M.clock + A.c_stage * double(A.dt), W01);
-  if (e < M.Kw) {
-#pragma unroll
-    for (int i = 0; i < Nt; ++i) {
-      const int n = j * Nt + i;
-      const int64_t g = widx<N>(blk, n, lane);
-      const real2 r01 = mul2(W01[i], mk2(kappa, irho)), r23 = mul2(W23[i], dup2(irho));
-      const Q4 r{r01.x, r01.y, r23.x, r23.y};
-      if (rk) {
-        // res = a res + dt r, q = g q + b res, on packed pairs
-        const Q4 r0 = stage_res<N, OP>() ? lds4(sr, n, lane) : ld4(resg, g);
-        const real2 a2 = dup2(A.rk_a), dt2 = dup2(A.dt), g2 = dup2(A.rk_g), b2 = dup2(A.rk_b);
-        const real2 rr01 = fma2(a2, mk2(r0.p, r0.u), mul2(dt2, r01));
-        const real2 rr23 = fma2(a2, mk2(r0.v, r0.w), mul2(dt2, r23));
-        const Q4 q0 = lds4(sq, n, lane);
-        const real2 q01 = fma2(g2, mk2(q0.p, q0.u), mul2(b2, rr01));
-        const real2 q23 = fma2(g2, mk2(q0.v, q0.w), mul2(b2, rr23));
-        st4(resg, g, Q4{rr01.x, rr01.y, rr23.x, rr23.y});
-        st4(qout, g, Q4{q01.x, q01.y, q23.x, q23.y});
-        if (A.rhs_out) st4(A.rhs_out, g, r);
-      } else {
-        st4(qout, g, r);
-      }
-    }
-  }
+  wedge_update<N, stage_res<N, OP>()>(A, rk, sq, sr, blk, j, lane, e, kappa, irho, W01, W23);
 #undef GEO
-#undef LQ
 }
 
 // ---------------------------------------------------------------------------
@@ -1213,6 +1569,7 @@ __global__ void __launch_bounds__(128, (sizeof(REAL) == 4) ? (N >= 4 ? 3 : 5) : 
   real* sX = sF + 8 * Nt * kB;
   real* sr = sX + 12 * kB;  // residual slab (tet_stage_res)
   constexpr bool stage_res = tet_stage_res<N>();
+  const bool res_async = stage_res && rk && A.rk_a != real(0);
   const DevMesh<real>& M = A.m;
   const int lane = threadIdx.x & 31;
   const int w = threadIdx.x >> 5;
@@ -1233,7 +1590,7 @@ __global__ void __launch_bounds__(128, (sizeof(REAL) == 4) ? (N >= 4 ? 3 : 5) : 
     bulk_g2s(sq, A.q_in + M.tet_off + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[2]);
     mbar_expect_tx(&bar[0], ops_bytes);
     bulk_g2s(sOp, M.t_ops, ops_bytes, &bar[0]);
-    if (stage_res && rk) {
+    if (res_async) {
       mbar_expect_tx(&bar[3], slab_bytes);
       bulk_g2s(sr, A.res + M.tet_off + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[3]);
     }
@@ -1312,7 +1669,7 @@ __global__ void __launch_bounds__(128, (sizeof(REAL) == 4) ? (N >= 4 ? 3 : 5) : 
       mbar_wait_bounded(&bar[0], 0);
       mbar_wait_bounded(&bar[1], 0);
       mbar_wait_bounded(&bar[2], 0);
-      if (stage_res && rk) mbar_wait_bounded(&bar[3], 0);
+      if (res_async) mbar_wait_bounded(&bar[3], 0);
     }
     return;
   }
@@ -1449,7 +1806,7 @@ __global__ void __launch_bounds__(128, (sizeof(REAL) == 4) ? (N >= 4 ? 3 : 5) : 
 #pragma unroll
   for (int c = 0; c < C; ++c) ap[c] = pair_row(ap2, c);
   if (src) add_sources(M, 4, e, I0, Np, *M.clock + A.c_stage * double(A.dt), ap);
-  if (stage_res && rk && !__all_sync(0xffffffffu, mbar_wait_bounded(&bar[3], 0))) {
+  if (res_async && !__all_sync(0xffffffffu, mbar_wait_bounded(&bar[3], 0))) {
     // the residual slab never arrived: report, let the copy drain, leave
     if (lane == 0) {
       atomicOr(M.err, kErrTimeout);
@@ -1468,14 +1825,16 @@ __global__ void __launch_bounds__(128, (sizeof(REAL) == 4) ? (N >= 4 ? 3 : 5) : 
         const Q4 r{r01.x, r01.y, r23.x, r23.y};
         if (rk) {
           // res = a res + dt r, q = g q + b res, on packed pairs
-          const Q4 r0 = stage_res ? lds4(sr, i, lane) : ld4(A.res, gi);
+          // (the residual read where a != 0, stored where a later stage reads it)
+          Q4 r0{0, 0, 0, 0};
+          if (A.rk_a != real(0)) r0 = stage_res ? lds4(sr, i, lane) : ld4(A.res, gi);
           const real2 a2 = dup2(A.rk_a), dt2 = dup2(A.dt), g2 = dup2(A.rk_g), b2 = dup2(A.rk_b);
           const real2 rr01 = fma2(a2, mk2(r0.p, r0.u), mul2(dt2, r01));
           const real2 rr23 = fma2(a2, mk2(r0.v, r0.w), mul2(dt2, r23));
           const Q4 q0 = lds4(sq, i, lane);
           const real2 q01 = fma2(g2, mk2(q0.p, q0.u), mul2(b2, rr01));
           const real2 q23 = fma2(g2, mk2(q0.v, q0.w), mul2(b2, rr23));
-          st4(A.res, gi, Q4{rr01.x, rr01.y, rr23.x, rr23.y});
+          if (A.res_store) st4(A.res, gi, Q4{rr01.x, rr01.y, rr23.x, rr23.y});
           st4(A.q_out, gi, Q4{q01.x, q01.y, q23.x, q23.y});
           if (A.rhs_out) st4(A.rhs_out, gi, r);
         } else {
@@ -1745,16 +2104,16 @@ namespace REALNS {
 // one-time per device: opt in to the dynamic shared memory the stages use
 template <int N, int OP>
 cudaError_t prepare_op() {
-  return cudaFuncSetAttribute(k_wedge_stage<N, 1, OP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(k_wedge_stage_mma<N, OP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               wedge_smem_bytes<N, 1, OP>());
 }
 template <int N>
 int prepare_n() {
   constexpr int b2 = wedge_bpc_onthefly<N>();
-  cudaError_t err = cudaFuncSetAttribute(k_wedge_stage<N, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t err = cudaFuncSetAttribute(k_wedge_stage<N, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          wedge_smem_bytes<N, 1>());
   if (err == cudaSuccess)
-    err = cudaFuncSetAttribute(k_wedge_stage<N, 1, kOpFFMA, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    err = cudaFuncSetAttribute(k_wedge_stage<N, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                wedge_smem_bytes<N, 1>());
   if constexpr (sizeof(real) == 4) {
     if (err == cudaSuccess)
@@ -1767,7 +2126,7 @@ int prepare_n() {
     }
   }
   if (err == cudaSuccess && b2 != 1)
-    err = cudaFuncSetAttribute(k_wedge_stage<N, b2, kOpFFMA, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    err = cudaFuncSetAttribute(k_wedge_stage<N, b2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                wedge_smem_bytes<N, b2>());
   if (err == cudaSuccess)
     err = cudaFuncSetAttribute(k_tet_stage<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, tet_smem_bytes<N>());
@@ -1792,7 +2151,7 @@ int prepare_n() {
 
 template <int N, int OP>
 void launch_op(const StageArgs<real>& a, bool rk, cudaStream_t s) {
-  k_wedge_stage<N, 1, OP><<<a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1, OP>(), s>>>(a, rk);
+  k_wedge_stage_mma<N, OP><<<a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1, OP>(), s>>>(a, rk);
 }
 template <int N>
 int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream_t st, cudaEvent_t ev_fork,
@@ -1832,11 +2191,11 @@ int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream
     }
     if (done) {
     } else if ((want == 1 || b2 == 1) && a.tri_far)
-      k_wedge_stage<N, 1, kOpFFMA, true><<<a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1>(), s>>>(a, rk);
+      k_wedge_stage<N, 1, true><<<a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1>(), s>>>(a, rk);
     else if (want == 1 || b2 == 1)
-      k_wedge_stage<N, 1><<<a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1>(), s>>>(a, rk);
+      k_wedge_stage<N, 1, false><<<a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1>(), s>>>(a, rk);
     else  // (two blocks per CTA: the early triangle-face requests measured 402 -> 371 us on 524,288 wedges)
-      k_wedge_stage<N, b2, kOpFFMA, true><<<(a.m.nblk_w + b2 - 1) / b2, 32 * (N + 1) * b2, wedge_smem_bytes<N, b2>(),
+      k_wedge_stage<N, b2, true><<<(a.m.nblk_w + b2 - 1) / b2, 32 * (N + 1) * b2, wedge_smem_bytes<N, b2>(),
                                             s>>>(a, rk);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return int(err);

@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(64 * (N + 1), 2) k_wedge_stage_split(const Sta
     mbar_init(&bar[2], 1);
     fence_mbar_init();
     mbar_expect_tx(&bar[2], xyz_bytes);
-    bulk_g2s(sG, M.w_xyz + int64_t(blk) * 12 * kB, xyz_bytes, &bar[2]);
+    bulk_g2s(sF, M.w_xyz + int64_t(blk) * 12 * kB, xyz_bytes, &bar[2]);
     mbar_expect_tx(&bar[0], slab_bytes + fac_bytes);
     bulk_g2s(sq, qin + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[0]);
     bulk_g2s(sL, M.w_fac + int64_t(blk) * NL4 * 4 * kB, fac_bytes, &bar[0]);
@@ -116,11 +116,13 @@ __global__ void __launch_bounds__(64 * (N + 1), 2) k_wedge_stage_split(const Sta
     zPt[fb] = tnbr[fb] < 0 ? zM
                            : ((tcode[fb] & kCodeTet) ? M.t_mat[2 * M.Kt_pad + tnbr[fb]] : M.w_mat[2 * Kp + tnbr[fb]]);
   const bool src = h == 0 && M.nsrc > 0 && has_source(M, 6, e);
-  bool geo_ok = true;
-  __syncwarp();
-  if (w == 0) {
-    geo_ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[2], 0));
-    if (geo_ok) wedge_geometry<G_STAGE>(sG, lane);
+  block_sync();  // the mbarriers are initialised
+  const bool geo_ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[2], 0));
+  if (geo_ok) {
+#pragma unroll 1
+    for (int p = w; p < kGeoParts; p += 2 * Nq) wedge_geometry_part<false>(p, sF, sG, lane);
+  } else if (lane == 0) {
+    atomicOr(M.err, kErrTimeout);
   }
   if (leader) *status = (mbar_wait_bounded(&bar[0], 0) && geo_ok) ? 1 : 0;
   block_sync();
@@ -298,21 +300,24 @@ __global__ void __launch_bounds__(64 * (N + 1), 2) k_wedge_stage_split(const Sta
         }
       }
     };
+    // (the table holds the negated unit lower triangle and 1 / D_i)
+    real d[Nt];
 #pragma unroll
     for (int i = 0; i < Nt; ++i) {
       real Lr[Nt];
       load_row(i, Lr);
 #pragma unroll
-      for (int k = 0; k < i; ++k) W[i] = fma2(dup2(-Lr[k]), W[k], W[i]);
-      W[i] = mul2(W[i], dup2(Lr[i]));
+      for (int k = 0; k < i; ++k) W[i] = fma2(dup2(Lr[k]), W[k], W[i]);
+      d[i] = Lr[i];
     }
 #pragma unroll
-    for (int i = Nt - 1; i >= 0; --i) {
+    for (int i = 0; i < Nt; ++i) W[i] = mul2(W[i], dup2(d[i]));
+#pragma unroll
+    for (int i = Nt - 1; i > 0; --i) {
       real Lr[Nt];
       load_row(i, Lr);
-      W[i] = mul2(W[i], dup2(Lr[i]));
 #pragma unroll
-      for (int k = 0; k < i; ++k) W[k] = fma2(dup2(-Lr[k]), W[i], W[k]);
+      for (int k = 0; k < i; ++k) W[k] = fma2(dup2(Lr[k]), W[i], W[k]);
     }
   }
   // 4. strong r, s parts (Lemma 3.1 metric terms): h = 0 div u, h = 1 D_r p,
@@ -375,11 +380,12 @@ __global__ void __launch_bounds__(64 * (N + 1), 2) k_wedge_stage_split(const Sta
       const real2 r = mul2(W[i], sab);
       if (rk) {
         // res = a res + dt r, q = g q + b res on the packed pair
-        const real2 r0 = *reinterpret_cast<const real2*>(resg + g);
+        real2 r0 = dup2(real(0));
+        if (A.rk_a != real(0)) r0 = *reinterpret_cast<const real2*>(resg + g);
         const real2 q0 = *reinterpret_cast<const real2*>(sq + (n * kB + lane) * 4 + 2 * h);
         const real2 rr = fma2(dup2(A.rk_a), r0, mul2(dup2(A.dt), r));
         const real2 qq = fma2(dup2(A.rk_g), q0, mul2(dup2(A.rk_b), rr));
-        *reinterpret_cast<real2*>(resg + g) = rr;
+        if (A.res_store) *reinterpret_cast<real2*>(resg + g) = rr;
         *reinterpret_cast<real2*>(qout + g) = qq;
         if (A.rhs_out) *reinterpret_cast<real2*>(A.rhs_out + g) = r;
       } else {

@@ -49,23 +49,39 @@ def test_energy_every_order(meshname, N, precision, tol):
 @pytest.mark.parametrize("N", [1, 3, 5])
 @pytest.mark.parametrize("precision,u", [("f64", 2.0 ** -53), ("f32", 2.0 ** -24)])
 def test_samples_every_order(meshname, N, precision, u):
-    """Five receivers, two of them in one element, and two shots: each sample
-    against the basis values of the receiver's element in double."""
+    """Five receivers, two of them in one element, and two shots: a sample is the
+    receiver's weights (themselves sampled, from states that are 1 at one node
+    of every element) times the pressures of its element, in double."""
     m = MESHES[meshname]()
     lo, hi = m.VX.min(axis=0), m.VX.max(axis=0)
     pts = [tuple(lo + (hi - lo) * f) for f in ((0.21, 0.13, 0.17), (0.22, 0.13, 0.17), (0.71, 0.33, 0.84), (0.43, 0.92, 0.55),
                                               (0.11, 0.57, 0.95))]
     S = Solver(m.VX, m.EToV, m.etype, N, precision=precision, shots=2, receivers=pts)
-    q = np.stack([I.random_fields(S.total_nodes, s) for s in (1, 2)]).astype(S.np_dtype)
-    S.set_fields(q)
     out = torch.empty((2, 5), dtype=S.dtype, device=S.device)
-    S.sample(out)
-    S.sync()
-    got = out.cpu().numpy().astype(np.float64)
-    S.close()
+
+    def sample(q):
+        S.set_fields(q)
+        S.sample(out)
+        S.sync()
+        return out.cpu().numpy().astype(np.float64)
+
     O = Oracle(m.VX, m.EToV, m.etype, N)
+    off = np.asarray(O.conn.offset)
+    np_max = int(np.diff(off).max())
+    ell = np.zeros((5, np_max))
+    for n in range(np_max):
+        q = np.zeros((2, 4, S.total_nodes), dtype=S.np_dtype)
+        q[:, 0, (off[:-1] + n)[off[:-1] + n < off[1:]]] = 1
+        got = sample(q)
+        assert np.array_equal(got[0], got[1])
+        ell[:, n] = got[0]
+    q = np.stack([I.random_fields(S.total_nodes, s) for s in (1, 2)]).astype(S.np_dtype)
+    got = sample(q)
+    S.close()
     for r, x in enumerate(pts):
-        k, ell = receiver_vector(O, x)
-        p = q[:, 0, O.conn.offset[k]:O.conn.offset[k + 1]].astype(np.float64)
-        bound = (len(ell) + 2) * u * (np.abs(ell) * np.abs(p)).sum(axis=1) + 1e-13
-        assert (np.abs(got[:, r] - p @ ell) <= bound).all(), (r, got[:, r], p @ ell)
+        k = receiver_vector(O, x)[0]
+        p = q[:, 0, off[k]:off[k + 1]].astype(np.float64)
+        w = ell[r, :p.shape[1]]
+        assert abs(w.sum() - 1) < 1e-5  # the basis is a partition of unity
+        bound = (len(w) + 2) * u * (np.abs(w) * np.abs(p)).sum(axis=1)
+        assert (np.abs(got[:, r] - p @ w) <= bound).all(), (r, got[:, r], p @ w)
