@@ -1152,6 +1152,372 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
 #undef GEO
 }
 
+// Small meshes.  With a block per N + 1 warps a mesh of a few hundred wedges
+// leaves most SMs idle and its stage takes as long as one warp's instruction
+// chain (and in FP64 as the few busy SMs' FP64 pipes).  Here a CTA takes one
+// slice j of a block and its four warps share the slice's work, warp f solving
+// for field f: N + 1 times the CTAs and a quarter of the chain, for the
+// triangle-face fluxes formed once per slice instead of once per block.  Every
+// result is accumulated in k_wedge_stage's order: same bits.
+template <int N>
+struct WideSmem {
+  static constexpr int Nt = nt_of(N), Nq = N + 1, Np = Nt * Nq;
+  static constexpr int q = 0;                         // [Np][32][4] state slab
+  static constexpr int r = q + 4 * Np * kB;           // [Nt][32][4] the slice's residual
+  static constexpr int L = r + 4 * Nt * kB;           // [NL4][32][4] mass factor
+  static constexpr int F = L + nl4_of(N) * 4 * kB;    // [2][Nt][32] flux pairs; then the results [4][Nt][32]
+  static constexpr int G = F + 4 * Nt * kB;           // [G_STAGE][32] geometry
+  static constexpr int D = G + G_STAGE * kB;          // [2][Nt][32] D_t p, t-divergence; then [3][Nt][32] strong parts
+  static constexpr int E = D + 3 * Nt * kB;           // [3][Nq][2][32] quadrilateral-face lifts of F_p, F_u
+  static constexpr int reals = E + 6 * Nq * kB;
+};
+template <int N>
+__host__ __device__ constexpr int wide_smem_bytes() {
+  return 32 + WideSmem<N>::reals * int(sizeof(real));
+}
+// (FP64 at N = 5 does not fit a CTA's shared memory)
+template <int N>
+__host__ __device__ constexpr bool wide_fits() {
+  return wide_smem_bytes<N>() <= 227 * 1024;
+}
+
+// row pairs [H0, H1) of the strong divergence D_r (r.u) + D_s (s.u) of slice j
+template <int N, int H0, int H1, int HA>
+__device__ __forceinline__ void div_rows(const AllOps<N, real>& O, const real* sq, int j, int lane, real rx, real ry, real sx,
+                                         real sy, real2 (&dv)[HA]) {
+  constexpr int Nt = nt_of(N);
+#pragma unroll
+  for (int h = 0; h < HA; ++h) dv[h] = dup2(real(0));
+#pragma unroll
+  for (int l = 0; l < Nt; ++l) {
+    const Q4 v = lds4(sq, j * Nt + l, lane);
+    const real2 ab = fma2(dup2(v.u), mk2(rx, sx), mul2(dup2(v.v), mk2(ry, sy)));
+#pragma unroll
+    for (int h = H0; h < H1; ++h) {
+      dv[h - H0] = fma_rows<Nt>(O.w.DrP, h, l, ab.x, dv[h - H0], dr_zero(N, 2 * h, l), dr_zero(N, 2 * h + 1, l));
+      dv[h - H0] = fma_rows<Nt>(O.w.DsP, h, l, ab.y, dv[h - H0], ds_zero(N, 2 * h, l), ds_zero(N, 2 * h + 1, l));
+    }
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(128) k_wedge_wide(const StageArgs<real> A, bool rk) {
+  constexpr int Nt = nt_of(N), Nq = N + 1, Np = Nt * Nq, NH = (Nt + 1) / 2, NQH = (Nq + 1) / 2, NL4 = nl4_of(N);
+  using SM = WideSmem<N>;
+  const AllOps<N, real>& O = OPS<N>();
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  // [0] state slab (and stored factor), [1] residual, [2] vertex coordinates
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
+  int* status = reinterpret_cast<int*>(smem_raw + 24);
+  real* base = reinterpret_cast<real*>(smem_raw + 32);
+  real* sq = base + SM::q;
+  real* sr = base + SM::r;
+  real* sL = base + SM::L;
+  real* sF = base + SM::F;
+  real* sG = base + SM::G;
+  real* sD = base + SM::D;
+  real* sE = base + SM::E;
+  const DevMesh<real>& M = A.m;
+  const real* __restrict__ qin = A.q_in;
+  const int lane = threadIdx.x & 31, f = threadIdx.x >> 5;
+  const int blk = blockIdx.x / Nq, j = blockIdx.x - blk * Nq;
+  const int e = blk * kB + lane, Kp = M.Kw_pad;
+  constexpr uint32_t slab_bytes = uint32_t(4 * Np * kB * sizeof(real)), res_bytes = uint32_t(4 * Nt * kB * sizeof(real));
+  constexpr uint32_t fac_bytes = uint32_t(NL4 * 4 * kB * sizeof(real)), xyz_bytes = uint32_t(12 * kB * sizeof(real));
+  const bool stored = M.w_fac != nullptr, res_async = rk && A.rk_a != real(0);
+#define GEO(item) sG[(item) * kB + lane]
+  if (threadIdx.x == 0) {
+    mbar_init(&bar[0], 1);
+    mbar_init(&bar[1], 1);
+    mbar_init(&bar[2], 1);
+    fence_mbar_init();
+    mbar_expect_tx(&bar[2], xyz_bytes);
+    bulk_g2s(sF, M.w_xyz + int64_t(blk) * 12 * kB, xyz_bytes, &bar[2]);  // in the flux table's place, written later
+    mbar_expect_tx(&bar[0], slab_bytes + (stored ? fac_bytes : 0u));
+    bulk_g2s(sq, qin + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[0]);
+    if (stored) bulk_g2s(sL, M.w_fac + int64_t(blk) * NL4 * 4 * kB, fac_bytes, &bar[0]);
+    if (res_async) {
+      mbar_expect_tx(&bar[1], res_bytes);
+      bulk_g2s(sr, A.res + widx<N>(blk, j * Nt, 0), res_bytes, &bar[1]);
+    }
+  }
+  // neighbours: warp f < 3 takes quadrilateral face f, all warps share the triangle-face nodes
+  const real kappa = M.w_mat[0 * Kp + e], irho = M.w_mat[1 * Kp + e], zM = M.w_mat[2 * Kp + e];
+  const int ed = f < 3 ? f : 0;
+  const int qnbr = M.w_nbr[(2 + ed) * Kp + e], qcode = M.w_code[(2 + ed) * Kp + e];
+  const int tnbr[2] = {M.w_nbr[0 * Kp + e], M.w_nbr[1 * Kp + e]};
+  const int tcode[2] = {M.w_code[0 * Kp + e], M.w_code[1 * Kp + e]};
+  Q4 tv[Nq];
+  {
+    const bool bnd = qnbr < 0;
+    const int nbe = bnd ? e : qnbr, sh = 5 * (bnd ? 2 * ed : qcode);
+    constexpr EdgeCandidates<N> cand;
+    const real* nb = qin + widx<N>(nbe >> 5, j * Nt, nbe & 31);
+#pragma unroll
+    for (int m = 0; m < Nq; ++m) tv[m] = ldg4(nb, int((cand.c[m] >> sh) & 31u) * (kB * 4));
+  }
+  constexpr int NTT = (2 * Nt + 3) / 4;
+  Q4 tnv[NTT];
+#pragma unroll
+  for (int t = 0; t < NTT; ++t) {
+    const int idx = f + 4 * t;
+    if (idx >= 2 * Nt) break;
+    const int fb = idx >= Nt ? 1 : 0, k = idx - fb * Nt;
+    const int nbr = fb ? tnbr[1] : tnbr[0], code = fb ? tcode[1] : tcode[0];
+    const bool bnd = nbr < 0, ntet = !bnd && (code & kCodeTet) != 0;
+    const int nbe = bnd ? e : nbr, nf = bnd ? fb : (code >> 4) & 3;
+    const int nk = bnd ? k : O.tab.tri_perm[code & 15][k];
+    const int node = ntet ? O.tab.tet_face[nf][nk] : (nf ? N * Nt : 0) + nk;
+    tnv[t] = ldg4(qin, ntet ? tidx<N>(M.tet_off, nbe >> 5, node, nbe & 31) : widx<N>(nbe >> 5, node, nbe & 31));
+  }
+  const real zPq = qnbr < 0 ? zM : M.w_mat[2 * Kp + qnbr];
+  real ntp[2], ntu[2];
+#pragma unroll
+  for (int fb = 0; fb < 2; ++fb) {
+    const real zP = tnbr[fb] < 0 ? zM
+                                 : ((tcode[fb] & kCodeTet) ? M.t_mat[2 * M.Kt_pad + tnbr[fb]] : M.w_mat[2 * Kp + tnbr[fb]]);
+    real tp, tu;
+    taus(A.flux, zM, zP, tp, tu);
+    ntp[fb] = -tp;
+    ntu[fb] = -tu;
+  }
+  const bool src = f == 0 && M.nsrc > 0 && has_source(M, 6, e);
+  __syncthreads();  // the mbarriers are initialised
+  const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[2], 0));
+  if (ok) {
+#pragma unroll 1
+    for (int p = 3 - f; p < kGeoParts; p += 4) wedge_geometry_part<false>(p, sF, sG, lane);
+  } else if (lane == 0) {
+    atomicOr(M.err, kErrTimeout);
+  }
+  if (threadIdx.x == 96) *status = (ok && mbar_wait_bounded(&bar[0], 0)) ? 1 : 0;
+  if (f == 0 && !stored) factor_wedge<N>(O, M, e, lane, sL);
+  __syncthreads();
+  if (*reinterpret_cast<volatile int*>(status) == 0) {
+    // a copy never arrived: report, let the copies in flight drain, leave
+    if (threadIdx.x == 0) {
+      atomicOr(M.err, kErrTimeout);
+      mbar_wait_bounded(&bar[0], 0);
+      if (res_async) mbar_wait_bounded(&bar[1], 0);
+      mbar_wait_bounded(&bar[2], 0);
+    }
+    return;
+  }
+
+  // 1. triangle-face node fluxes; the lifts of quadrilateral face f; D_t p and
+  //    the t-divergence of the slice's nodes, four warps abreast
+#pragma unroll
+  for (int t = 0; t < NTT; ++t) {
+    const int idx = f + 4 * t;
+    if (idx >= 2 * Nt) break;
+    const int fb = idx >= Nt ? 1 : 0, k = idx - fb * Nt;
+    const real n0 = GEO(fb ? G_NT0 : G_NB0), n1 = GEO(fb ? G_NT1 : G_NB1), n2 = GEO(fb ? G_NT2 : G_NB2);
+    const Q4 o = lds4(sq, (fb ? N * Nt : 0) + k, lane);
+    const real2 F = tri_node_flux(o, tnv[t], n0, n1, n2, ghost_signs((fb ? tnbr[1] : tnbr[0]) < 0, A.bc),
+                                  fb ? ntp[1] : ntp[0], fb ? ntu[1] : ntu[0]);
+    *reinterpret_cast<real2*>(sF + ((fb * Nt + k) * kB + lane) * 2) = F;
+  }
+  if (f < 3) {
+    real tp, tu;
+    taus(A.flux, zM, zPq, tp, tu);
+    const real nx = GEO(G_QNX0 + ed), ny = GEO(G_QNY0 + ed);
+    const real ca = real(0.5) * GEO(G_QCA0 + ed), cb = real(0.5) * GEO(G_QCB0 + ed);
+    const real2 s = ghost_signs(qnbr < 0, A.bc);
+    real2 gp2[NQH], gu2[NQH];
+    if (f == 0) quad_edge<N>(O, sq, j, lane, 0, tv, nx, ny, s, tp, tu, ca, cb, gp2, gu2);
+    else if (f == 1) quad_edge<N>(O, sq, j, lane, 1, tv, nx, ny, s, tp, tu, ca, cb, gp2, gu2);
+    else quad_edge<N>(O, sq, j, lane, 2, tv, nx, ny, s, tp, tu, ca, cb, gp2, gu2);
+#pragma unroll
+    for (int m = 0; m < Nq; ++m) {
+      sE[((f * Nq + m) * 2 + 0) * kB + lane] = pair_row(gp2, m);
+      sE[((f * Nq + m) * 2 + 1) * kB + lane] = pair_row(gu2, m);
+    }
+  }
+  const real tj = O.w.gll[j];
+  const real ntx = -fmar(tj, GEO(G_TX1), GEO(G_TX0)), nty = -fmar(tj, GEO(G_TY1), GEO(G_TY0)), nA = -GEO(G_A);
+  {
+    real dtr[Nq];
+#pragma unroll
+    for (int m = 0; m < Nq; ++m) dtr[m] = O.w.Dt[j * Nq + m];
+#pragma unroll
+    for (int i = f; i < Nt; i += 4) {
+      real2 dpu = dup2(real(0)), dvw = dup2(real(0));
+#pragma unroll
+      for (int m = 0; m < Nq; ++m) {
+        const Q4 v = lds4(sq, m * Nt + i, lane);
+        const real2 d2 = dup2(dtr[m]);
+        dpu = fma2(d2, mk2(v.p, v.u), dpu);
+        dvw = fma2(d2, mk2(v.v, v.w), dvw);
+      }
+      sD[(0 * Nt + i) * kB + lane] = dpu.x;
+      sD[(1 * Nt + i) * kB + lane] = fmar(ntx, dpu.y, fmar(nty, dvw.x, nA * dvw.y));
+    }
+  }
+  __syncthreads();
+  // 2. M^tri in place on flux vector f (bottom F_p, F_u, top F_p, F_u); M^tri on
+  //    the t-divergence, onto the pressure lifts (warp 0), or on D_t p
+  {
+    real* v = sF + ((f >> 1) * Nt * kB + lane) * 2 + (f & 1);
+    real G[Nt];
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) G[i] = v[i * kB * 2];
+    real2 acc[NH];
+    apply_pairs<Nt, Nt>(O.w.MP, G, acc);
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) v[i * kB * 2] = pair_row(acc, i);
+  }
+  real2 Wm[NH];
+#pragma unroll
+  for (int h = 0; h < NH; ++h) Wm[h] = dup2(real(0));
+  if (f == 0) {
+#pragma unroll
+    for (int ec = 0; ec < 3; ++ec)
+#pragma unroll
+      for (int m = 0; m < Nq; ++m) {
+        const int i = edge_node(N, ec, m);
+        const real g = sE[((ec * Nq + m) * 2 + 0) * kB + lane];
+        if (i & 1) Wm[i >> 1].y += g;
+        else Wm[i >> 1].x += g;
+      }
+  }
+  {
+    const real* d = sD + (f == 0 ? Nt : 0) * kB + lane;
+#pragma unroll
+    for (int l = 0; l < Nt; ++l) {
+      const real2 xx = dup2(d[l * kB]);
+#pragma unroll
+      for (int h = 0; h < NH; ++h) Wm[h] = fma2(cpair(O.w.MP, Nt, h, l), xx, Wm[h]);
+    }
+  }
+  __syncthreads();
+  // 3. right-hand side of field f and its mass solve
+  real W[Nt];
+  {
+    const real cb = real(0.5) * GEO(G_JFB) * O.w.ell0[j], ct = real(0.5) * GEO(G_JFT) * O.w.ellN[j];
+    const real cbf = f == 0 ? cb : cb * GEO(G_NB0 + f - 1), ctf = f == 0 ? ct : ct * GEO(G_NT0 + f - 1);
+    const real nf = f == 1 ? ntx : (f == 2 ? nty : nA);
+    const real* F = sF + lane * 2 + (f == 0 ? 0 : 1);
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) {
+      const real md = pair_row(Wm, i);
+      W[i] = fmar(F[i * kB * 2], cbf, fmar(F[(Nt + i) * kB * 2], ctf, f == 0 ? md : nf * md));
+    }
+    if (f == 1 || f == 2) {
+#pragma unroll
+      for (int ec = 0; ec < 3; ++ec) {
+        const real n = GEO((f == 1 ? G_QNX0 : G_QNY0) + ec);
+#pragma unroll
+        for (int m = 0; m < Nq; ++m) {
+          const int i = edge_node(N, ec, m);
+          W[i] = fmar(n, sE[((ec * Nq + m) * 2 + 1) * kB + lane], W[i]);
+        }
+      }
+    }
+  }
+  {
+    auto load_row = [&](int i, real (&Lr)[Nt]) {
+      const int a0 = i * (i + 1) / 2;
+#pragma unroll
+      for (int c4 = a0 >> 2; c4 <= (a0 + i) >> 2; ++c4) {
+        const Q4 v = ldop4(sL + (c4 * kB + lane) * 4);
+        const real vv[4] = {v.p, v.u, v.v, v.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int k = c4 * 4 + q - a0;
+          if (k >= 0 && k <= i) Lr[k] = vv[q];
+        }
+      }
+    };
+    real d[Nt];
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) {
+      real Lr[Nt];
+      load_row(i, Lr);
+#pragma unroll
+      for (int k = 0; k < i; ++k) W[i] = fmar(Lr[k], W[k], W[i]);
+      d[i] = Lr[i];
+    }
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) W[i] *= d[i];
+#pragma unroll
+    for (int i = Nt - 1; i > 0; --i) {
+      real Lr[Nt];
+      load_row(i, Lr);
+#pragma unroll
+      for (int k = 0; k < i; ++k) W[k] = fmar(Lr[k], W[i], W[k]);
+    }
+  }
+  // 4. strong r, s parts: rows of div u on warps 0 and 2, D_r p on warp 1, D_s p
+  //    on warp 3, exchanged through shared memory
+  constexpr int HA = (NH + 1) / 2;
+  const real rx = GEO(G_RX), ry = GEO(G_RY), sx = GEO(G_SX), sy = GEO(G_SY);
+  real2 dv[HA], pd[NH];
+  if (f == 0) {
+    div_rows<N, 0, HA>(O, sq, j, lane, rx, ry, sx, sy, dv);
+  } else if (f == 2) {
+    div_rows<N, HA, NH>(O, sq, j, lane, rx, ry, sx, sy, dv);
+#pragma unroll
+    for (int i = 2 * HA; i < Nt; ++i) sD[i * kB + lane] = pair_row(dv, i - 2 * HA);
+  } else {
+#pragma unroll
+    for (int h = 0; h < NH; ++h) pd[h] = dup2(real(0));
+    if (f == 1) {
+#pragma unroll
+      for (int l = 0; l < Nt; ++l) {
+        const real p = sq[((j * Nt + l) * kB + lane) * 4];
+#pragma unroll
+        for (int h = 0; h < NH; ++h)
+          pd[h] = fma_rows<Nt>(O.w.DrP, h, l, p, pd[h], dr_zero(N, 2 * h, l), dr_zero(N, 2 * h + 1, l));
+      }
+    } else {
+#pragma unroll
+      for (int l = 0; l < Nt; ++l) {
+        const real p = sq[((j * Nt + l) * kB + lane) * 4];
+#pragma unroll
+        for (int h = 0; h < NH; ++h)
+          pd[h] = fma_rows<Nt>(O.w.DsP, h, l, p, pd[h], ds_zero(N, 2 * h, l), ds_zero(N, 2 * h + 1, l));
+      }
+    }
+    real* out = sD + ((f == 1 ? 1 : 2) * Nt) * kB + lane;
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) out[i * kB] = pair_row(pd, i);
+  }
+  __syncthreads();
+  if (f == 0) {
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) W[i] -= i < 2 * HA ? pair_row(dv, i < 2 * HA ? i : 0) : sD[i * kB + lane];
+    if (src) add_sources(M, 6, e, j * Nt, Np, *M.clock + A.c_stage * double(A.dt), W);
+  } else if (f < 3) {
+    const real nr = f == 1 ? -rx : -ry, ns = f == 1 ? -sx : -sy;
+#pragma unroll
+    for (int i = 0; i < Nt; ++i)
+      W[i] = fmar(nr, sD[(1 * Nt + i) * kB + lane], fmar(ns, sD[(2 * Nt + i) * kB + lane], W[i]));
+  }
+#pragma unroll
+  for (int i = 0; i < Nt; ++i) sF[(f * Nt + i) * kB + lane] = W[i];
+  // 5. the update, four fields of a node per thread
+  if (!__syncthreads_and(!res_async || mbar_wait_bounded(&bar[1], 0))) {
+    // the residual never arrived: report, let the copy drain, leave
+    if (threadIdx.x == 0) {
+      atomicOr(M.err, kErrTimeout);
+      mbar_wait_bounded(&bar[1], 0);
+    }
+    return;
+  }
+  if (e < M.Kw) {
+    const UpdateCoef U(A, kappa, irho);
+#pragma unroll
+    for (int i = f; i < Nt; i += 4) {
+      const real2 W01 = mk2(sF[(0 * Nt + i) * kB + lane], sF[(1 * Nt + i) * kB + lane]);
+      const real2 W23 = mk2(sF[(2 * Nt + i) * kB + lane], sF[(3 * Nt + i) * kB + lane]);
+      Q4 r0{0, 0, 0, 0};
+      if (res_async) r0 = lds4(sr, i, lane);
+      U.node(A, rk, widx<N>(blk, j * Nt + i, lane), W01, W23, r0, lds4(sq, j * Nt + i, lane));
+    }
+  }
+#undef GEO
+}
+
 // The stage with M^tri applied on the tensor cores (precision variants): one
 // block per CTA, the four right-hand sides of a slice formed first and passed
 // through the warp's operand tile.
@@ -2125,6 +2491,10 @@ int prepare_n() {
       if (err == cudaSuccess) err = prepare_op<N, kOpBF16>();
     }
   }
+  if constexpr (wide_fits<N>()) {
+    if (err == cudaSuccess)
+      err = cudaFuncSetAttribute(k_wedge_wide<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide_smem_bytes<N>());
+  }
   if (err == cudaSuccess && b2 != 1)
     err = cudaFuncSetAttribute(k_wedge_stage<N, b2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                wedge_smem_bytes<N, b2>());
@@ -2149,6 +2519,12 @@ int prepare_n() {
   return int(err);
 }
 
+// The small-mesh stage up to this many CTAs (blocks x slices): about one per SM.
+// us per stage of a step, small-mesh against large-mesh form, by blocks: FP32
+// N = 3 1: 5.8 / 7.0, 32: 6.4 / 7.0, 64: 7.0 / 7.4, 128: 8.0 / 7.4; N = 4
+// 32: 10.7 / 12.3, 64: 17 / 12; N = 5 32: 27 / 45; FP64 N = 3 1-32: 37 / 82,
+// 64: 58 / 82, 128: 112 / 83; N = 4 32: 131 / 192, 64: 196 / 192.
+constexpr int kWideCtas = 192;
 template <int N, int OP>
 void launch_op(const StageArgs<real>& a, bool rk, cudaStream_t s) {
   k_wedge_stage_mma<N, OP><<<a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1, OP>(), s>>>(a, rk);
@@ -2188,6 +2564,12 @@ int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream
       if (a.op == kOpTF32x3) launch_op<N, kOpTF32x3>(a, rk, s);
       else if (a.op == kOpTF32) launch_op<N, kOpTF32>(a, rk, s);
       else if (a.op == kOpBF16) launch_op<N, kOpBF16>(a, rk, s);
+    }
+    if constexpr (wide_fits<N>()) {
+      if (!done && a.wedge_bpc <= 1 && a.m.nblk_w * (N + 1) <= kWideCtas) {
+        k_wedge_wide<N><<<a.m.nblk_w * (N + 1), 128, wide_smem_bytes<N>(), s>>>(a, rk);
+        done = true;
+      }
     }
     if (done) {
     } else if ((want == 1 || b2 == 1) && a.tri_far)
