@@ -454,11 +454,12 @@ BlobLayout blob_layout(const dg_ctx* c) {
   L.wxyz = take(size_t(Kwp) * 12 * rs);
   // per tet block [12][32]: x, y, z of the four vertices
   L.txyz = take(size_t(Ktp) * 12 * rs);
-  // tet stage operators in the stage's shared-memory image: [l][i] (D_r, D_s, D_t, 0)(i, l),
-  // then the lift per warp chunk of C = ceil(Np/4) output nodes, [warp][f Nt + k][c < CP]
+  // tet stage operators in the stage's shared-memory image, per warp chunk of
+  // C = ceil(Np/4) output nodes (padded to pairs): [warp][l] records of the
+  // D_r, D_s, D_t entries (i, l) of the chunk, then [warp][f Nt + k] lift rows
   {
-    const int np = npt_of(c->N), ch = (np + 3) / 4, cp = (ch + 3) / 4 * 4;
-    L.tops = take(size_t(4 * np * np + 4 * 4 * nt_of(c->N) * cp) * rs);
+    const int np = npt_of(c->N), cp = ((np + 3) / 4 + 1) / 2 * 2;
+    L.tops = take(size_t(4 * np * ((3 * cp + 3) / 4 * 4) + 4 * 4 * nt_of(c->N) * ((cp + 3) / 4 * 4)) * rs);
   }
   L.total = o;
   return L;
@@ -623,24 +624,21 @@ void fill_blob(const dg_ctx* c, const BlobLayout& L, std::vector<unsigned char>&
   for (int i = 0; i < c->ref->Npt * c->ref->Npt; ++i) tm[i] = real(c->ref->tM.a[i]);
   // wedge energy operators: barycentric-weighted triangle masses, then the line mass
   {
+    // tet stage image, per warp chunk of output nodes by output pairs (zero past the chunk)
     const RefElems& R = *c->ref;
-    const int np = R.Npt, nt = R.Nt, ch = (np + 3) / 4, cp = (ch + 3) / 4 * 4;
+    const int np = R.Npt, nt = R.Nt, ch = (np + 3) / 4, cp = (ch + 1) / 2 * 2;
+    const int rs = (3 * cp + 3) / 4 * 4, ls = (cp + 3) / 4 * 4;
+    const Mat* D[3] = {&R.tDr, &R.tDs, &R.tDt};
     real* to = reinterpret_cast<real*>(blob.data() + L.tops);
-    for (int l = 0; l < np; ++l)
-      for (int i = 0; i < np; ++i) {
-        real* v = to + (size_t(l) * np + i) * 4;
-        v[0] = real(R.tDr(i, l));
-        v[1] = real(R.tDs(i, l));
-        v[2] = real(R.tDt(i, l));
-        v[3] = real(0);
-      }
-    real* lt = to + size_t(4) * np * np;
+    real* lt = to + size_t(4) * np * rs;
     for (int w = 0; w < 4; ++w)
-      for (int fk = 0; fk < 4 * nt; ++fk)
-        for (int cc = 0; cc < cp; ++cc) {
-          const int i = w * ch + cc;
-          lt[(size_t(w) * 4 * nt + fk) * cp + cc] = (cc < ch && i < np) ? real(R.tLIFT(i, fk)) : real(0);
-        }
+      for (int cc = 0; cc < ch; ++cc) {
+        const int i = w * ch + cc;
+        if (i >= np) continue;
+        for (int l = 0; l < np; ++l)
+          for (int m = 0; m < 3; ++m) to[(size_t(w) * np + l) * rs + m * cp + cc] = real((*D[m])(i, l));
+        for (int fk = 0; fk < 4 * nt; ++fk) lt[(size_t(w) * 4 * nt + fk) * ls + cc] = real(R.tLIFT(i, fk));
+      }
   }
   real* wo = reinterpret_cast<real*>(blob.data() + L.wops);
   const int nt2 = c->ref->Nt * c->ref->Nt;

@@ -1870,12 +1870,16 @@ __global__ void __launch_bounds__(32 * (N + 1), wedge_min_ctas<N, 1, OP>())
 
 // ---------------------------------------------------------------------------
 // tet stage: one 32-tet block per CTA (lane = tet), 4 warps.  Bulk copies move
-// the tet operators ([l][i] (D_r, D_s, D_t)(i, l) records and the lift, laid
-// out per warp chunk), the block's vertex coordinates and its state slab into
-// shared memory.  Every warp evaluates the affine geometry of the 32 tets;
-// warp f forms the fluxes of face f into a shared table; warp w then forms
-// the volume terms of output nodes [w C, w C + C) and, after one barrier,
-// their lift and update.
+// the tet operators (laid out per warp chunk by output pairs), the block's
+// vertex coordinates and its state slab into shared memory.  Warp f forms the
+// normal and the fluxes of face f; warp w forms the volume terms, the lift and
+// the update of output nodes [w C, w C + C).  Bound by instruction issue (and
+// by the FP64 pipe in FP64), so what the four warps would repeat is done once:
+// each face's normal, and (p, -w) with w the reference-direction velocities of
+// every node, which the volume terms read (tet_wtab): 2,380 -> 1,919
+// instructions per warp at N = 3.  us per stage: 221,184 tets N = 3 FP32 92.3 ->
+// 88.1, 41,472 tets N = 4 45.2 -> 41.4 and N = 5 171 -> 99; 27,648 tets N = 3 FP64
+// 184 -> 150.
 // All warps run the same code.
 // ---------------------------------------------------------------------------
 template <int N>
@@ -1883,57 +1887,79 @@ __host__ __device__ constexpr int tet_chunk() {  // output nodes per warp
   return (npt_of(N) + 3) / 4;
 }
 template <int N>
-__host__ __device__ constexpr int tet_chunk_pad() {  // lift record length per face node (multiple of 4)
-  return (tet_chunk<N>() + 3) / 4 * 4;
+__host__ __device__ constexpr int tet_pairs() {  // output pairs per warp
+  return (tet_chunk<N>() + 1) / 2;
+}
+template <int N>
+__host__ __device__ constexpr int tet_rec() {  // reals of a (warp, l) record: D_r, D_s, D_t pairs (a multiple of 4)
+  return (6 * tet_pairs<N>() + 3) / 4 * 4;
+}
+template <int N>
+__host__ __device__ constexpr int tet_lrec() {  // reals of a (warp, face node) lift record (a multiple of 4)
+  return (2 * tet_pairs<N>() + 3) / 4 * 4;
+}
+template <int N>
+__host__ __device__ constexpr int tet_drecs() {  // reals of all derivative records
+  return 4 * npt_of(N) * tet_rec<N>();
 }
 template <int N>
 __host__ __device__ constexpr int tet_ops_image_reals() {  // the global image t_ops: D records, then the lift
-  return 4 * npt_of(N) * npt_of(N) + 4 * (4 * nt_of(N)) * tet_chunk_pad<N>();
+  return tet_drecs<N>() + 4 * (4 * nt_of(N)) * tet_lrec<N>();
+}
+// The table of (p, -w): N <= 3, where it costs no CTA per SM.  In FP32 the
+// residual slab is bulk-copied into its place once the volume terms are done
+// (elsewhere the update reads the residual from global memory).
+template <int N>
+__host__ __device__ constexpr bool tet_wtab() {
+  return N <= 3;
+}
+template <int N>
+__host__ __device__ constexpr bool tet_stage_res() {
+  return sizeof(real) == 4 && tet_wtab<N>();
 }
 // Whether the lift rows are copied to shared memory with the derivative
 // records: everywhere but FP64 at N = 5, where the whole image would exceed a
 // CTA's shared memory; there the warps read their lift rows (uniform
 // addresses) from global memory.
 template <int N>
+__host__ __device__ constexpr int tet_work_reals() {  // slab, flux pairs, coordinates, normals, (p, -w) table
+  return 4 * npt_of(N) * kB + 8 * nt_of(N) * kB + 24 * kB + (tet_wtab<N>() ? 4 * npt_of(N) * kB : 0);
+}
+template <int N>
 __host__ __device__ constexpr bool tet_lift_smem() {
-  return 128 + (tet_ops_image_reals<N>() + 4 * npt_of(N) * kB + 8 * nt_of(N) * kB + 12 * kB +
-                ((sizeof(real) == 4 && N <= 3) ? 4 * npt_of(N) * kB : 0)) * int(sizeof(real)) <= 227 * 1024;
+  return 128 + (tet_ops_image_reals<N>() + tet_work_reals<N>()) * int(sizeof(real)) <= 227 * 1024;
 }
 template <int N>
 __host__ __device__ constexpr int tet_ops_reals() {  // the part of the image in shared memory
-  return tet_lift_smem<N>() ? tet_ops_image_reals<N>() : 4 * npt_of(N) * npt_of(N);
+  return tet_lift_smem<N>() ? tet_ops_image_reals<N>() : tet_drecs<N>();
 }
-// The residual slab is bulk-copied too where it costs no CTA per SM (FP32,
-// N <= 3); elsewhere the update reads it from global memory.
-template <int N>
-__host__ __device__ constexpr bool tet_stage_res() {
-  return sizeof(real) == 4 && N <= 3;
-}
-// 128-byte header (4 mbarriers), operators, slab [Np][32][4], fluxes
-// [4 faces][2][Nt][32], vertex coordinates [12][32], residual slab [Np][32][4]
-template <int N>
-__host__ __device__ constexpr int tet_smem_reals() {
-  return tet_ops_reals<N>() + 4 * npt_of(N) * kB + 8 * nt_of(N) * kB + 12 * kB +
-         (tet_stage_res<N>() ? 4 * npt_of(N) * kB : 0);
-}
+// 128-byte header (4 mbarriers), operators, slab [Np][32][4], flux pairs
+// [4 faces][Nt][32][2], vertex coordinates [12][32], normals [4][3][32], (p, -w) [Np][32][4]
 template <int N>
 __host__ __device__ constexpr int tet_smem_bytes() {
-  return 128 + tet_smem_reals<N>() * int(sizeof(real));
+  return 128 + (tet_ops_reals<N>() + tet_work_reals<N>()) * int(sizeof(real));
+}
+// acc.x += a.x b, acc.y += a.y b; FP64 leaves out the second where it is padding
+template <bool PAD>
+__device__ __forceinline__ real2 fma_pair(const real2 a, real b, const real2 acc) {
+  if constexpr (sizeof(real) == 8 && PAD) return mk2(fmar(a.x, b, acc.x), acc.y);
+  else return fma2(a, dup2(b), acc);
 }
 
 template <int N>
 __global__ void __launch_bounds__(128, (sizeof(REAL) == 4) ? (N >= 4 ? 3 : 5) : 2)
     k_tet_stage(const StageArgs<real> A, bool rk) {
-  constexpr int Np = npt_of(N), Nt = nt_of(N), C = tet_chunk<N>(), CP = tet_chunk_pad<N>();
+  constexpr int Np = npt_of(N), Nt = nt_of(N), C = tet_chunk<N>(), CH = tet_pairs<N>(), RS = tet_rec<N>(), LS = tet_lrec<N>();
   const AllOps<N, real>& O = OPS<N>();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);  // [0] operators, [1] coordinates, [2] state, [3] residual
   real* sOp = reinterpret_cast<real*>(smem_raw + 128);
-  real* sL = sOp + 4 * Np * Np;  // lift [warp][4 Nt][CP]
+  real* sL = sOp + tet_drecs<N>();  // lift [warp][4 Nt][LS]
   real* sq = sOp + tet_ops_reals<N>();
   real* sF = sq + 4 * Np * kB;
   real* sX = sF + 8 * Nt * kB;
-  real* sr = sX + 12 * kB;  // residual slab (tet_stage_res)
+  real* sN = sX + 12 * kB;
+  real* sW = sN + 12 * kB;  // (p, -w), then the residual slab
   constexpr bool stage_res = tet_stage_res<N>();
   const bool res_async = stage_res && rk && A.rk_a != real(0);
   const DevMesh<real>& M = A.m;
@@ -1956,222 +1982,224 @@ __global__ void __launch_bounds__(128, (sizeof(REAL) == 4) ? (N >= 4 ? 3 : 5) : 
     bulk_g2s(sq, A.q_in + M.tet_off + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[2]);
     mbar_expect_tx(&bar[0], ops_bytes);
     bulk_g2s(sOp, M.t_ops, ops_bytes, &bar[0]);
-    if (res_async) {
-      mbar_expect_tx(&bar[3], slab_bytes);
-      bulk_g2s(sr, A.res + M.tet_off + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[3]);
-    }
   }
   // face neighbours, impedances, material and the source flag while the copies fly
   const real kappa = M.t_mat[0 * Kp + e], irho = M.t_mat[1 * Kp + e], zM = M.t_mat[2 * Kp + e];
-  int nbr = M.t_nbr[w * Kp + e], code = M.t_code[w * Kp + e];  // this warp's face w
+  const int nbr = M.t_nbr[w * Kp + e], code = M.t_code[w * Kp + e];  // this warp's face w
   const real zP = nbr < 0 ? zM : ((code & kCodeTet) ? M.t_mat[2 * Kp + nbr] : M.w_mat[2 * M.Kw_pad + nbr]);
   const bool src = M.nsrc > 0 && has_source(M, 4, e);
   // out-of-block neighbour face nodes of this warp's face, requested before the waits
   Q4 nvs[Nt];
-  const bool t_bnd = nbr < 0;
-  const bool t_ntet = !t_bnd && (code & kCodeTet) != 0;
-  const int t_nbe = t_bnd ? e : nbr;
-  const bool t_inblk = t_bnd || (t_ntet && (t_nbe >> 5) == blk);
-  if (!t_inblk) {
-    const int nfc = (code >> 4) & 3, perm = code & 15;
-    const real* nb = A.q_in + (t_ntet ? tidx<N>(M.tet_off, t_nbe >> 5, 0, t_nbe & 31) : widx<N>(t_nbe >> 5, 0, t_nbe & 31));
+  const bool bnd = nbr < 0;
+  const bool ntet = !bnd && (code & kCodeTet) != 0;
+  const int nbe = bnd ? e : nbr;
+  const bool inblk = bnd || (ntet && (nbe >> 5) == blk);
+  const int nfc = (code >> 4) & 3, perm = code & 15;
+  if (!inblk) {
+    const real* nb = A.q_in + (ntet ? tidx<N>(M.tet_off, nbe >> 5, 0, nbe & 31) : widx<N>(nbe >> 5, 0, nbe & 31));
 #pragma unroll
     for (int k = 0; k < Nt; ++k) {
       const int nk = O.tab.tri_perm[perm][k];
-      nvs[k] = ldg4(nb, int64_t(t_ntet ? O.tab.tet_face[nfc][nk] : (nfc ? N * Nt : 0) + nk) * (kB * 4));
+      nvs[k] = ldg4(nb, int64_t(ntet ? O.tab.tet_face[nfc][nk] : (nfc ? N * Nt : 0) + nk) * (kB * 4));
     }
   }
   __syncthreads();  // the mbarriers are initialised
 
   // affine geometry: x = sum_v lambda_v X_v on the bi-unit reference tet
   bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[1], 0));
-  real Ri[3][3], nf[4][3], sJ[4];  // d r_m / d x_d, outward unit normals, J_f / J
+  real nR[3][3], n0, n1, n2, sj;  // -d r_m / d x_d; this warp's face: outward unit normal, J_f / J
   {
-    real X[4][3];
-#pragma unroll
-    for (int v = 0; v < 4; ++v)
-#pragma unroll
-      for (int d = 0; d < 3; ++d) X[v][d] = sX[(v * 3 + d) * kB + lane];
+    auto X = [&](int v, int d) { return sX[(v * 3 + d) * kB + lane]; };
     real G[3][3];  // G[d][m] = d x_d / d r_m
 #pragma unroll
-    for (int d = 0; d < 3; ++d)
+    for (int d = 0; d < 3; ++d) {
+      const real xd = X(0, d);
 #pragma unroll
-      for (int m = 0; m < 3; ++m) G[d][m] = real(0.5) * (X[m + 1][d] - X[0][d]);
+      for (int m = 0; m < 3; ++m) G[d][m] = real(0.5) * (X(m + 1, d) - xd);
+    }
     const real J = G[0][0] * (G[1][1] * G[2][2] - G[1][2] * G[2][1]) -
                    G[0][1] * (G[1][0] * G[2][2] - G[1][2] * G[2][0]) + G[0][2] * (G[1][0] * G[2][1] - G[1][1] * G[2][0]);
-    const real iJ = real(1) / J;
-    Ri[0][0] = (G[1][1] * G[2][2] - G[1][2] * G[2][1]) * iJ;
-    Ri[0][1] = (G[0][2] * G[2][1] - G[0][1] * G[2][2]) * iJ;
-    Ri[0][2] = (G[0][1] * G[1][2] - G[0][2] * G[1][1]) * iJ;
-    Ri[1][0] = (G[1][2] * G[2][0] - G[1][0] * G[2][2]) * iJ;
-    Ri[1][1] = (G[0][0] * G[2][2] - G[0][2] * G[2][0]) * iJ;
-    Ri[1][2] = (G[0][2] * G[1][0] - G[0][0] * G[1][2]) * iJ;
-    Ri[2][0] = (G[1][0] * G[2][1] - G[1][1] * G[2][0]) * iJ;
-    Ri[2][1] = (G[0][1] * G[2][0] - G[0][0] * G[2][1]) * iJ;
-    Ri[2][2] = (G[0][0] * G[1][1] - G[0][1] * G[1][0]) * iJ;
-    constexpr int fv[4][3] = {{0, 1, 2}, {0, 1, 3}, {1, 2, 3}, {0, 2, 3}};
-    constexpr int fo[4] = {3, 2, 0, 1};
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      const real ax = X[fv[f][1]][0] - X[fv[f][0]][0], ay = X[fv[f][1]][1] - X[fv[f][0]][1],
-                 az = X[fv[f][1]][2] - X[fv[f][0]][2];
-      const real bx = X[fv[f][2]][0] - X[fv[f][0]][0], by = X[fv[f][2]][1] - X[fv[f][0]][1],
-                 bz = X[fv[f][2]][2] - X[fv[f][0]][2];
-      const real cx = ay * bz - az * by, cy = az * bx - ax * bz, cz = ax * by - ay * bx;
-      const real cc = cx * cx + cy * cy + cz * cz, ic = rsqrt_r(cc);
-      const real ox = X[fo[f]][0] - X[fv[f][0]][0], oy = X[fo[f]][1] - X[fv[f][0]][1], oz = X[fo[f]][2] - X[fv[f][0]][2];
-      const real sgn = (cx * ox + cy * oy + cz * oz > 0) ? real(-1) : real(1);  // away from the opposite vertex
-      nf[f][0] = sgn * cx * ic;
-      nf[f][1] = sgn * cy * ic;
-      nf[f][2] = sgn * cz * ic;
-      sJ[f] = real(0.25) * cc * ic * iJ;
-    }
+    const real iJ = real(1) / J, niJ = -iJ;
+    nR[0][0] = (G[1][1] * G[2][2] - G[1][2] * G[2][1]) * niJ;
+    nR[0][1] = (G[0][2] * G[2][1] - G[0][1] * G[2][2]) * niJ;
+    nR[0][2] = (G[0][1] * G[1][2] - G[0][2] * G[1][1]) * niJ;
+    nR[1][0] = (G[1][2] * G[2][0] - G[1][0] * G[2][2]) * niJ;
+    nR[1][1] = (G[0][0] * G[2][2] - G[0][2] * G[2][0]) * niJ;
+    nR[1][2] = (G[0][2] * G[1][0] - G[0][0] * G[1][2]) * niJ;
+    nR[2][0] = (G[1][0] * G[2][1] - G[1][1] * G[2][0]) * niJ;
+    nR[2][1] = (G[0][1] * G[2][0] - G[0][0] * G[2][1]) * niJ;
+    nR[2][2] = (G[0][0] * G[1][1] - G[0][1] * G[1][0]) * niJ;
+    // face w: vertices {0,1,2}, {0,1,3}, {1,2,3}, {0,2,3}, opposite 3, 2, 0, 1
+    const int a0 = w == 2 ? 1 : 0, a1 = w < 2 ? 1 : 2, a2 = w == 0 ? 2 : 3, ao = (0x1023 >> (4 * w)) & 3;
+    const real px = X(a0, 0), py = X(a0, 1), pz = X(a0, 2);
+    const real ax = X(a1, 0) - px, ay = X(a1, 1) - py, az = X(a1, 2) - pz;
+    const real bx = X(a2, 0) - px, by = X(a2, 1) - py, bz = X(a2, 2) - pz;
+    const real cx = ay * bz - az * by, cy = az * bx - ax * bz, cz = ax * by - ay * bx;
+    const real cc = cx * cx + cy * cy + cz * cz, ic = rsqrt_r(cc);
+    const real ox = X(ao, 0) - px, oy = X(ao, 1) - py, oz = X(ao, 2) - pz;
+    const real sc = (cx * ox + cy * oy + cz * oz > 0) ? -ic : ic;  // away from the opposite vertex
+    n0 = sc * cx;
+    n1 = sc * cy;
+    n2 = sc * cz;
+    sj = real(0.25) * cc * ic * iJ;
+    sN[(w * 3 + 0) * kB + lane] = n0;
+    sN[(w * 3 + 1) * kB + lane] = n1;
+    sN[(w * 3 + 2) * kB + lane] = n2;
   }
-  ok = ok && __all_sync(0xffffffffu, mbar_wait_bounded(&bar[2], 0));
-  if (!ok) {
-    // a copy never arrived: report, let the copies in flight drain, leave
-    if (threadIdx.x == 0) atomicOr(M.err, kErrTimeout);
-    if (lane == 0) {
-      mbar_wait_bounded(&bar[0], 0);
-      mbar_wait_bounded(&bar[1], 0);
-      mbar_wait_bounded(&bar[2], 0);
-      if (res_async) mbar_wait_bounded(&bar[3], 0);
-    }
-    return;
-  }
+  ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[2], 0)) && ok;
 
   // fluxes of face w, scaled by J_f / J, into the shared flux table
   {
-    const int f = w;
-    real n0 = nf[0][0], n1 = nf[0][1], n2 = nf[0][2], sj = sJ[0];
-#pragma unroll
-    for (int g = 1; g < 4; ++g)
-      if (f == g) {
-        n0 = nf[g][0];
-        n1 = nf[g][1];
-        n2 = nf[g][2];
-        sj = sJ[g];
-      }
-    real tau_p, tau_u;
-    taus(A.flux, zM, zP, tau_p, tau_u);
-    const bool bnd = nbr < 0;
-    const bool ntet = !bnd && (code & kCodeTet) != 0;
-    const int nfc = (code >> 4) & 3, perm = code & 15;
-    const int nbe = bnd ? e : nbr;
-    const bool inblk = bnd || (ntet && (nbe >> 5) == blk);
-    // the neighbour's face nodes, all requested at once: this block's own slab
-    // (shared loads), or another tet block's or a wedge block's in global memory
+    real tp, tu;
+    taus(A.flux, zM, zP, tp, tu);
+    const real2 s = ghost_signs(bnd, A.bc);
+    const real hs = real(0.5) * sj;
+    // the neighbour's face nodes in this block's own slab (a boundary face reads its own)
     if (inblk) {
 #pragma unroll
       for (int k = 0; k < Nt; ++k) {
         const int nk = bnd ? k : O.tab.tri_perm[perm][k];
-        nvs[k] = lds4(sq, bnd ? O.tab.tet_face[f][k] : O.tab.tet_face[nfc][nk], nbe & 31);
+        nvs[k] = lds4(sq, bnd ? O.tab.tet_face[w][k] : O.tab.tet_face[nfc][nk], nbe & 31);
       }
     }
 #pragma unroll
     for (int k = 0; k < Nt; ++k) {
-      const int own = O.tab.tet_face[f][k];
-      const Q4 o = lds4(sq, own, lane);
-      const real unM = n0 * o.u + n1 * o.v + n2 * o.w;
-      const Q4 nv = nvs[k];
-      real bdp, bdun;
-      boundary_jumps(A.bc, o.p, unM, bdp, bdun);
-      const real dp = bnd ? bdp : nv.p - o.p;
-      const real dun = bnd ? bdun : n0 * nv.u + n1 * nv.v + n2 * nv.w - unM;
-      real Fp, Fu;
-      penalty_flux(dp, dun, tau_p, tau_u, Fp, Fu);
-      sF[((f * 2 + 0) * Nt + k) * kB + lane] = sj * Fp;
-      sF[((f * 2 + 1) * Nt + k) * kB + lane] = sj * Fu;
+      const Q4 o = lds4(sq, O.tab.tet_face[w][k], lane);
+      const real2 F = mul2(tri_node_flux(o, nvs[k], n0, n1, n2, s, -tp, -tu), dup2(hs));
+      *reinterpret_cast<real2*>(sF + ((w * Nt + k) * kB + lane) * 2) = F;
     }
   }
-  if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bar[0], 0)) && lane == 0) atomicOr(M.err, kErrTimeout);
-
-  // output nodes [I0, I0 + C) of this warp: volume terms (the slab and the
-  // operators only), then, once every warp's face fluxes are in the table,
-  // the lift and the update
-  const int I0 = w * C;
-  // results of the warp's outputs by output pairs (c, c + 1): ap2 the pressure,
-  // au2[d] the velocity components (packed multiply-adds)
-  constexpr int CH = (C + 1) / 2;
-  real2 ap2[CH], au2[3][CH];
-  {
-    // per output: (D_r p, D_s p) and D_t p; (D_r w_r + D_t w_t, D_s w_s) with
-    // w = the reference-direction velocity components
-    real2 drs[C], sab[C];
-    real dt[C];
+  const int I0 = w * C;  // this warp's output nodes
+  if constexpr (tet_wtab<N>()) {
+    // (p, -w) of this warp's nodes, w_m = sum_d (d r_m / d x_d) u_d
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-      drs[c] = sab[c] = dup2(real(0));
-      dt[c] = real(0);
+      if (I0 + c < Np) {
+        const Q4 v = lds4(sq, I0 + c, lane);
+        st4(sW, ((I0 + c) * kB + lane) * 4,
+            Q4{v.p, fmar(nR[0][0], v.u, fmar(nR[0][1], v.v, nR[0][2] * v.w)),
+               fmar(nR[1][0], v.u, fmar(nR[1][1], v.v, nR[1][2] * v.w)),
+               fmar(nR[2][0], v.u, fmar(nR[2][1], v.v, nR[2][2] * v.w))});
+      }
     }
-    const real* opI = sOp + I0 * 4;  // records (l, I0 + c) at opI + (l Np + c) 4
+  }
+  ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[0], 0)) && ok;
+  if (!__syncthreads_and(ok)) {
+    // a copy never arrived: report, let the copies in flight drain, leave
+    if (threadIdx.x == 0) {
+      atomicOr(M.err, kErrTimeout);
+      mbar_wait_bounded(&bar[0], 0);
+      mbar_wait_bounded(&bar[1], 0);
+      mbar_wait_bounded(&bar[2], 0);
+    }
+    return;
+  }
+
+  // results of the warp's outputs by pairs (c, c + 1): ap the pressure, au[d]
+  // the velocity components; first the volume terms
+  constexpr bool odd = (C & 1) != 0;  // the last pair's second row is padding
+  real2 ap[CH], au[3][CH];
+  {
+    real2 dr[CH], ds[CH], dt[CH];
+#pragma unroll
+    for (int h = 0; h < CH; ++h) ap[h] = dr[h] = ds[h] = dt[h] = dup2(real(0));
+    const real* rec = sOp + w * Np * RS;
 #pragma unroll 4
     for (int l = 0; l < Np; ++l) {
-      const Q4 v = lds4(sq, l, lane);
-      const real wr = Ri[0][0] * v.u + Ri[0][1] * v.v + Ri[0][2] * v.w;
-      const real ws = Ri[1][0] * v.u + Ri[1][1] * v.v + Ri[1][2] * v.w;
-      const real wt = Ri[2][0] * v.u + Ri[2][1] * v.v + Ri[2][2] * v.w;
-      const real2 pp = dup2(v.p), wrs = mk2(wr, ws);
+      Q4 v;
+      if constexpr (tet_wtab<N>()) {
+        v = lds4(sW, l, lane);
+      } else {
+        const Q4 u = lds4(sq, l, lane);
+        v = Q4{u.p, fmar(nR[0][0], u.u, fmar(nR[0][1], u.v, nR[0][2] * u.w)),
+               fmar(nR[1][0], u.u, fmar(nR[1][1], u.v, nR[1][2] * u.w)),
+               fmar(nR[2][0], u.u, fmar(nR[2][1], u.v, nR[2][2] * u.w))};
+      }
+      real d[RS];
 #pragma unroll
-      for (int c = 0; c < C; ++c) {
-        const Q4 d = ldop4(opI + (l * Np + c) * 4);  // I0 + c >= Np: unused records, results dropped
-        const real2 dpu = mk2(d.p, d.u);
-        drs[c] = fma2(dpu, pp, drs[c]);
-        dt[c] += d.v * v.p;
-        sab[c] = fma2(dpu, wrs, sab[c]);
-        sab[c].x += d.v * wt;
+      for (int c4 = 0; c4 < RS; c4 += 4) {
+        const Q4 t = ldop4(rec + l * RS + c4);
+        d[c4] = t.p;
+        d[c4 + 1] = t.u;
+        d[c4 + 2] = t.v;
+        d[c4 + 3] = t.w;
+      }
+#pragma unroll
+      for (int h = 0; h < CH; ++h) {
+        const real2 r2 = mk2(d[2 * h], d[2 * h + 1]), s2 = mk2(d[2 * (CH + h)], d[2 * (CH + h) + 1]),
+                    t2 = mk2(d[2 * (2 * CH + h)], d[2 * (2 * CH + h) + 1]);
+        if (odd && h == CH - 1) {
+          dr[h] = fma_pair<true>(r2, v.p, dr[h]);
+          ds[h] = fma_pair<true>(s2, v.p, ds[h]);
+          dt[h] = fma_pair<true>(t2, v.p, dt[h]);
+          ap[h] = fma_pair<true>(t2, v.w, fma_pair<true>(s2, v.v, fma_pair<true>(r2, v.u, ap[h])));
+        } else {
+          dr[h] = fma_pair<false>(r2, v.p, dr[h]);
+          ds[h] = fma_pair<false>(s2, v.p, ds[h]);
+          dt[h] = fma_pair<false>(t2, v.p, dt[h]);
+          ap[h] = fma_pair<false>(t2, v.w, fma_pair<false>(s2, v.v, fma_pair<false>(r2, v.u, ap[h])));
+        }
       }
     }
 #pragma unroll
-    for (int h = 0; h < CH; ++h) {
-      const int c0 = 2 * h, c1 = 2 * h + 1 < C ? 2 * h + 1 : 2 * h;
-      ap2[h] = mk2(-(sab[c0].x + sab[c0].y), -(sab[c1].x + sab[c1].y));
+    for (int d = 0; d < 3; ++d)
 #pragma unroll
-      for (int d = 0; d < 3; ++d)
-        au2[d][h] = mk2(-(Ri[0][d] * drs[c0].x + Ri[1][d] * drs[c0].y + Ri[2][d] * dt[c0]),
-                        -(Ri[0][d] * drs[c1].x + Ri[1][d] * drs[c1].y + Ri[2][d] * dt[c1]));
+      for (int h = 0; h < CH; ++h)
+        au[d][h] = fma2(dup2(nR[0][d]), dr[h], fma2(dup2(nR[1][d]), ds[h], mul2(dup2(nR[2][d]), dt[h])));
+  }
+  if (res_async) {
+    // every warp is done with the (p, -w) table: the residual slab may land in its place
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      mbar_expect_tx(&bar[3], slab_bytes);
+      bulk_g2s(sW, A.res + M.tet_off + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[3]);
     }
   }
-  __syncthreads();
+  // the lift of the four faces: this warp's records [4 Nt][LS] (shared memory, or the global image)
   {
-    // this warp's lift records [4 Nt][CP] (shared memory, or the global image)
-    const real* lw = (tet_lift_smem<N>() ? sL : M.t_ops + 4 * Np * Np) + w * (4 * Nt) * CP;
+    const real* lw = (tet_lift_smem<N>() ? sL : M.t_ops + tet_drecs<N>()) + w * (4 * Nt) * LS;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      real2 lu2[CH];
+      real2 lu[CH];
 #pragma unroll
-      for (int h = 0; h < CH; ++h) lu2[h] = dup2(real(0));
+      for (int h = 0; h < CH; ++h) lu[h] = dup2(real(0));
 #pragma unroll 5
       for (int k = 0; k < Nt; ++k) {
-        const real2 fp2 = dup2(sF[((f * 2 + 0) * Nt + k) * kB + lane]);
-        const real2 fu2 = dup2(sF[((f * 2 + 1) * Nt + k) * kB + lane]);
+        const real2 F = *reinterpret_cast<const real2*>(sF + ((f * Nt + k) * kB + lane) * 2);
+        real d[LS];
 #pragma unroll
-        for (int c4 = 0; c4 < CP; c4 += 4) {
-          const Q4 L = ldop4(lw + (f * Nt + k) * CP + c4);
-          const real2 La = mk2(L.p, L.u), Lb = mk2(L.v, L.w);
-          const int h = c4 / 2;
-          if (h < CH) {
-            ap2[h] = fma2(La, fp2, ap2[h]);
-            lu2[h] = fma2(La, fu2, lu2[h]);
-          }
-          if (h + 1 < CH) {
-            ap2[h + 1] = fma2(Lb, fp2, ap2[h + 1]);
-            lu2[h + 1] = fma2(Lb, fu2, lu2[h + 1]);
+        for (int c4 = 0; c4 < LS; c4 += 4) {
+          const Q4 t = ldop4(lw + (f * Nt + k) * LS + c4);
+          d[c4] = t.p;
+          d[c4 + 1] = t.u;
+          d[c4 + 2] = t.v;
+          d[c4 + 3] = t.w;
+        }
+#pragma unroll
+        for (int h = 0; h < CH; ++h) {
+          const real2 L = mk2(d[2 * h], d[2 * h + 1]);
+          if (odd && h == CH - 1) {
+            ap[h] = fma_pair<true>(L, F.x, ap[h]);
+            lu[h] = fma_pair<true>(L, F.y, lu[h]);
+          } else {
+            ap[h] = fma_pair<false>(L, F.x, ap[h]);
+            lu[h] = fma_pair<false>(L, F.y, lu[h]);
           }
         }
       }
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        const real2 n2 = dup2(nf[f][d]);
+        const real2 nd = dup2(sN[(f * 3 + d) * kB + lane]);
 #pragma unroll
-        for (int h = 0; h < CH; ++h) au2[d][h] = fma2(n2, lu2[h], au2[d][h]);
+        for (int h = 0; h < CH; ++h) au[d][h] = fma2(nd, lu[h], au[d][h]);
       }
     }
   }
-  real ap[C];
+  real p[C];
 #pragma unroll
-  for (int c = 0; c < C; ++c) ap[c] = pair_row(ap2, c);
-  if (src) add_sources(M, 4, e, I0, Np, *M.clock + A.c_stage * double(A.dt), ap);
+  for (int c = 0; c < C; ++c) p[c] = pair_row(ap, c);
+  if (src) add_sources(M, 4, e, I0, Np, *M.clock + A.c_stage * double(A.dt), p);
   if (res_async && !__all_sync(0xffffffffu, mbar_wait_bounded(&bar[3], 0))) {
     // the residual slab never arrived: report, let the copy drain, leave
     if (lane == 0) {
@@ -2181,31 +2209,15 @@ __global__ void __launch_bounds__(128, (sizeof(REAL) == 4) ? (N >= 4 ? 3 : 5) : 
     return;
   }
   if (e < M.Kt) {
+    const UpdateCoef U(A, kappa, irho);
 #pragma unroll
     for (int c = 0; c < C; ++c) {
       if (I0 + c < Np) {
         const int i = I0 + c;
-        const int64_t gi = tidx<N>(M.tet_off, blk, i, lane);
-        const real2 r01 = mul2(mk2(ap[c], pair_row(au2[0], c)), mk2(kappa, irho));
-        const real2 r23 = mul2(mk2(pair_row(au2[1], c), pair_row(au2[2], c)), dup2(irho));
-        const Q4 r{r01.x, r01.y, r23.x, r23.y};
-        if (rk) {
-          // res = a res + dt r, q = g q + b res, on packed pairs
-          // (the residual read where a != 0, stored where a later stage reads it)
-          Q4 r0{0, 0, 0, 0};
-          if (A.rk_a != real(0)) r0 = stage_res ? lds4(sr, i, lane) : ld4(A.res, gi);
-          const real2 a2 = dup2(A.rk_a), dt2 = dup2(A.dt), g2 = dup2(A.rk_g), b2 = dup2(A.rk_b);
-          const real2 rr01 = fma2(a2, mk2(r0.p, r0.u), mul2(dt2, r01));
-          const real2 rr23 = fma2(a2, mk2(r0.v, r0.w), mul2(dt2, r23));
-          const Q4 q0 = lds4(sq, i, lane);
-          const real2 q01 = fma2(g2, mk2(q0.p, q0.u), mul2(b2, rr01));
-          const real2 q23 = fma2(g2, mk2(q0.v, q0.w), mul2(b2, rr23));
-          if (A.res_store) st4(A.res, gi, Q4{rr01.x, rr01.y, rr23.x, rr23.y});
-          st4(A.q_out, gi, Q4{q01.x, q01.y, q23.x, q23.y});
-          if (A.rhs_out) st4(A.rhs_out, gi, r);
-        } else {
-          st4(A.q_out, gi, r);
-        }
+        const int64_t g = tidx<N>(M.tet_off, blk, i, lane);
+        Q4 r0{0, 0, 0, 0};
+        if (rk && A.rk_a != real(0)) r0 = stage_res ? lds4(sW, i, lane) : ld4(A.res, g);
+        U.node(A, rk, g, mk2(p[c], pair_row(au[0], c)), mk2(pair_row(au[1], c), pair_row(au[2], c)), r0, lds4(sq, i, lane));
       }
     }
   }
