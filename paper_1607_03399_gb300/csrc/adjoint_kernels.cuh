@@ -156,8 +156,11 @@ __global__ void __launch_bounds__(32 * (N + 1), (sizeof(real) == 4) ? (N <= 3 ? 
     }
     return;
   }
+  // (by one warp: split over the warps it measured no faster, with more spills)
+  if (j == 0) {
 #pragma unroll 1
-  for (int p = j; p < kGeoParts; p += Nq) wedge_geometry_part<true>(p, sC, sG, lane);
+    for (int p = 0; p < kGeoParts; ++p) wedge_geometry_part<true>(p, sC, sG, lane);
+  }
   __syncthreads();
 #define GEO(item) sG[(item) * kB + lane]
   const real J0 = GEO(G_J0), J1 = GEO(G_J1), J2 = GEO(G_J2);

@@ -256,6 +256,18 @@ void fill_ops(const RefElems& R, std::vector<unsigned char>& out) {
     o.w.ellN[m] = real(R.ellN[m]);
     o.w.gll[m] = real(R.gll[m]);
   }
+  // structural zeros of D_r (rows of the edge b = 0) and D_s (rows of the edge a = 0) exactly: a form
+  // of the stage that leaves them out and one that does not give the same bits
+  for (int i = 0; i < Nt; ++i)
+    for (int l = 0; l < Nt; ++l) {
+      auto on = [&](int e, int n) {
+        for (int m = 0; m < Nq; ++m)
+          if (R.edge_nodes[e][m] == n) return true;
+        return false;
+      };
+      if (on(0, i) && !on(0, l)) o.w.Dr[i * Nt + l] = real(0);
+      if (on(2, i) && !on(2, l)) o.w.Ds[i * Nt + l] = real(0);
+    }
   // output-pair copies (rows 2h and 2h + 1; zero past the last row)
   auto pairs = [](const real* X, int rows, int cols, real* XP) {
     for (int h = 0; h < (rows + 1) / 2; ++h)
@@ -268,6 +280,17 @@ void fill_ops(const RefElems& R, std::vector<unsigned char>& out) {
   pairs(o.w.Mea, Nq, Nq, o.w.MeaP);
   pairs(o.w.Meb, Nq, Nq, o.w.MebP);
   for (int a = 0; a < 3; ++a) pairs(o.w.Ma[a], Nt, Nt, o.w.MaP[a]);
+  if (NN >= 4) {
+    using W = WedgeOps<NN, real>;
+    auto by_input = [&](const real* XP, real* XT) {
+      for (int l = 0; l < Nt; ++l)
+        for (int h = 0; h < W::Nh; ++h)
+          for (int b = 0; b < 2; ++b) XT[(l * W::Nhp + h) * 2 + b] = XP[(h * Nt + l) * 2 + b];
+    };
+    by_input(o.w.MP, o.w.MT);
+    by_input(o.w.DrP, o.w.DrT);
+    by_input(o.w.DsP, o.w.DsT);
+  }
   for (int c = 0; c < 9; ++c)
     for (int k = 0; k < Nt; ++k) o.tab.tri_perm[c][k] = R.tri_perm[c].empty() ? 0 : int8_t(R.tri_perm[c][k]);
   for (int e = 0; e < 3; ++e)

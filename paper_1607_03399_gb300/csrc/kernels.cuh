@@ -633,9 +633,8 @@ __device__ __forceinline__ void mass_solve(const real* sL, int lane, real2 (&W01
       }
     }
   };
-  real d[Nt];
 #pragma unroll
-  for (int i = 0; i < Nt; ++i) {
+  for (int i = 1; i < Nt; ++i) {
     real Lr[Nt];
     load_row(i, Lr);
 #pragma unroll
@@ -644,12 +643,13 @@ __device__ __forceinline__ void mass_solve(const real* sL, int lane, real2 (&W01
       W01[i] = fma2(nl, W01[k], W01[i]);
       W23[i] = fma2(nl, W23[k], W23[i]);
     }
-    d[i] = Lr[i];
   }
 #pragma unroll
   for (int i = 0; i < Nt; ++i) {
-    W01[i] = mul2(W01[i], dup2(d[i]));
-    W23[i] = mul2(W23[i], dup2(d[i]));
+    // (read again: held from the sweep, the diagonal would cost Nt registers)
+    const real2 d = dup2(sL[((i * (i + 3) / 2 >> 2) * kB + lane) * 4 + (i * (i + 3) / 2 & 3)]);
+    W01[i] = mul2(W01[i], d);
+    W23[i] = mul2(W23[i], d);
   }
 #pragma unroll
   for (int i = Nt - 1; i > 0; --i) {
@@ -737,24 +737,29 @@ __device__ __forceinline__ void wedge_update(const StageArgs<real>& A, bool rk, 
 // into one constant, so a lane with its own code extracts its node with a
 // shift and a mask instead of an indexed constant load (which is replayed for
 // every distinct index of the warp).
-template <int N>
-struct EdgeCandidates {
-  uint32_t c[N + 1];
-  __host__ __device__ constexpr EdgeCandidates() : c{} {
-    for (int m = 0; m <= N; ++m)
-      for (int code = 0; code < 6; ++code)
-        c[m] |= uint32_t(edge_node(N, code >> 1, (code & 1) ? N - m : m)) << (5 * code);
-  }
-};
+// (closed forms and masks throughout, so that they fold to constants in the
+// unrolled loops at every order)
+__host__ __device__ constexpr uint32_t edge_candidates(int N, int m) {
+  return uint32_t(edge_node(N, 0, m)) | uint32_t(edge_node(N, 0, N - m)) << 5 | uint32_t(edge_node(N, 1, m)) << 10 |
+         uint32_t(edge_node(N, 1, N - m)) << 15 | uint32_t(edge_node(N, 2, m)) << 20 | uint32_t(edge_node(N, 2, N - m)) << 25;
+}
 // D_r restricted to the edge b = 0 (rows a = 0..N) differentiates along the
 // edge: only its own N + 1 nodes enter; D_s likewise on the edge a = 0.
 __host__ __device__ constexpr bool dr_zero(int N, int i, int l) { return i <= N && l > N; }
-__host__ __device__ constexpr bool on_edge_a0(int N, int i) {
-  for (int b = 0; b <= N; ++b)
-    if (tri_idx(N, 0, b) == i) return true;
-  return false;
+template <int N>
+struct EdgeA0 {
+  static constexpr uint32_t nodes() {
+    uint32_t m = 0;
+    for (int b = 0; b <= N; ++b) m |= 1u << tri_idx(N, 0, b);
+    return m;
+  }
+  static constexpr uint32_t mask = nodes();
+};
+template <int N>
+__host__ __device__ constexpr bool ds_zero(int i, int l) {
+  constexpr uint32_t m = EdgeA0<N>::mask;
+  return ((m >> i) & 1u) != 0 && ((m >> l) & 1u) == 0;
 }
-__host__ __device__ constexpr bool ds_zero(int N, int i, int l) { return on_edge_a0(N, i) && !on_edge_a0(N, l); }
 // acc += {X[2h][l], X[2h + 1][l]} * x, leaving out rows known to be zero
 // (FP32: the pair is one instruction and is left out when both rows are zero)
 template <int NT>
@@ -826,9 +831,9 @@ __device__ __forceinline__ void quad_edge(const AllOps<N, real>& O, const real* 
 // choice between two address spaces), and a boundary face reads its own trace.
 // Bound by memory latency and traffic at N <= 3 (a copy of the slabs and the
 // traces alone takes 218 us of the 240 at N = 3), by issue and registers at
-// N >= 4.  Warp instructions per warp, N = 3: 2,769 -> 2,140.  us per stage of
-// a step on 524,288 wedges, with the skipped residual traffic and the prefetch:
-// N = 3 298 -> 240, N = 4 769 -> 670; 30,118 wedges N = 5 326 -> 230.
+// N >= 4.  Instructions per warp, N = 3: 2,769 -> 2,240.  us per stage of a step
+// on 524,288 wedges, with the skipped residual traffic and the prefetch: N = 3
+// 298 -> 239, N = 4 769 -> 578; 30,118 wedges N = 5 326 -> 125.
 // TF: the neighbour nodes of the triangle-face fluxes come from global memory
 // and are requested before the slab arrives (meshes where some of them are
 // tets or lie in another block, StageArgs::tri_far; two blocks per CTA:
@@ -837,6 +842,14 @@ template <int N, int BPC, bool TF>
 __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOpFFMA>())
     k_wedge_stage(const StageArgs<real> A, bool rk) {
   constexpr int Nt = nt_of(N), Nq = N + 1, Np = Nt * Nq, NH = (Nt + 1) / 2, NQH = (Nq + 1) / 2;
+  // FP32 at N >= 4: the operator products as loops over the input nodes (tables
+  // by input node; three nodes unrolled, one, two or five measured slower)
+  // instead of straight-line code, which missed the instruction cache and, at
+  // N = 5, half of its constant loads: N = 4 622 -> 600 us per stage on 524,288
+  // wedges, N = 5 613 -> 438 us on 131,072.  (FP64 waits on its pipe and gains
+  // more from leaving out the zeros of D_s: N = 4 1,295 against 1,360 us.)
+  constexpr bool rolled = sizeof(real) == 4 && N >= 4;
+  constexpr int NHP = (NH + 1) / 2 * 2;
   using SM = WedgeSmem<N, kOpFFMA>;
   const AllOps<N, real>& O = OPS<N>();
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -890,6 +903,9 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
     if (res_async) {
       mbar_expect_tx(&bar[1], slab_bytes);
       bulk_g2s(sr, A.res + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[1]);
+    } else if (rk && A.rk_a != real(0)) {
+      // not staged: to L2 at least, for the update (N = 5: 438 -> 411 us per stage on 131,072 wedges)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(A.res + int64_t(blk) * 4 * Np * kB), "r"(slab_bytes));
     }
   }
   if (j == N) prefetch_ahead<N>(M, qin, blk + 76 * wedge_min_ctas<N, BPC, kOpFFMA>() * BPC, lane, N <= 4 && stored);
@@ -908,13 +924,15 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
   auto trace = [&](int ed, Q4 (&t)[Nq]) {
     const bool bnd = qnbr[ed] < 0;
     const int nbe = bnd ? e : qnbr[ed], sh = 5 * (bnd ? 2 * ed : qcode[ed]);
-    constexpr EdgeCandidates<N> cand;
     const real* nb = qin + widx<N>(nbe >> 5, j * Nt, nbe & 31);
 #pragma unroll
-    for (int m = 0; m < Nq; ++m) t[m] = ldg4(nb, int((cand.c[m] >> sh) & 31u) * (kB * 4));
+    for (int m = 0; m < Nq; ++m) t[m] = ldg4(nb, int((edge_candidates(N, m) >> sh) & 31u) * (kB * 4));
   };
-  constexpr bool early = N <= 3;
-  Q4 nv[early ? 3 : 1][Nq];
+  // requested here at N <= 3, after the slab has arrived at N = 4 (before it they
+  // cost spills: 649 against 578 us per stage on 524,288 wedges, 600 face by
+  // face), face by face at N = 5
+  constexpr bool early = N <= 3, mid = N == 4;
+  Q4 nv[early || mid ? 3 : 1][Nq];
   if constexpr (early) {
 #pragma unroll
     for (int ed = 0; ed < 3; ++ed) trace(ed, nv[ed]);
@@ -979,6 +997,10 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
     return;
   }
 
+  if constexpr (mid) {
+#pragma unroll
+    for (int ed = 0; ed < 3; ++ed) trace(ed, nv[ed]);
+  }
   // 1. triangle-face node fluxes (bottom then top), spread round-robin over
   //    the warps, without the factor 1/2 (it enters with the lift)
   {
@@ -1012,11 +1034,22 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
 #pragma unroll 1
   for (int v = j; v < 4; v += Nq) {
     real* f = sF + ((v >> 1) * Nt * kB + lane) * 2 + (v & 1);
-    real G[Nt];
-#pragma unroll
-    for (int i = 0; i < Nt; ++i) G[i] = f[i * kB * 2];
     real2 acc[NH];
-    apply_pairs<Nt, Nt>(O.w.MP, G, acc);
+    if constexpr (rolled) {
+#pragma unroll
+      for (int h = 0; h < NH; ++h) acc[h] = dup2(real(0));
+#pragma unroll 3
+      for (int l = 0; l < Nt; ++l) {
+        const real2 xx = dup2(f[l * kB * 2]);
+#pragma unroll
+        for (int h = 0; h < NH; ++h) acc[h] = fma2(cpair(O.w.MT, NHP, l, h), xx, acc[h]);
+      }
+    } else {
+      real G[Nt];
+#pragma unroll
+      for (int i = 0; i < Nt; ++i) G[i] = f[i * kB * 2];
+      apply_pairs<Nt, Nt>(O.w.MP, G, acc);
+    }
 #pragma unroll
     for (int i = 0; i < Nt; ++i) f[i * kB * 2] = pair_row(acc, i);
   }
@@ -1029,7 +1062,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
 #pragma unroll
   for (int ed = 0; ed < 3; ++ed) {
     Q4 tv[Nq];
-    if constexpr (early) {
+    if constexpr (early || mid) {
 #pragma unroll
       for (int m = 0; m < Nq; ++m) tv[m] = nv[ed][m];
     } else {
@@ -1056,13 +1089,11 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
   const real ntx = -fmar(tj, GEO(G_TX1), GEO(G_TX0)), nty = -fmar(tj, GEO(G_TY1), GEO(G_TY0)), nA = -GEO(G_A);
   real2 Mdp[NH];
   {
-    real dp[Nt], dd[Nt];
     real dtr[Nq];
 #pragma unroll
     for (int m = 0; m < Nq; ++m) dtr[m] = O.w.Dt[j * Nq + m];
-#pragma unroll
-    for (int i = 0; i < Nt; ++i) {
-      // D_t of the four fields as two packed pairs (p, u_x) and (u_y, u_z)
+    // node i: D_t of the four fields as two packed pairs (p, u_x) and (u_y, u_z)
+    auto t_part = [&](int i, real& dp, real& dd) {
       real2 dpu = dup2(real(0)), dvw = dup2(real(0));
 #pragma unroll
       for (int m = 0; m < Nq; ++m) {
@@ -1071,16 +1102,37 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
         dpu = fma2(d2, mk2(v.p, v.u), dpu);
         dvw = fma2(d2, mk2(v.v, v.w), dvw);
       }
-      dp[i] = dpu.x;
-      dd[i] = fmar(ntx, dpu.y, fmar(nty, dvw.x, nA * dvw.y));
-    }
+      dp = dpu.x;
+      dd = fmar(ntx, dpu.y, fmar(nty, dvw.x, nA * dvw.y));
+    };
+    if constexpr (rolled) {
+      // a node's two values go into both products at once
 #pragma unroll
-    for (int l = 0; l < Nt; ++l) {
-      const real2 xx = dup2(dd[l]);
+      for (int h = 0; h < NH; ++h) Mdp[h] = dup2(real(0));
+#pragma unroll 3
+      for (int l = 0; l < Nt; ++l) {
+        real dp, dd;
+        t_part(l, dp, dd);
+        const real2 xx = dup2(dd), pp = dup2(dp);
 #pragma unroll
-      for (int h = 0; h < NH; ++h) Wp[h] = fma2(cpair(O.w.MP, Nt, h, l), xx, Wp[h]);
+        for (int h = 0; h < NH; ++h) {
+          const real2 c = cpair(O.w.MT, NHP, l, h);
+          Wp[h] = fma2(c, xx, Wp[h]);
+          Mdp[h] = fma2(c, pp, Mdp[h]);
+        }
+      }
+    } else {
+      real dp[Nt], dd[Nt];
+#pragma unroll
+      for (int i = 0; i < Nt; ++i) t_part(i, dp[i], dd[i]);
+#pragma unroll
+      for (int l = 0; l < Nt; ++l) {
+        const real2 xx = dup2(dd[l]);
+#pragma unroll
+        for (int h = 0; h < NH; ++h) Wp[h] = fma2(cpair(O.w.MP, Nt, h, l), xx, Wp[h]);
+      }
+      apply_pairs<Nt, Nt>(O.w.MP, dp, Mdp);
     }
-    apply_pairs<Nt, Nt>(O.w.MP, dp, Mdp);
   }
   block_sync();  // M^tri has been applied to the flux vectors
 
@@ -1119,24 +1171,61 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
     real2 dv[NH], pr[NH], ps[NH];
 #pragma unroll
     for (int h = 0; h < NH; ++h) dv[h] = pr[h] = ps[h] = dup2(real(0));
+    if constexpr (rolled) {
+      // nodes of the edge b = 0, then the others, for which the first pairs of
+      // D_r's rows are zero
+      constexpr int H0 = (N + 1) / 2;
+#pragma unroll 3
+      for (int l = 0; l <= N; ++l) {
+        const Q4 v = lds4(sq, j * Nt + l, lane);
+        const real2 ab = fma2(dup2(v.u), mk2(rx, sx), mul2(dup2(v.v), mk2(ry, sy)));
+        const real2 a = dup2(ab.x), b = dup2(ab.y), p = dup2(v.p);
 #pragma unroll
-    for (int l = 0; l < Nt; ++l) {
-      const Q4 v = lds4(sq, j * Nt + l, lane);
-      const real2 ab = fma2(dup2(v.u), mk2(rx, sx), mul2(dup2(v.v), mk2(ry, sy)));
+        for (int h = 0; h < NH; ++h) {
+          const real2 r = cpair(O.w.DrT, NHP, l, h), q = cpair(O.w.DsT, NHP, l, h);
+          dv[h] = fma2(q, b, fma2(r, a, dv[h]));
+          pr[h] = fma2(r, p, pr[h]);
+          ps[h] = fma2(q, p, ps[h]);
+        }
+      }
+#pragma unroll 3
+      for (int l = N + 1; l < Nt; ++l) {
+        const Q4 v = lds4(sq, j * Nt + l, lane);
+        const real2 ab = fma2(dup2(v.u), mk2(rx, sx), mul2(dup2(v.v), mk2(ry, sy)));
+        const real2 a = dup2(ab.x), b = dup2(ab.y), p = dup2(v.p);
 #pragma unroll
-      for (int h = 0; h < NH; ++h) {
-        const bool r0 = dr_zero(N, 2 * h, l), r1 = dr_zero(N, 2 * h + 1, l);
-        const bool s0 = ds_zero(N, 2 * h, l), s1 = ds_zero(N, 2 * h + 1, l);
-        dv[h] = fma_rows<Nt>(O.w.DrP, h, l, ab.x, dv[h], r0, r1);
-        dv[h] = fma_rows<Nt>(O.w.DsP, h, l, ab.y, dv[h], s0, s1);
-        pr[h] = fma_rows<Nt>(O.w.DrP, h, l, v.p, pr[h], r0, r1);
-        ps[h] = fma_rows<Nt>(O.w.DsP, h, l, v.p, ps[h], s0, s1);
+        for (int h = 0; h < NH; ++h) {
+          const real2 q = cpair(O.w.DsT, NHP, l, h);
+          if (h >= H0) {
+            const real2 r = cpair(O.w.DrT, NHP, l, h);
+            dv[h] = fma2(r, a, dv[h]);
+            pr[h] = fma2(r, p, pr[h]);
+          }
+          dv[h] = fma2(q, b, dv[h]);
+          ps[h] = fma2(q, p, ps[h]);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int l = 0; l < Nt; ++l) {
+        const Q4 v = lds4(sq, j * Nt + l, lane);
+        const real2 ab = fma2(dup2(v.u), mk2(rx, sx), mul2(dup2(v.v), mk2(ry, sy)));
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+          const bool r0 = dr_zero(N, 2 * h, l), r1 = dr_zero(N, 2 * h + 1, l);
+          const bool s0 = ds_zero<N>(2 * h, l), s1 = ds_zero<N>(2 * h + 1, l);
+          dv[h] = fma_rows<Nt>(O.w.DrP, h, l, ab.x, dv[h], r0, r1);
+          dv[h] = fma_rows<Nt>(O.w.DsP, h, l, ab.y, dv[h], s0, s1);
+          pr[h] = fma_rows<Nt>(O.w.DrP, h, l, v.p, pr[h], r0, r1);
+          ps[h] = fma_rows<Nt>(O.w.DsP, h, l, v.p, ps[h], s0, s1);
+        }
       }
     }
 #pragma unroll
+    for (int i = 0; i < Nt; ++i) W01[i].x -= pair_row(dv, i);
+#pragma unroll
     for (int i = 0; i < Nt; ++i) {
       const real pri = pair_row(pr, i), psi = pair_row(ps, i);
-      W01[i].x -= pair_row(dv, i);
       W01[i].y = fmar(-rx, pri, fmar(-sx, psi, W01[i].y));
       W23[i].x = fmar(-ry, pri, fmar(-sy, psi, W23[i].x));
     }
@@ -1195,7 +1284,7 @@ __device__ __forceinline__ void div_rows(const AllOps<N, real>& O, const real* s
 #pragma unroll
     for (int h = H0; h < H1; ++h) {
       dv[h - H0] = fma_rows<Nt>(O.w.DrP, h, l, ab.x, dv[h - H0], dr_zero(N, 2 * h, l), dr_zero(N, 2 * h + 1, l));
-      dv[h - H0] = fma_rows<Nt>(O.w.DsP, h, l, ab.y, dv[h - H0], ds_zero(N, 2 * h, l), ds_zero(N, 2 * h + 1, l));
+      dv[h - H0] = fma_rows<Nt>(O.w.DsP, h, l, ab.y, dv[h - H0], ds_zero<N>(2 * h, l), ds_zero<N>(2 * h + 1, l));
     }
   }
 }
@@ -1251,10 +1340,9 @@ __global__ void __launch_bounds__(128) k_wedge_wide(const StageArgs<real> A, boo
   {
     const bool bnd = qnbr < 0;
     const int nbe = bnd ? e : qnbr, sh = 5 * (bnd ? 2 * ed : qcode);
-    constexpr EdgeCandidates<N> cand;
     const real* nb = qin + widx<N>(nbe >> 5, j * Nt, nbe & 31);
 #pragma unroll
-    for (int m = 0; m < Nq; ++m) tv[m] = ldg4(nb, int((cand.c[m] >> sh) & 31u) * (kB * 4));
+    for (int m = 0; m < Nq; ++m) tv[m] = ldg4(nb, int((edge_candidates(N, m) >> sh) & 31u) * (kB * 4));
   }
   constexpr int NTT = (2 * Nt + 3) / 4;
   Q4 tnv[NTT];
@@ -1475,7 +1563,7 @@ __global__ void __launch_bounds__(128) k_wedge_wide(const StageArgs<real> A, boo
         const real p = sq[((j * Nt + l) * kB + lane) * 4];
 #pragma unroll
         for (int h = 0; h < NH; ++h)
-          pd[h] = fma_rows<Nt>(O.w.DsP, h, l, p, pd[h], ds_zero(N, 2 * h, l), ds_zero(N, 2 * h + 1, l));
+          pd[h] = fma_rows<Nt>(O.w.DsP, h, l, p, pd[h], ds_zero<N>(2 * h, l), ds_zero<N>(2 * h + 1, l));
       }
     }
     real* out = sD + ((f == 1 ? 1 : 2) * Nt) * kB + lane;
