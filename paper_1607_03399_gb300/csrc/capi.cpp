@@ -54,8 +54,8 @@ int pack_f64(int N, const DevMesh<double>& m, const double* c, double* p, bool u
   DGW_SWITCH_N(N, launch_pack_f64, (m, c, p, u, s))
 }
 int energy_f32(int N, const DevMesh<float>& m, const float* q, void* s) { DGW_SWITCH_N(N, launch_energy_f32, (m, q, s)) }
-int clock_f32(int N, double* c, double dt, void* s) { DGW_SWITCH_N(N, launch_clock_f32, (c, dt, s)) }
-int clock_f64(int N, double* c, double dt, void* s) { DGW_SWITCH_N(N, launch_clock_f64, (c, dt, s)) }
+int clock_f32(int N, const double* c, double* o, double dt, void* s) { DGW_SWITCH_N(N, launch_clock_f32, (c, o, dt, s)) }
+int clock_f64(int N, const double* c, double* o, double dt, void* s) { DGW_SWITCH_N(N, launch_clock_f64, (c, o, dt, s)) }
 int set_clock_f32(int N, double* c, double t, void* s) { DGW_SWITCH_N(N, launch_set_clock_f32, (c, t, s)) }
 int set_clock_f64(int N, double* c, double t, void* s) { DGW_SWITCH_N(N, launch_set_clock_f64, (c, t, s)) }
 int wait_expire_f32(int N, int* e, void* s) { DGW_SWITCH_N(N, launch_wait_expire_f32, (e, s)) }
@@ -187,6 +187,9 @@ struct dg_ctx {
   // joined back into the launching stream by these events
   cudaStream_t tet_stream = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  // the branch of the step graph that advances the clock (capture only)
+  cudaStream_t clk_stream = nullptr;
+  cudaEvent_t ev_cfork = nullptr, ev_cjoin = nullptr;
   void* d_mesh = nullptr;
   void* d_q[2] = {nullptr, nullptr};
   void* d_res = nullptr;
@@ -469,7 +472,7 @@ BlobLayout blob_layout(const dg_ctx* c) {
   size_t ng = 0;
   for (const auto& sc : c->sources) ng += sc.g.size();
   L.srcg = take((ng > 0 ? ng : 1) * rs);
-  L.clock = take(sizeof(double));
+  L.clock = take(2 * sizeof(double));
   // stored mass factors: per wedge block [NL4][32][4], the stage's shared-memory layout
   const int64_t nl4 = nl4_of(c->N);
   L.wfac = take(c->mass == DG_MASS_STORED ? size_t(Kwp * nl4 * 4) * rs : 0);
@@ -698,14 +701,13 @@ void fill_blob(const dg_ctx* c, const BlobLayout& L, std::vector<unsigned char>&
           Lk[size_t(i) * nt + l] = (l < i) ? sum / Lk[size_t(l) * nt + l] : std::sqrt(sum);
         }
       }
-      for (int i = 0; i < nt; ++i)
-        for (int l = 0; l <= i; ++l)
-        {
-          // M = L L^T = (L S^-1) S^2 (L S^-1)^T with S = diag(L): the negated
-          // unit lower triangle and 1 / S_i^2, as the stage's sweeps use them
-          const double lii = Lk[size_t(i) * nt + i];
-          one[size_t(w) * nl + i * (i + 1) / 2 + l] = real(l < i ? -Lk[size_t(i) * nt + l] / Lk[size_t(l) * nt + l] : 1.0 / (lii * lii));
-        }
+      // M = L L^T = (L S^-1) S^2 (L S^-1)^T with S = diag(L): the negated unit
+      // lower triangle and 1 / S_i^2, as the stage's sweeps use them
+      for (int l = 0; l < nt; ++l) {
+        const double inv = 1.0 / Lk[size_t(l) * nt + l];
+        one[size_t(w) * nl + l * (l + 3) / 2] = real(inv * inv);
+        for (int i = l + 1; i < nt; ++i) one[size_t(w) * nl + i * (i + 1) / 2 + l] = real(-Lk[size_t(i) * nt + l] * inv);
+      }
     }
     const int64_t nl4 = nl4_of(c->N);
     for (int64_t w = 0; w < Kwp; ++w) {
@@ -790,7 +792,11 @@ struct StageExtra {
   void* rhs_out = nullptr;
   bool no_sources = false;
   bool res_store = true;
+  bool pdl = false;     // the stage before it on the stream is the only work it waits for
 };
+
+// the slot of the device clock that holds the current time: it moves with the state buffer
+double* clock_of(const dg_ctx* c) { return ((c->prec == DG_F64) ? c->m64.clock : c->m32.clock) + c->cur; }
 
 int launch_stage(dg_ctx* c, const void* q_in, void* q_out, void* res, double a, double b, double dt, bool rk,
                  cudaStream_t s, double cst = 0.0, const StageExtra& x = StageExtra()) {
@@ -812,6 +818,8 @@ int launch_stage(dg_ctx* c, const void* q_in, void* q_out, void* res, double a, 
     A.tri_far = c->tri_far ? 1 : 0;
     A.rk_g = x.g;
     A.res_store = x.res_store ? 1 : 0;
+    A.clk = c->cur;
+    A.pdl = x.pdl ? 1 : 0;
     A.rhs_out = static_cast<double*>(x.rhs_out);
     if (x.no_sources) A.m.nsrc = 0;
     rc = stage_f64(c->N, A, rk, s, c->tet_stream, c->ev_fork, c->ev_join);
@@ -834,6 +842,8 @@ int launch_stage(dg_ctx* c, const void* q_in, void* q_out, void* res, double a, 
     A.tri_far = c->tri_far ? 1 : 0;
     A.rk_g = float(x.g);
     A.res_store = x.res_store ? 1 : 0;
+    A.clk = c->cur;
+    A.pdl = x.pdl ? 1 : 0;
     A.rhs_out = static_cast<float*>(x.rhs_out);
     if (x.no_sources) A.m.nsrc = 0;
     rc = stage_f32(c->N, A, rk, s, c->tet_stream, c->ev_fork, c->ev_join);
@@ -1447,6 +1457,9 @@ int dg_bind(dg_ctx* c, void* d_mesh, void* d_q0, void* d_q1, void* d_res, void* 
   const int rc = ensure_ops(c);
   if (rc) return rc;
   e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->clk_stream, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_cfork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_cjoin, cudaEventDisableTiming);
   if (e != cudaSuccess) return cuda_fail(c, e, "capture stream");
   if (vKw(c) > 0 && vKt(c) > 0) {
     e = cudaStreamCreateWithFlags(&c->tet_stream, cudaStreamNonBlocking);
@@ -1497,9 +1510,8 @@ int dg_set_fields(dg_ctx* c, const void* q, int on_device) {
   }
   rc = launch_pack(c, src, c->d_q[c->cur], false, c->stream);
   if (rc) return rc;
-  cudaError_t e = cudaMemsetAsync(c->d_res, 0, c->field_bytes, c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "residual clear");
-  e = cudaMemsetAsync((c->prec == DG_F64) ? c->m64.clock : c->m32.clock, 0, sizeof(double), c->stream);
+  // (the residual needs no clearing: a step's first stage, a = 0, does not read it)
+  cudaError_t e = cudaMemsetAsync(clock_of(c), 0, sizeof(double), c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "clock reset");
   if (!on_device) {
     e = cudaStreamSynchronize(c->stream);
@@ -1547,9 +1559,6 @@ int dg_rhs(dg_ctx* c, const void* d_q, void* d_rhs) {
   if (rc) return rc;
   rc = launch_pack(c, d_rhs, B, true, c->stream);
   if (rc) return rc;
-  // the residual buffer was used as scratch; the next step starts from zero
-  cudaError_t e = cudaMemsetAsync(c->d_res, 0, c->field_bytes, c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "residual clear");
   return DG_OK;
 }
 
@@ -1573,17 +1582,32 @@ int dg_step(dg_ctx* c, double dt, int64_t nsteps) {
       if (e != cudaSuccess) return cuda_fail(c, e, "graph capture begin");
       int src = p;
       int lrc = DG_OK;
+      // the time of the next step into the other slot, on a branch of its own
+      // beside the stages, which read this step's slot
+      e = cudaEventRecord(c->ev_cfork, c->cap_stream);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(c->clk_stream, c->ev_cfork, 0);
+      if (e != cudaSuccess) lrc = cuda_fail(c, e, "clock fork");
+      if (lrc == DG_OK) {
+        double* other = clock_of(c) + (c->cur ? -1 : 1);
+        const int crc = (c->prec == DG_F64) ? clock_f64(c->N, clock_of(c), other, dt, c->clk_stream)
+                                            : clock_f32(c->N, clock_of(c), other, dt, c->clk_stream);
+        if (crc) lrc = cuda_fail(c, cudaError_t(crc), "clock launch");
+      }
+      if (lrc == DG_OK) {
+        e = cudaEventRecord(c->ev_cjoin, c->clk_stream);
+        if (e != cudaSuccess) lrc = cuda_fail(c, e, "clock fork");
+      }
       for (int s = 0; s < 5 && lrc == DG_OK; ++s) {
         StageExtra x;
         x.res_store = s < 4;  // the next step's first stage (a = 0) reads no residual
+        x.pdl = true;
         lrc = launch_stage(c, c->d_q[src], c->d_q[1 - src], c->d_res, kLSRK_A[s], kLSRK_B[s], dt, true, c->cap_stream,
                            kLSRK_C[s], x);
         src = 1 - src;
       }
       if (lrc == DG_OK) {
-        double* clk = (c->prec == DG_F64) ? c->m64.clock : c->m32.clock;
-        const int crc = (c->prec == DG_F64) ? clock_f64(c->N, clk, dt, c->cap_stream) : clock_f32(c->N, clk, dt, c->cap_stream);
-        if (crc) lrc = cuda_fail(c, cudaError_t(crc), "clock launch");
+        e = cudaStreamWaitEvent(c->cap_stream, c->ev_cjoin, 0);
+        if (e != cudaSuccess) lrc = cuda_fail(c, e, "clock join");
       }
       e = cudaStreamEndCapture(c->cap_stream, &g);
       if (lrc) {
@@ -1850,8 +1874,8 @@ int dg_load_state(dg_ctx* c, const void* d_src, double t) {
   if (e != cudaSuccess) return cuda_fail(c, e, "state load");
   c->t = t;
   // the clock by a one-thread kernel on the stream: the call stays asynchronous
-  const int rc = c->prec == DG_F64 ? set_clock_f64(c->N, c->m64.clock, t, c->stream)
-                                   : set_clock_f32(c->N, c->m32.clock, t, c->stream);
+  const int rc = c->prec == DG_F64 ? set_clock_f64(c->N, clock_of(c), t, c->stream)
+                                   : set_clock_f32(c->N, clock_of(c), t, c->stream);
   if (rc) return cuda_fail(c, cudaError_t(rc), "clock set");
   return DG_OK;
 }
@@ -2015,7 +2039,7 @@ int dg_step_record_chain(dg_ctx* c, double dt, int64_t nsteps, void* const* d_re
   // the same launches as captured steps, one state copy per chain
   cudaError_t e = cudaMemcpyAsync(d_recs[0], c->d_q[c->cur], fb, cudaMemcpyDeviceToDevice, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "record copy");
-  double* clk = (c->prec == DG_F64) ? c->m64.clock : c->m32.clock;
+  double* clk = clock_of(c);
   for (int64_t i = 0; i < nsteps; ++i) {
     unsigned char* rec = static_cast<unsigned char*>(d_recs[i]);
     for (int st = 0; st < 5 && rc == DG_OK; ++st) {
@@ -2028,7 +2052,7 @@ int dg_step_record_chain(dg_ctx* c, double dt, int64_t nsteps, void* const* d_re
                         kLSRK_C[st], x);
     }
     if (rc) return rc;
-    const int crc = (c->prec == DG_F64) ? clock_f64(c->N, clk, dt, c->stream) : clock_f32(c->N, clk, dt, c->stream);
+    const int crc = (c->prec == DG_F64) ? clock_f64(c->N, clk, clk, dt, c->stream) : clock_f32(c->N, clk, clk, dt, c->stream);
     if (crc) return cuda_fail(c, cudaError_t(crc), "clock launch");
     c->t += dt;
   }
@@ -2256,6 +2280,9 @@ void dg_destroy(dg_ctx* c) {
   drop_graphs(c);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->tet_stream) cudaStreamDestroy(c->tet_stream);
+  if (c->clk_stream) cudaStreamDestroy(c->clk_stream);
+  if (c->ev_cfork) cudaEventDestroy(c->ev_cfork);
+  if (c->ev_cjoin) cudaEventDestroy(c->ev_cjoin);
   if (c->grad_stream) cudaStreamDestroy(c->grad_stream);
   if (c->ev_gfork) cudaEventDestroy(c->ev_gfork);
   if (c->ev_gjoin) cudaEventDestroy(c->ev_gjoin);

@@ -132,7 +132,7 @@ struct DevMesh {
   const SourceDev* src = nullptr;    // point sources
   const real* src_g = nullptr;       // their vectors g
   int nsrc = 0;
-  double* clock = nullptr;           // simulation time of the current step
+  double* clock = nullptr;           // simulation time, two slots: StageArgs::clk holds the current step's
   const real* w_fac = nullptr;       // stored mass factors per wedge block, or null (factor in the stage)
   const real* w_xyz = nullptr;       // per wedge block [12][32]: bottom x, y; bottom and top z
   const real* t_xyz = nullptr;       // per tet block [12][32]: x, y, z of the four vertices
@@ -159,9 +159,11 @@ struct StageArgs {
   real rk_g = 1;                // RK: q_out = rk_g q_in + rk_b res' (1 in the forward method)
   int res_store = 1;            // RK: store the residual (0: no later stage reads it)
   real* rhs_out = nullptr;      // RK: also store the stage right-hand side here (optional)
-  double c_stage = 0;           // stage time = *clock + c_stage * dt
+  double c_stage = 0;           // stage time = clock[clk] + c_stage * dt
+  int clk = 0;                  // slot of the step's time
+  int pdl = 0;                  // launch as a programmatic dependent of the stage before it
   int bc = 1, flux = 0;
-  int wedge_bpc = 0;            // wedge blocks per CTA: 0 = the default for the mass mode
+  int wedge_bpc = 0;            // wedge blocks per CTA: 0 = one, unless a launch variant asks for two
   int op = 0;                   // kOpFFMA, or a tensor-core variant (FP32 fields)
   int split = 0;                // wedge stage split over field pairs: 1 yes, otherwise no
   int tri_far = 0;              // some wedge's triangle-face neighbour is a tet or in another block
@@ -197,7 +199,7 @@ __host__ __device__ constexpr int tile_at(int r, int c) { return r * kTP + (c ^ 
                              void* ev_join);                                                       \
   int launch_pack_##P##n##N(const DevMesh<T>& m, const T* canon, T* packed, bool unpack, void* s); \
   int launch_energy_##P##n##N(const DevMesh<T>& m, const T* q, void* stream);                      \
-  int launch_clock_##P##n##N(double* clock, double dt, void* stream);                              \
+  int launch_clock_##P##n##N(const double* from, double* to, double dt, void* stream);             \
   int launch_wait_expire_##P##n##N(int* err, void* stream);                                        \
   int launch_set_clock_##P##n##N(double* clock, double t, void* stream);                           \
   int launch_sample_##P##n##N(const DevMesh<T>& m, const T* q, T* out, int nshots, void* stream);     \

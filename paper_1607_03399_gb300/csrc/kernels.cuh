@@ -383,8 +383,17 @@ __device__ __forceinline__ void add_sources(const DevMesh<real>& M, int type, in
   }
 }
 
-__global__ void k_clock(double* clock, double dt) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) *clock += dt;
+// Programmatic dependent launch (StageArgs::pdl): the stage after this one may
+// be scheduled now; what it does before its own pdl_wait reads mesh tables
+// only.  pdl_wait returns when the stage before this one has completed and its
+// writes are visible (at once in an ordinary launch).
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// advances the time: a step's stages read one slot of the device clock, the
+// next step's the other, so in a captured step this runs beside the stages
+__global__ void k_clock(const double* from, double* to, double dt) {
+  if (threadIdx.x == 0 && blockIdx.x == 0) *to = *from + dt;
 }
 // sets the device clock (state loads: no host staging, so no synchronisation)
 __global__ void k_set_clock(double* clock, double t) {
@@ -494,13 +503,13 @@ template <int N, int OP = kOpFFMA>
 __host__ __device__ constexpr int wedge_smem_reals() {
   return WedgeSmem<N, OP>::reals;
 }
-// Element blocks per CTA.  The warps that work on slice j of the CTA's blocks
-// share an SM sub-partition and run the same straight-line code side by side,
-// so they share its instruction cache lines.  With the mass factor computed in
-// the stage (a long serial factorisation on one warp per block) two blocks per
-// CTA measured faster at N = 3 FP32; with the stored factor, one.
+// Element blocks per CTA of the launch variant with several (a candidate of
+// dg_autotune): the warps that work on slice j of the CTA's blocks share an SM
+// sub-partition and run the same straight-line code side by side.  One block
+// is the default in both mass modes (factor formed in the stage, N = 3,
+// 524,288 wedges: 304 us against 401 us with two).
 template <int N>
-__host__ __device__ constexpr int wedge_bpc_onthefly() {
+__host__ __device__ constexpr int wedge_bpc_multi() {
   return (sizeof(real) == 4 && N == 3) ? 2 : 1;
 }
 // bytes: per block two mbarriers and a status word (32 bytes), then per block
@@ -589,24 +598,54 @@ __device__ __forceinline__ void factor_wedge(const AllOps<N, real>& O, const Dev
   const real x0 = M.vx[v0], y0 = M.vy[v0];
   const real Ah = real(0.125) * ((M.vx[v1] - x0) * (M.vy[v2] - y0) - (M.vx[v2] - x0) * (M.vy[v1] - y0));
   const real J0 = Ah * (M.vz[v3] - M.vz[v0]), J1 = Ah * (M.vz[v4] - M.vz[v1]), J2 = Ah * (M.vz[v5] - M.vz[v2]);
+  auto mass = [&](int i, int l) {
+    return J0 * O.w.Ma[0][i * Nt + l] + J1 * O.w.Ma[1][i * Nt + l] + J2 * O.w.Ma[2][i * Nt + l];
+  };
+  if constexpr (Nt <= 10) {
+    // the whole factor in registers (its latency is what the block waits for), then four entries per store
+    constexpr int NL4 = nl4_of(N);
+    real F[NL4 * 4];
 #pragma unroll
-  for (int i = 0; i < Nt; ++i) {
-    real row[Nt];  // l_il D_l
+    for (int q = Nt * (Nt + 1) / 2; q < NL4 * 4; ++q) F[q] = real(0);
 #pragma unroll
-    for (int l = 0; l < i; ++l) {
-      real s = J0 * O.w.Ma[0][i * Nt + l] + J1 * O.w.Ma[1][i * Nt + l] + J2 * O.w.Ma[2][i * Nt + l];
+    for (int i = 0; i < Nt; ++i) {
+      real row[Nt];  // l_il D_l
 #pragma unroll
-      for (int k = 0; k < l; ++k) s += row[k] * LQ(l * (l + 1) / 2 + k);
-      row[l] = s;
+      for (int l = 0; l < i; ++l) {
+        row[l] = mass(i, l);
+#pragma unroll
+        for (int k = 0; k < l; ++k) row[l] += row[k] * F[l * (l + 1) / 2 + k];
+      }
+      real d = mass(i, i);
+#pragma unroll
+      for (int k = 0; k < i; ++k) {
+        const real nl = -(row[k] * F[k * (k + 1) / 2 + k]);
+        d += row[k] * nl;
+        F[i * (i + 1) / 2 + k] = nl;
+      }
+      F[i * (i + 1) / 2 + i] = real(1) / d;
     }
-    real d = J0 * O.w.Ma[0][i * Nt + i] + J1 * O.w.Ma[1][i * Nt + i] + J2 * O.w.Ma[2][i * Nt + i];
 #pragma unroll
-    for (int k = 0; k < i; ++k) {
-      const real nl = -(row[k] * LQ(k * (k + 1) / 2 + k));
-      d += row[k] * nl;
-      LQ(i * (i + 1) / 2 + k) = nl;
+    for (int c = 0; c < NL4; ++c) st4(sL, (c * kB + lane) * 4, Q4{F[c * 4], F[c * 4 + 1], F[c * 4 + 2], F[c * 4 + 3]});
+  } else {
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) {
+      real row[Nt];
+#pragma unroll
+      for (int l = 0; l < i; ++l) {
+        row[l] = mass(i, l);
+#pragma unroll
+        for (int k = 0; k < l; ++k) row[l] += row[k] * LQ(l * (l + 1) / 2 + k);
+      }
+      real d = mass(i, i);
+#pragma unroll
+      for (int k = 0; k < i; ++k) {
+        const real nl = -(row[k] * LQ(k * (k + 1) / 2 + k));
+        d += row[k] * nl;
+        LQ(i * (i + 1) / 2 + k) = nl;
+      }
+      LQ(i * (i + 1) / 2 + i) = real(1) / d;
     }
-    LQ(i * (i + 1) / 2 + i) = real(1) / d;
   }
 #undef LQ
 }
@@ -838,8 +877,16 @@ __device__ __forceinline__ void quad_edge(const AllOps<N, real>& O, const real* 
 // and are requested before the slab arrives (meshes where some of them are
 // tets or lie in another block, StageArgs::tri_far; two blocks per CTA:
 // always); otherwise they are all in this block's slab.
-template <int N, int BPC, bool TF>
-__global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOpFFMA>())
+// OTF: the mass factor is formed in the stage, by warp 1 while the slab is in
+// flight (the other warps take its part of the geometry, and no traces are
+// requested before the slab has arrived, whose registers the factor needs: 322
+// us with, 304 without, 332 in an earlier form with two blocks per CTA; N = 3,
+// 524,288 wedges).
+// OP: M^tri on the CUDA cores, or (precision variants) on the tensor cores: the
+// four right-hand sides of a slice are then formed first and pass through the
+// warp's operand tile, which shares the residual slab's place.
+template <int N, int BPC, bool TF, bool OTF, int OP = kOpFFMA>
+__global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>())
     k_wedge_stage(const StageArgs<real> A, bool rk) {
   constexpr int Nt = nt_of(N), Nq = N + 1, Np = Nt * Nq, NH = (Nt + 1) / 2, NQH = (Nq + 1) / 2;
   // FP32 at N >= 4: the operator products as loops over the input nodes (tables
@@ -850,7 +897,8 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
   // more from leaving out the zeros of D_s: N = 4 1,295 against 1,360 us.)
   constexpr bool rolled = sizeof(real) == 4 && N >= 4;
   constexpr int NHP = (NH + 1) / 2 * 2;
-  using SM = WedgeSmem<N, kOpFFMA>;
+  static_assert(OP == kOpFFMA || (sizeof(real) == 4 && BPC == 1 && Nt <= 16), "tensor-core applies: FP32, Nt <= 16");
+  using SM = WedgeSmem<N, OP>;
   const AllOps<N, real>& O = OPS<N>();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   // block sb of this CTA: warps sb (N+1) .. sb (N+1) + N, one per slice
@@ -874,7 +922,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
   const int e = blk * kB + lane;
   const int Kp = M.Kw_pad;
   constexpr uint32_t slab_bytes = uint32_t(4 * Np * kB * sizeof(real));
-  const bool res_async = rk && stage_res<N, kOpFFMA>() && A.rk_a != real(0);
+  const bool res_async = rk && stage_res<N, OP>() && A.rk_a != real(0);
 #define GEO(item) sG[(item) * kB + lane]
   // the warps of one block synchronise among themselves (named barrier 1 + sb)
   auto block_sync = [&]() {
@@ -885,8 +933,12 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
   // 0. bulk copies of the block's state (and residual) slabs; geometry meanwhile
   constexpr int NL4 = nl4_of(N);
   constexpr uint32_t fac_bytes = uint32_t(NL4 * 4 * kB * sizeof(real));
-  const bool stored = M.w_fac != nullptr;
+  constexpr bool stored = !OTF;
   constexpr uint32_t xyz_bytes = uint32_t(12 * kB * sizeof(real));
+  if (A.pdl) {
+    pdl_launch_dependents();
+    pdl_wait();
+  }
   if (leader) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
@@ -900,15 +952,15 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
     bulk_g2s(sq, qin + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[0]);
     // stored mass factor: straight into the factor table with the state slab
     if (stored) bulk_g2s(sL, M.w_fac + int64_t(blk) * NL4 * 4 * kB, fac_bytes, &bar[0]);
-    if (res_async) {
+    if (res_async && OP == kOpFFMA) {
       mbar_expect_tx(&bar[1], slab_bytes);
       bulk_g2s(sr, A.res + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[1]);
-    } else if (rk && A.rk_a != real(0)) {
+    } else if (!res_async && rk && A.rk_a != real(0)) {
       // not staged: to L2 at least, for the update (N = 5: 438 -> 411 us per stage on 131,072 wedges)
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(A.res + int64_t(blk) * 4 * Np * kB), "r"(slab_bytes));
     }
   }
-  if (j == N) prefetch_ahead<N>(M, qin, blk + 76 * wedge_min_ctas<N, BPC, kOpFFMA>() * BPC, lane, N <= 4 && stored);
+  if (j == N) prefetch_ahead<N>(M, qin, blk + 76 * wedge_min_ctas<N, BPC, OP>() * BPC, lane, N <= 4 && stored);
   // face neighbours, their impedances and the source flag, loaded while the
   // slabs are in flight; so are (N <= 3) the neighbour traces
   const real kappa = M.w_mat[0 * Kp + e], irho = M.w_mat[1 * Kp + e], zM = M.w_mat[2 * Kp + e];
@@ -931,7 +983,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
   // requested here at N <= 3, after the slab has arrived at N = 4 (before it they
   // cost spills: 649 against 578 us per stage on 524,288 wedges, 600 face by
   // face), face by face at N = 5
-  constexpr bool early = N <= 3, mid = N == 4;
+  constexpr bool early = N <= 3 && !OTF, mid = N == 4 || (N <= 3 && OTF);
   Q4 nv[early || mid ? 3 : 1][Nq];
   if constexpr (early) {
 #pragma unroll
@@ -977,11 +1029,12 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
   const bool geo_ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[2], 0));
   if (geo_ok) {
 #pragma unroll 1
-    for (int p = j; p < kGeoParts; p += Nq) wedge_geometry_part<false>(p, sF, sG, lane);
+    for (int p = OTF ? (j == 1 ? kGeoParts : j - (j > 1)) : j; p < kGeoParts; p += OTF ? Nq - 1 : Nq)
+      wedge_geometry_part<false>(p, sF, sG, lane);
   } else if (lane == 0) {
     atomicOr(M.err, kErrTimeout);
   }
-  if (j == 1 && !stored) {
+  if (OTF && j == 1) {
     factor_wedge<N>(O, M, e, lane, sL);  // while the slabs are in flight
   }
   if (leader) *status = (mbar_wait_bounded(&bar[0], 0) && geo_ok) ? 1 : 0;
@@ -990,7 +1043,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
     // a copy never arrived: report, let any copy in flight drain, leave
     if (leader) {
       atomicOr(M.err, kErrTimeout);
-      if (res_async) mbar_wait_bounded(&bar[1], 0);
+      if (res_async && OP == kOpFFMA) mbar_wait_bounded(&bar[1], 0);
       mbar_wait_bounded(&bar[0], 0);
       mbar_wait_bounded(&bar[2], 0);
     }
@@ -1032,7 +1085,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
   // 2. M^tri applied in place to the four flux vectors (bottom F_p, F_u, top
   //    F_p, F_u), one per warp
 #pragma unroll 1
-  for (int v = j; v < 4; v += Nq) {
+  for (int v = OP == kOpFFMA ? j : 4; v < 4; v += Nq) {
     real* f = sF + ((v >> 1) * Nt * kB + lane) * 2 + (v & 1);
     real2 acc[NH];
     if constexpr (rolled) {
@@ -1087,24 +1140,41 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
   //    + A D_t u_z) and D_t p; W_p += M^tri dd, Mdp = M^tri D_t p
   const real tj = O.w.gll[j];
   const real ntx = -fmar(tj, GEO(G_TX1), GEO(G_TX0)), nty = -fmar(tj, GEO(G_TY1), GEO(G_TY0)), nA = -GEO(G_A);
-  real2 Mdp[NH];
-  {
-    real dtr[Nq];
+      real dtr[Nq];
 #pragma unroll
-    for (int m = 0; m < Nq; ++m) dtr[m] = O.w.Dt[j * Nq + m];
-    // node i: D_t of the four fields as two packed pairs (p, u_x) and (u_y, u_z)
-    auto t_part = [&](int i, real& dp, real& dd) {
-      real2 dpu = dup2(real(0)), dvw = dup2(real(0));
+      for (int m = 0; m < Nq; ++m) dtr[m] = O.w.Dt[j * Nq + m];
+      // node i: D_t of the four fields as two packed pairs (p, u_x) and (u_y, u_z)
+      auto t_part = [&](int i, real& dp, real& dd) {
+        real2 dpu = dup2(real(0)), dvw = dup2(real(0));
 #pragma unroll
-      for (int m = 0; m < Nq; ++m) {
-        const Q4 v = lds4(sq, m * Nt + i, lane);
-        const real2 d2 = dup2(dtr[m]);
-        dpu = fma2(d2, mk2(v.p, v.u), dpu);
-        dvw = fma2(d2, mk2(v.v, v.w), dvw);
-      }
-      dp = dpu.x;
-      dd = fmar(ntx, dpu.y, fmar(nty, dvw.x, nA * dvw.y));
-    };
+        for (int m = 0; m < Nq; ++m) {
+          const Q4 v = lds4(sq, m * Nt + i, lane);
+          const real2 d2 = dup2(dtr[m]);
+          dpu = fma2(d2, mk2(v.p, v.u), dpu);
+          dvw = fma2(d2, mk2(v.v, v.w), dvw);
+        }
+        dp = dpu.x;
+        dd = fmar(ntx, dpu.y, fmar(nty, dvw.x, nA * dvw.y));
+      };
+  real2 W01[Nt], W23[Nt];
+  // the coefficients of the four right-hand sides, and node i's values from the
+  // flux pairs, the pressure's (a) and D_t p's (d) part
+  struct Lift {
+    real2 b01, t01, b23, t23, n23;
+    real ntx;
+    __device__ __forceinline__ void node(const real2 fb, const real2 ft, real a, real d, real2& w01, real2& w23) const {
+      w01 = fma2(fb, b01, fma2(ft, t01, mk2(a, ntx * d)));
+      w23 = fma2(dup2(fb.y), b23, fma2(dup2(ft.y), t23, mul2(dup2(d), n23)));
+    }
+  };
+  auto lift_coef = [&]() {
+    const real cb = real(0.5) * GEO(G_JFB) * O.w.ell0[j], ct = real(0.5) * GEO(G_JFT) * O.w.ellN[j];
+    return Lift{mk2(cb, cb * GEO(G_NB0)), mk2(ct, ct * GEO(G_NT0)), mk2(cb * GEO(G_NB1), cb * GEO(G_NB2)),
+                mk2(ct * GEO(G_NT1), ct * GEO(G_NT2)), mk2(nty, nA), ntx};
+  };
+  auto flux_pair = [&](int fb, int i) { return *reinterpret_cast<const real2*>(sF + ((fb * Nt + i) * kB + lane) * 2); };
+  if constexpr (OP == kOpFFMA) {
+    real2 Mdp[NH];
     if constexpr (rolled) {
       // a node's two values go into both products at once
 #pragma unroll
@@ -1133,25 +1203,59 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
       }
       apply_pairs<Nt, Nt>(O.w.MP, dp, Mdp);
     }
-  }
-  block_sync();  // M^tri has been applied to the flux vectors
-
-  // 5. right-hand sides of the mass solve by field pairs (p, u_x), (u_y, u_z):
-  //    the lifted triangle-face fluxes, -t_cJ M D_t p and the quadrilateral faces
-  real2 W01[Nt], W23[Nt];
-  {
-    const real cb = real(0.5) * GEO(G_JFB) * O.w.ell0[j], ct = real(0.5) * GEO(G_JFT) * O.w.ellN[j];
-    const real2 b01 = mk2(cb, cb * GEO(G_NB0)), t01 = mk2(ct, ct * GEO(G_NT0));
-    const real2 b23 = mk2(cb * GEO(G_NB1), cb * GEO(G_NB2)), t23 = mk2(ct * GEO(G_NT1), ct * GEO(G_NT2));
-    const real2 n23 = mk2(nty, nA);
+    block_sync();  // M^tri has been applied to the flux vectors
+    // 5. right-hand sides of the mass solve by field pairs (p, u_x), (u_y, u_z):
+    //    the lifted triangle-face fluxes, -t_cJ M D_t p and the quadrilateral faces
+    const Lift C = lift_coef();
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) C.node(flux_pair(0, i), flux_pair(1, i), pair_row(Wp, i), pair_row(Mdp, i), W01[i], W23[i]);
+  } else {
+    // 4, 5 on the tensor cores: the four vectors of every element of the block go
+    // to this warp's tile (columns lane * 4 + field), M^tri is applied one 16 x 8
+    // output tile at a time in place, and each lane reads its element's results back
+    real* sT = base + SM::T + j * Nt * kTP;
+    const Lift C = lift_coef();
 #pragma unroll
     for (int i = 0; i < Nt; ++i) {
-      const real2 fb = *reinterpret_cast<const real2*>(sF + ((0 * Nt + i) * kB + lane) * 2);
-      const real2 ft = *reinterpret_cast<const real2*>(sF + ((1 * Nt + i) * kB + lane) * 2);
-      const real md = pair_row(Mdp, i);
-      W01[i] = fma2(fb, b01, fma2(ft, t01, mk2(pair_row(Wp, i), ntx * md)));
-      W23[i] = fma2(dup2(fb.y), b23, fma2(dup2(ft.y), t23, mul2(dup2(md), n23)));
+      real dp, dd;
+      real2 g01, g23;
+      t_part(i, dp, dd);
+      C.node(flux_pair(0, i), flux_pair(1, i), dd, dp, g01, g23);
+      *reinterpret_cast<float4*>(sT + tile_at(i, lane * 4)) = make_float4(g01.x, g01.y, g23.x, g23.y);
     }
+    __syncwarp();
+    {
+      AFrag<OP> Am;
+      afrag_load<Nt, OP>(O.w.M, lane, Am);
+      const int g = lane >> 2, t = lane & 3;
+#pragma unroll 2
+      for (int nt = 0; nt < 16; ++nt) {
+        BFrag<OP> Bf;
+        bfrag_load<Nt, OP>(sT, nt * 8 + g, lane, Bf);
+        float d[4] = {0.f, 0.f, 0.f, 0.f};
+        op_mma<Nt, OP>(Am, Bf, d);
+        if (g < Nt) *reinterpret_cast<float2*>(sT + tile_at(g, nt * 8 + 2 * t)) = make_float2(d[0], d[1]);
+        if (g + 8 < Nt) *reinterpret_cast<float2*>(sT + tile_at(g + 8, nt * 8 + 2 * t)) = make_float2(d[2], d[3]);
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < Nt; ++i) {
+      const float4 w = *reinterpret_cast<const float4*>(sT + tile_at(i, lane * 4));
+      W01[i] = mk2(w.x + pair_row(Wp, i), w.y);
+      W23[i] = mk2(w.z, w.w);
+    }
+    if (res_async) {
+      // every warp is done with its tile: the residual slab may now land in their space
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      block_sync();
+      if (leader) {
+        mbar_expect_tx(&bar[1], slab_bytes);
+        bulk_g2s(sr, A.res + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[1]);
+      }
+    }
+  }
+  {
 #pragma unroll
     for (int ed = 0; ed < 3; ++ed) {
       const real nx = GEO(G_QNX0 + ed), ny = GEO(G_QNY0 + ed);
@@ -1236,8 +1340,8 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, kOp
     mbar_wait_bounded(&bar[1], 0);
     return;
   }
-  if (src) add_sources(M, 6, e, j * Nt, Np, *M.clock + A.c_stage * double(A.dt), W01);
-  wedge_update<N, stage_res<N, kOpFFMA>()>(A, rk, sq, sr, blk, j, lane, e, kappa, irho, W01, W23);
+  if (src) add_sources(M, 6, e, j * Nt, Np, M.clock[A.clk] + A.c_stage * double(A.dt), W01);
+  wedge_update<N, stage_res<N, OP>()>(A, rk, sq, sr, blk, j, lane, e, kappa, irho, W01, W23);
 #undef GEO
 }
 
@@ -1323,19 +1427,44 @@ __global__ void __launch_bounds__(128) k_wedge_wide(const StageArgs<real> A, boo
     mbar_expect_tx(&bar[2], xyz_bytes);
     bulk_g2s(sF, M.w_xyz + int64_t(blk) * 12 * kB, xyz_bytes, &bar[2]);  // in the flux table's place, written later
     mbar_expect_tx(&bar[0], slab_bytes + (stored ? fac_bytes : 0u));
-    bulk_g2s(sq, qin + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[0]);
     if (stored) bulk_g2s(sL, M.w_fac + int64_t(blk) * NL4 * 4 * kB, fac_bytes, &bar[0]);
-    if (res_async) {
-      mbar_expect_tx(&bar[1], res_bytes);
-      bulk_g2s(sr, A.res + widx<N>(blk, j * Nt, 0), res_bytes, &bar[1]);
-    }
   }
+  pdl_launch_dependents();
   // neighbours: warp f < 3 takes quadrilateral face f, all warps share the triangle-face nodes
   const real kappa = M.w_mat[0 * Kp + e], irho = M.w_mat[1 * Kp + e], zM = M.w_mat[2 * Kp + e];
   const int ed = f < 3 ? f : 0;
   const int qnbr = M.w_nbr[(2 + ed) * Kp + e], qcode = M.w_code[(2 + ed) * Kp + e];
   const int tnbr[2] = {M.w_nbr[0 * Kp + e], M.w_nbr[1 * Kp + e]};
   const int tcode[2] = {M.w_code[0 * Kp + e], M.w_code[1 * Kp + e]};
+  const real zPq = qnbr < 0 ? zM : M.w_mat[2 * Kp + qnbr];
+  real ntp[2], ntu[2];
+#pragma unroll
+  for (int fb = 0; fb < 2; ++fb) {
+    const real zP = tnbr[fb] < 0 ? zM
+                                 : ((tcode[fb] & kCodeTet) ? M.t_mat[2 * M.Kt_pad + tnbr[fb]] : M.w_mat[2 * Kp + tnbr[fb]]);
+    real tp, tu;
+    taus(A.flux, zM, zP, tp, tu);
+    ntp[fb] = -tp;
+    ntu[fb] = -tu;
+  }
+  const bool src = f == 0 && M.nsrc > 0 && has_source(M, 6, e);
+  // the geometry needs the mesh alone: before the wait for the previous stage
+  __syncthreads();  // the mbarriers are initialised
+  const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[2], 0));
+  if (ok) {
+#pragma unroll 1
+    for (int p = 3 - f; p < kGeoParts; p += 4) wedge_geometry_part<false>(p, sF, sG, lane);
+  } else if (lane == 0) {
+    atomicOr(M.err, kErrTimeout);
+  }
+  pdl_wait();
+  if (threadIdx.x == 0) {
+    bulk_g2s(sq, qin + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[0]);
+    if (res_async) {
+      mbar_expect_tx(&bar[1], res_bytes);
+      bulk_g2s(sr, A.res + widx<N>(blk, j * Nt, 0), res_bytes, &bar[1]);
+    }
+  }
   Q4 tv[Nq];
   {
     const bool bnd = qnbr < 0;
@@ -1357,26 +1486,6 @@ __global__ void __launch_bounds__(128) k_wedge_wide(const StageArgs<real> A, boo
     const int nk = bnd ? k : O.tab.tri_perm[code & 15][k];
     const int node = ntet ? O.tab.tet_face[nf][nk] : (nf ? N * Nt : 0) + nk;
     tnv[t] = ldg4(qin, ntet ? tidx<N>(M.tet_off, nbe >> 5, node, nbe & 31) : widx<N>(nbe >> 5, node, nbe & 31));
-  }
-  const real zPq = qnbr < 0 ? zM : M.w_mat[2 * Kp + qnbr];
-  real ntp[2], ntu[2];
-#pragma unroll
-  for (int fb = 0; fb < 2; ++fb) {
-    const real zP = tnbr[fb] < 0 ? zM
-                                 : ((tcode[fb] & kCodeTet) ? M.t_mat[2 * M.Kt_pad + tnbr[fb]] : M.w_mat[2 * Kp + tnbr[fb]]);
-    real tp, tu;
-    taus(A.flux, zM, zP, tp, tu);
-    ntp[fb] = -tp;
-    ntu[fb] = -tu;
-  }
-  const bool src = f == 0 && M.nsrc > 0 && has_source(M, 6, e);
-  __syncthreads();  // the mbarriers are initialised
-  const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[2], 0));
-  if (ok) {
-#pragma unroll 1
-    for (int p = 3 - f; p < kGeoParts; p += 4) wedge_geometry_part<false>(p, sF, sG, lane);
-  } else if (lane == 0) {
-    atomicOr(M.err, kErrTimeout);
   }
   if (threadIdx.x == 96) *status = (ok && mbar_wait_bounded(&bar[0], 0)) ? 1 : 0;
   if (f == 0 && !stored) factor_wedge<N>(O, M, e, lane, sL);
@@ -1574,7 +1683,7 @@ __global__ void __launch_bounds__(128) k_wedge_wide(const StageArgs<real> A, boo
   if (f == 0) {
 #pragma unroll
     for (int i = 0; i < Nt; ++i) W[i] -= i < 2 * HA ? pair_row(dv, i < 2 * HA ? i : 0) : sD[i * kB + lane];
-    if (src) add_sources(M, 6, e, j * Nt, Np, *M.clock + A.c_stage * double(A.dt), W);
+    if (src) add_sources(M, 6, e, j * Nt, Np, M.clock[A.clk] + A.c_stage * double(A.dt), W);
   } else if (f < 3) {
     const real nr = f == 1 ? -rx : -ry, ns = f == 1 ? -sx : -sy;
 #pragma unroll
@@ -1603,356 +1712,6 @@ __global__ void __launch_bounds__(128) k_wedge_wide(const StageArgs<real> A, boo
       U.node(A, rk, widx<N>(blk, j * Nt + i, lane), W01, W23, r0, lds4(sq, j * Nt + i, lane));
     }
   }
-#undef GEO
-}
-
-// The stage with M^tri applied on the tensor cores (precision variants): one
-// block per CTA, the four right-hand sides of a slice formed first and passed
-// through the warp's operand tile.
-template <int N, int OP>
-__global__ void __launch_bounds__(32 * (N + 1), wedge_min_ctas<N, 1, OP>())
-    k_wedge_stage_mma(const StageArgs<real> A, bool rk) {
-  constexpr int Nt = nt_of(N), Nq = N + 1, Np = Nt * Nq;
-  static_assert(sizeof(real) == 4 && Nt <= 16, "tensor-core applies: FP32, Nt <= 16");
-  using SM = WedgeSmem<N, OP>;
-  const AllOps<N, real>& O = OPS<N>();
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  const int j = threadIdx.x >> 5;
-  const bool leader = threadIdx.x == 0;
-  // [0] state slab (and stored factor), [1] residual slab, [2] vertex coordinates
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
-  int* status = reinterpret_cast<int*>(smem_raw + 24);
-  real* base = reinterpret_cast<real*>(smem_raw + 32);
-  real* sq = base + SM::q;
-  real* sr = base + SM::r;
-  real* sL = base + SM::L;
-  real* sF = base + SM::F;
-  real* sG = base + SM::G;
-  real* sT = base + SM::T + j * Nt * kTP;  // this warp's operand tile (tensor cores)
-  const DevMesh<real>& M = A.m;
-  const real* __restrict__ qin = A.q_in;
-  const int lane = threadIdx.x & 31;
-  const int blk = blockIdx.x;
-  const int e = blk * kB + lane;
-  const int Kp = M.Kw_pad;
-  constexpr uint32_t slab_bytes = uint32_t(4 * Np * kB * sizeof(real));
-  // the residual copy is issued after the weak-form accumulation, once the
-  // operand tiles in its space are free
-  const bool res_async = rk && stage_res<N, OP>() && A.rk_a != real(0);
-#define GEO(item) sG[(item) * kB + lane]
-
-  auto block_sync = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(32 * Nq) : "memory"); };
-  // 0. bulk copies of the block's state (and residual) slabs; geometry meanwhile
-  constexpr int NL4 = nl4_of(N);
-  constexpr uint32_t fac_bytes = uint32_t(NL4 * 4 * kB * sizeof(real));
-  const bool stored = M.w_fac != nullptr;
-  constexpr uint32_t xyz_bytes = uint32_t(12 * kB * sizeof(real));
-  if (leader) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
-    mbar_init(&bar[2], 1);
-    fence_mbar_init();
-    // the block's vertex coordinates first (the geometry warp waits on them alone)
-    mbar_expect_tx(&bar[2], xyz_bytes);
-    bulk_g2s(sF, M.w_xyz + int64_t(blk) * 12 * kB, xyz_bytes, &bar[2]);
-    mbar_expect_tx(&bar[0], slab_bytes + (stored ? fac_bytes : 0u));
-    bulk_g2s(sq, qin + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[0]);
-    // stored mass factor: straight into the factor table with the state slab
-    if (stored) bulk_g2s(sL, M.w_fac + int64_t(blk) * NL4 * 4 * kB, fac_bytes, &bar[0]);
-  }
-  if (j == N) prefetch_ahead<N>(M, qin, blk + 76 * wedge_min_ctas<N, 1, OP>(), lane, stored);
-  // face neighbours, their impedances and the source flag, loaded while the
-  // slabs are in flight; so are the traces of quadrilateral-face neighbours
-  // outside this block (global memory, read-only during the stage)
-  const real kappa = M.w_mat[0 * Kp + e], irho = M.w_mat[1 * Kp + e], zM = M.w_mat[2 * Kp + e];
-  int qnbr[3], qcode[3];
-  real zPq[3];
-#pragma unroll
-  for (int ed = 0; ed < 3; ++ed) {
-    qnbr[ed] = M.w_nbr[(2 + ed) * Kp + e];
-    qcode[ed] = M.w_code[(2 + ed) * Kp + e];
-  }
-  // (at N = 4 the traces held across the wait cost spills, and with the factor
-  // computed in the stage they slow the factorising warp: there they are
-  // requested after the wait, with the in-block ones)
-  const bool early = N <= 3 && stored;
-  Q4 nv[3][Nq];
-#pragma unroll
-  for (int ed = 0; ed < 3; ++ed) {
-    const int nbr = qnbr[ed];
-    if (early && nbr >= 0 && (nbr >> 5) != blk) {
-      const int ep = qcode[ed] >> 1, rev = qcode[ed] & 1;
-      const real* base = qin + widx<N>(nbr >> 5, 0, nbr & 31);
-#pragma unroll
-      for (int m = 0; m < Nq; ++m) nv[ed][m] = ldg4(base, int64_t(j * Nt + O.tab.edge[ep][rev ? N - m : m]) * (kB * 4));
-    }
-  }
-#pragma unroll
-  for (int ed = 0; ed < 3; ++ed) zPq[ed] = qnbr[ed] < 0 ? zM : M.w_mat[2 * Kp + qnbr[ed]];
-  const int tnbr[2] = {M.w_nbr[0 * Kp + e], M.w_nbr[1 * Kp + e]};
-  const int tcode[2] = {M.w_code[0 * Kp + e], M.w_code[1 * Kp + e]};
-  real zPt[2];
-#pragma unroll
-  for (int fb = 0; fb < 2; ++fb)
-    zPt[fb] = tnbr[fb] < 0 ? zM
-                           : ((tcode[fb] & kCodeTet) ? M.t_mat[2 * M.Kt_pad + tnbr[fb]] : M.w_mat[2 * Kp + tnbr[fb]]);
-  const bool src = M.nsrc > 0 && has_source(M, 6, e);
-  block_sync();  // the mbarriers are initialised
-  const bool geo_ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[2], 0));
-  if (geo_ok) {
-#pragma unroll 1
-    for (int p = j; p < kGeoParts; p += Nq) wedge_geometry_part<false>(p, sF, sG, lane);
-  } else if (lane == 0) {
-    atomicOr(M.err, kErrTimeout);
-  }
-  if (j == 1 && !stored) {
-    factor_wedge<N>(O, M, e, lane, sL);  // while the slabs are in flight
-  }
-  if (leader) *status = (mbar_wait_bounded(&bar[0], 0) && geo_ok) ? 1 : 0;
-  block_sync();
-  if (*reinterpret_cast<volatile int*>(status) == 0) {
-    // the state slab never arrived: report, let any copy in flight drain, leave
-    if (leader) {
-      atomicOr(M.err, kErrTimeout);
-      mbar_wait_bounded(&bar[0], 0);
-      mbar_wait_bounded(&bar[2], 0);
-    }
-    return;
-  }
-
-  // 1. prologue: quadrilateral-face fluxes of slice j applied straight into the
-  //    weak-form accumulators (every warp); triangle-face fluxes (warps 0 and N)
-  // accumulators of node i of the slice by field pairs: W01[i] = (p, u_x),
-  // W23[i] = (u_y, u_z), so that the mass solve and the update run on packed pairs
-  constexpr int NH = (Nt + 1) / 2;
-  real2 W01[Nt], W23[Nt];
-#pragma unroll
-  for (int i = 0; i < Nt; ++i) W01[i] = W23[i] = dup2(real(0));
-  // the neighbour node of triangle-face flux t of this warp (round-robin over
-  // the warps, bottom then top): a tet's face node, or a wedge's bottom/top
-  // node in this block's slab or in global memory; a boundary face reads its
-  // own node
-  constexpr int NTT = (2 * Nt + Nq - 1) / Nq;
-  auto tri_nbr_node = [&](int t) {
-    const int idx = j + t * Nq;
-    const int fb = idx >= Nt ? 1 : 0;
-    const int k = idx - fb * Nt;
-    const int nbr = tnbr[fb];
-    const int code = tcode[fb];
-    const bool bnd = nbr < 0;
-    const bool ntet = !bnd && (code & kCodeTet) != 0;
-    const int nf = bnd ? fb : (code >> 4) & 3;
-    const int nk = bnd ? k : O.tab.tri_perm[code & 15][k];
-    const int nbe = bnd ? e : nbr;
-    const int node = ntet ? O.tab.tet_face[nf][nk] : (nf ? N * Nt : 0) + nk;
-    const bool inblk = !ntet && (nbe >> 5) == blk;
-    // explicit shared or global loads (a generic load would wait on the long scoreboard either way)
-    return inblk ? lds4(sq, node, nbe & 31)
-                 : ldg4(qin, ntet ? tidx<N>(M.tet_off, nbe >> 5, node, nbe & 31) : widx<N>(nbe >> 5, node, nbe & 31));
-  };
-  // neighbour traces of quadrilateral faces whose neighbour lies in this block
-  // (or, on a boundary face, the element's own trace, which the ghost state
-  // then replaces) from the shared slab; the others were requested above (or,
-  // at N = 4, now, from global memory)
-#pragma unroll
-  for (int ed = 0; ed < 3; ++ed) {
-    const int nbr = qnbr[ed];
-    const bool bnd = nbr < 0;
-    const bool inblk = bnd || (nbr >> 5) == blk;
-    const int ep = bnd ? ed : qcode[ed] >> 1, rev = bnd ? 0 : qcode[ed] & 1;
-    if (inblk) {
-      const int nl = bnd ? lane : (nbr & 31);
-#pragma unroll
-      for (int m = 0; m < Nq; ++m) nv[ed][m] = lds4(sq, j * Nt + O.tab.edge[ep][rev ? N - m : m], nl);
-    } else if (!early) {
-      const real* base = qin + widx<N>(nbr >> 5, 0, nbr & 31);
-#pragma unroll
-      for (int m = 0; m < Nq; ++m) nv[ed][m] = ldg4(base, int64_t(j * Nt + O.tab.edge[ep][rev ? N - m : m]) * (kB * 4));
-    }
-  }
-#pragma unroll
-  for (int ed = 0; ed < 3; ++ed) {
-    const real nx = GEO(G_QNX0 + ed), ny = GEO(G_QNY0 + ed);
-    real Fp[Nq], Fu[Nq];
-    real tau_p, tau_u;
-    taus(A.flux, zM, zPq[ed], tau_p, tau_u);
-#pragma unroll
-    for (int m = 0; m < Nq; ++m) {
-      const Q4 o = lds4(sq, j * Nt + edge_node(N, ed, m), lane);
-      real bdp, bdun;
-      boundary_jumps(A.bc, o.p, nx * o.u + ny * o.v, bdp, bdun);
-      const bool bnd = qnbr[ed] < 0;
-      const real dp = bnd ? bdp : nv[ed][m].p - o.p;
-      const real dun = bnd ? bdun : nx * (nv[ed][m].u - o.u) + ny * (nv[ed][m].v - o.v);
-      penalty_flux(dp, dun, tau_p, tau_u, Fp[m], Fu[m]);
-    }
-    // W += M~_e F, M~_e = (L_e/4)(h_a Mea + h_b Meb) along the edge, identity in t
-    // (Mea, Meb applied by output pairs: packed multiply-adds)
-    const real ca = GEO(G_QCA0 + ed), cbq = GEO(G_QCB0 + ed);
-    constexpr int NQH = (Nq + 1) / 2;
-    real2 gpa[NQH], gpb[NQH], gua[NQH], gub[NQH];
-#pragma unroll
-    for (int h = 0; h < NQH; ++h) gpa[h] = gpb[h] = gua[h] = gub[h] = dup2(real(0));
-#pragma unroll
-    for (int n = 0; n < Nq; ++n) {
-      const real2 fp2 = dup2(Fp[n]), fu2 = dup2(Fu[n]);
-#pragma unroll
-      for (int h = 0; h < NQH; ++h) {
-        const real2 ea = cpair(O.w.MeaP, Nq, h, n), eb = cpair(O.w.MebP, Nq, h, n);
-        gpa[h] = fma2(ea, fp2, gpa[h]);
-        gpb[h] = fma2(eb, fp2, gpb[h]);
-        gua[h] = fma2(ea, fu2, gua[h]);
-        gub[h] = fma2(eb, fu2, gub[h]);
-      }
-    }
-#pragma unroll
-    for (int m = 0; m < Nq; ++m) {
-      const bool hi = m & 1;
-      const real2 pa = gpa[m >> 1], pb = gpb[m >> 1], ua = gua[m >> 1], ub = gub[m >> 1];
-      const real gp = ca * (hi ? pa.y : pa.x) + cbq * (hi ? pb.y : pb.x);
-      const real gu = ca * (hi ? ua.y : ua.x) + cbq * (hi ? ub.y : ub.x);
-      const int i = edge_node(N, ed, m);
-      W01[i].x += gp;
-      W01[i].y += nx * gu;
-      W23[i].x += ny * gu;
-    }
-  }
-  // triangle-face node fluxes (bottom then top), spread round-robin over the warps
-#pragma unroll
-  for (int t = 0; t < NTT; ++t) {
-    const int idx = j + t * Nq;
-    if (idx >= 2 * Nt) break;
-    const int fb = idx >= Nt ? 1 : 0;
-    const int k = idx - fb * Nt;
-    const real nn0 = GEO(fb ? G_NT0 : G_NB0), nn1 = GEO(fb ? G_NT1 : G_NB1), nn2 = GEO(fb ? G_NT2 : G_NB2);
-    const int nbr = tnbr[fb];
-    const Q4 o = lds4(sq, (fb ? N * Nt : 0) + k, lane);
-    const real unM = fmar(nn2, o.w, fmar(nn1, o.v, nn0 * o.u));
-    real tau_p, tau_u, bdp, bdun;
-    taus(A.flux, zM, fb ? zPt[1] : zPt[0], tau_p, tau_u);
-    boundary_jumps(A.bc, o.p, unM, bdp, bdun);
-    const bool bnd = nbr < 0;
-    const Q4 nv = tri_nbr_node(t);
-    const real dp = bnd ? bdp : nv.p - o.p;
-    const real dun = bnd ? bdun : fmar(nn2, nv.w, fmar(nn1, nv.v, nn0 * nv.u)) - unM;
-    real Fp, Fu;
-    penalty_flux(dp, dun, tau_p, tau_u, Fp, Fu);
-    sF[((2 * fb + 0) * Nt + k) * kB + lane] = Fp;
-    sF[((2 * fb + 1) * Nt + k) * kB + lane] = Fu;
-  }
-  block_sync();
-
-  // 2. slice j of every element of the block
-  {
-    real dtr[Nq];
-#pragma unroll
-    for (int m = 0; m < Nq; ++m) dtr[m] = O.w.Dt[j * Nq + m];
-    const real tj = O.w.gll[j];
-    const real txJ = GEO(G_TX0) + tj * GEO(G_TX1);
-    const real tyJ = GEO(G_TY0) + tj * GEO(G_TY1);
-    const real Aj = GEO(G_A);
-    const real cb = GEO(G_JFB) * O.w.ell0[j];
-    const real ct = GEO(G_JFT) * O.w.ellN[j];
-    {
-      // (a, b) on the tensor cores: the four vectors G of every element of
-      // the block go to this warp's tile (columns lane * 4 + field), M^tri G
-      // is formed one 16 x 8 output tile at a time in place, and each lane
-      // reads its element's four results back
-      const real nb0 = GEO(G_NB0) * cb, nb1 = GEO(G_NB1) * cb, nb2 = GEO(G_NB2) * cb;
-      const real nt0 = GEO(G_NT0) * ct, nt1 = GEO(G_NT1) * ct, nt2 = GEO(G_NT2) * ct;
-#pragma unroll
-      for (int i = 0; i < Nt; ++i) {
-        real dpp = 0, dux = 0, duy = 0, duz = 0;
-#pragma unroll
-        for (int m = 0; m < Nq; ++m) {
-          const Q4 v = lds4(sq, m * Nt + i, lane);
-          dpp += dtr[m] * v.p;
-          dux += dtr[m] * v.u;
-          duy += dtr[m] * v.v;
-          duz += dtr[m] * v.w;
-        }
-        const real fp = sF[(1 * Nt + i) * kB + lane], fq = sF[(3 * Nt + i) * kB + lane];
-        const float4 gv = make_float4(
-            cb * sF[(0 * Nt + i) * kB + lane] + ct * sF[(2 * Nt + i) * kB + lane] - (txJ * dux + tyJ * duy + Aj * duz),
-            nb0 * fp + nt0 * fq - txJ * dpp, nb1 * fp + nt1 * fq - tyJ * dpp, nb2 * fp + nt2 * fq - Aj * dpp);
-        *reinterpret_cast<float4*>(sT + tile_at(i, lane * 4)) = gv;
-      }
-      __syncwarp();
-      {
-        AFrag<OP> Am;
-        afrag_load<Nt, OP>(O.w.M, lane, Am);
-        const int g = lane >> 2, t = lane & 3;
-#pragma unroll 2
-        for (int nt = 0; nt < 16; ++nt) {
-          BFrag<OP> Bf;
-          bfrag_load<Nt, OP>(sT, nt * 8 + g, lane, Bf);
-          float d[4] = {0.f, 0.f, 0.f, 0.f};
-          op_mma<Nt, OP>(Am, Bf, d);
-          if (g < Nt) *reinterpret_cast<float2*>(sT + tile_at(g, nt * 8 + 2 * t)) = make_float2(d[0], d[1]);
-          if (g + 8 < Nt) *reinterpret_cast<float2*>(sT + tile_at(g + 8, nt * 8 + 2 * t)) = make_float2(d[2], d[3]);
-        }
-      }
-      __syncwarp();
-#pragma unroll
-      for (int i = 0; i < Nt; ++i) {
-        const float4 w = *reinterpret_cast<const float4*>(sT + tile_at(i, lane * 4));
-        W01[i] = add2(W01[i], mk2(w.x, w.y));
-        W23[i] = add2(W23[i], mk2(w.z, w.w));
-      }
-      if (res_async) {
-        // every warp is done with its tile: the residual slab may now land in their space
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        block_sync();
-        if (leader) {
-          mbar_expect_tx(&bar[1], slab_bytes);
-          bulk_g2s(sr, A.res + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[1]);
-        }
-      }
-    }
-  }
-  // (d) X = (M^{tri,k})^{-1} W
-  mass_solve<N>(sL, lane, W01, W23);
-  // (e) strong r, s parts of slice j (constant metric terms, Lemma 3.1), on
-  // the CUDA cores for every variant (on the tensor cores the results would
-  // have to pass through shared memory back to the element's lane, which
-  // measured slower than these FMAs with constant operands)
-  {
-    // (D_r, D_s applied by output pairs, node l of the slice at a time)
-    const real rx = GEO(G_RX), ry = GEO(G_RY), sx = GEO(G_SX), sy = GEO(G_SY);
-    real2 dv[NH], pr[NH], ps[NH];
-#pragma unroll
-    for (int h = 0; h < NH; ++h) dv[h] = pr[h] = ps[h] = dup2(real(0));
-#pragma unroll
-    for (int l = 0; l < Nt; ++l) {
-      const Q4 v = lds4(sq, j * Nt + l, lane);
-      const real2 p2 = dup2(v.p), a2 = dup2(rx * v.u + ry * v.v), b2 = dup2(sx * v.u + sy * v.v);
-#pragma unroll
-      for (int h = 0; h < NH; ++h) {
-        const real2 r2 = cpair(O.w.DrP, Nt, h, l), s2 = cpair(O.w.DsP, Nt, h, l);
-        dv[h] = fma2(r2, a2, dv[h]);
-        dv[h] = fma2(s2, b2, dv[h]);
-        pr[h] = fma2(r2, p2, pr[h]);
-        ps[h] = fma2(s2, p2, ps[h]);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < Nt; ++i) {
-      const bool hi = i & 1;
-      const real dvi = hi ? dv[i >> 1].y : dv[i >> 1].x;
-      const real pri = hi ? pr[i >> 1].y : pr[i >> 1].x, psi = hi ? ps[i >> 1].y : ps[i >> 1].x;
-      W01[i].x -= dvi;
-      W01[i].y -= rx * pri + sx * psi;
-      W23[i].x -= ry * pri + sy * psi;
-    }
-  }
-  // (f) fused low-storage Runge-Kutta update (or plain right-hand side)
-  if (res_async && !mbar_wait_bounded(&bar[1], 0)) {
-    if (lane == 0) atomicOr(M.err, kErrTimeout);
-    mbar_wait_bounded(&bar[1], 0);
-    return;
-  }
-  if (src) add_sources(M, 6, e, j * Nt, Np, *M.clock + A.c_stage * double(A.dt), W01);
-  wedge_update<N, stage_res<N, OP>()>(A, rk, sq, sr, blk, j, lane, e, kappa, irho, W01, W23);
 #undef GEO
 }
 
@@ -2287,7 +2046,7 @@ __global__ void __launch_bounds__(128, (sizeof(REAL) == 4) ? (N >= 4 ? 3 : 5) : 
   real p[C];
 #pragma unroll
   for (int c = 0; c < C; ++c) p[c] = pair_row(ap, c);
-  if (src) add_sources(M, 4, e, I0, Np, *M.clock + A.c_stage * double(A.dt), p);
+  if (src) add_sources(M, 4, e, I0, Np, M.clock[A.clk] + A.c_stage * double(A.dt), p);
   if (res_async && !__all_sync(0xffffffffu, mbar_wait_bounded(&bar[3], 0))) {
     // the residual slab never arrived: report, let the copy drain, leave
     if (lane == 0) {
@@ -2570,16 +2329,22 @@ namespace REALNS {
 // one-time per device: opt in to the dynamic shared memory the stages use
 template <int N, int OP>
 cudaError_t prepare_op() {
-  return cudaFuncSetAttribute(k_wedge_stage_mma<N, OP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              wedge_smem_bytes<N, 1, OP>());
+  const cudaError_t err = cudaFuncSetAttribute(k_wedge_stage<N, 1, true, false, OP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               wedge_smem_bytes<N, 1, OP>());
+  return err != cudaSuccess ? err
+                            : cudaFuncSetAttribute(k_wedge_stage<N, 1, true, true, OP>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, wedge_smem_bytes<N, 1, OP>());
 }
 template <int N>
 int prepare_n() {
-  constexpr int b2 = wedge_bpc_onthefly<N>();
-  cudaError_t err = cudaFuncSetAttribute(k_wedge_stage<N, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  constexpr int b2 = wedge_bpc_multi<N>();
+  cudaError_t err = cudaFuncSetAttribute(k_wedge_stage<N, 1, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          wedge_smem_bytes<N, 1>());
   if (err == cudaSuccess)
-    err = cudaFuncSetAttribute(k_wedge_stage<N, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    err = cudaFuncSetAttribute(k_wedge_stage<N, 1, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               wedge_smem_bytes<N, 1>());
+  if (err == cudaSuccess)
+    err = cudaFuncSetAttribute(k_wedge_stage<N, 1, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                wedge_smem_bytes<N, 1>());
   if constexpr (sizeof(real) == 4) {
     if (err == cudaSuccess)
@@ -2595,9 +2360,14 @@ int prepare_n() {
     if (err == cudaSuccess)
       err = cudaFuncSetAttribute(k_wedge_wide<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide_smem_bytes<N>());
   }
-  if (err == cudaSuccess && b2 != 1)
-    err = cudaFuncSetAttribute(k_wedge_stage<N, b2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               wedge_smem_bytes<N, b2>());
+  if constexpr (b2 != 1) {
+    if (err == cudaSuccess)
+      err = cudaFuncSetAttribute(k_wedge_stage<N, b2, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 wedge_smem_bytes<N, b2>());
+    if (err == cudaSuccess)
+      err = cudaFuncSetAttribute(k_wedge_stage<N, b2, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 wedge_smem_bytes<N, b2>());
+  }
   if (err == cudaSuccess)
     err = cudaFuncSetAttribute(k_tet_stage<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, tet_smem_bytes<N>());
   if (err == cudaSuccess)
@@ -2619,15 +2389,34 @@ int prepare_n() {
   return int(err);
 }
 
-// The small-mesh stage up to this many CTAs (blocks x slices): about one per SM.
+// The small-mesh stage up to this many CTAs (blocks x slices): about one wave.
 // us per stage of a step, small-mesh against large-mesh form, by blocks: FP32
-// N = 3 1: 5.8 / 7.0, 32: 6.4 / 7.0, 64: 7.0 / 7.4, 128: 8.0 / 7.4; N = 4
-// 32: 10.7 / 12.3, 64: 17 / 12; N = 5 32: 27 / 45; FP64 N = 3 1-32: 37 / 82,
-// 64: 58 / 82, 128: 112 / 83; N = 4 32: 131 / 192, 64: 196 / 192.
-constexpr int kWideCtas = 192;
+// N = 3 1: 4.9 / 6.2, 32: 5.3 / 6.2, 64: 6.2 / 6.6; N = 2 64: 4.3 / 4.9, 128:
+// 5.3 / 4.9; N = 4 32: 8.4 / 9.9, 64: 14 / 10; N = 5 4: 9 / 21, 32: 22 / 21;
+// FP64 N = 3 1: 32 / 77, 64: 54 / 77, 128: 106 / 78; N = 4 32: 116 / 186.
+template <int N>
+constexpr int kWideCtas = N <= 3 ? 256 : 160;
+constexpr int kPdlBlocks = 76;  // half the SMs
 template <int N, int OP>
 void launch_op(const StageArgs<real>& a, bool rk, cudaStream_t s) {
-  k_wedge_stage_mma<N, OP><<<a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1, OP>(), s>>>(a, rk);
+  auto kernel = a.m.w_fac == nullptr ? k_wedge_stage<N, 1, true, true, OP> : k_wedge_stage<N, 1, true, false, OP>;
+  kernel<<<a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1, OP>(), s>>>(a, rk);
+}
+// One kernel launch, as a programmatic dependent of the kernel before it on the
+// stream where pdl is set (inside a capture: a programmatic edge).
+template <typename... P>
+cudaError_t launch_dependent(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t s, bool pdl, P... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(grid));
+  cfg.blockDim = dim3(unsigned(block));
+  cfg.dynamicSmemBytes = size_t(smem);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 template <int N>
 int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream_t st, cudaEvent_t ev_fork,
@@ -2647,8 +2436,8 @@ int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream
     if (err != cudaSuccess) return int(err);
   }
   if (a.m.nblk_w > 0) {
-    constexpr int b2 = wedge_bpc_onthefly<N>();
-    const int want = a.wedge_bpc > 0 ? a.wedge_bpc : (a.m.w_fac != nullptr ? 1 : b2);
+    constexpr int b2 = wedge_bpc_multi<N>();
+    const int want = a.wedge_bpc > 0 ? a.wedge_bpc : 1;
     bool done = false;
     if constexpr (sizeof(real) == 4) {
       // the field-pair split kernel (FP32 CUDA-core applies, stored mass
@@ -2666,19 +2455,29 @@ int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream
       else if (a.op == kOpBF16) launch_op<N, kOpBF16>(a, rk, s);
     }
     if constexpr (wide_fits<N>()) {
-      if (!done && a.wedge_bpc <= 1 && a.m.nblk_w * (N + 1) <= kWideCtas) {
-        k_wedge_wide<N><<<a.m.nblk_w * (N + 1), 128, wide_smem_bytes<N>(), s>>>(a, rk);
+      if (!done && a.wedge_bpc <= 1 && a.m.nblk_w * (N + 1) <= kWideCtas<N>) {
+        const cudaError_t err = launch_dependent(k_wedge_wide<N>, a.m.nblk_w * (N + 1), 128, wide_smem_bytes<N>(), s,
+                                                 a.pdl && a.m.nblk_t == 0, a, rk);
+        if (err != cudaSuccess) return int(err);
         done = true;
       }
     }
-    if (done) {
-    } else if ((want == 1 || b2 == 1) && a.tri_far)
-      k_wedge_stage<N, 1, true><<<a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1>(), s>>>(a, rk);
-    else if (want == 1 || b2 == 1)
-      k_wedge_stage<N, 1, false><<<a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1>(), s>>>(a, rk);
-    else  // (two blocks per CTA: the early triangle-face requests measured 402 -> 371 us on 524,288 wedges)
-      k_wedge_stage<N, b2, true><<<(a.m.nblk_w + b2 - 1) / b2, 32 * (N + 1) * b2, wedge_smem_bytes<N, b2>(),
-                                            s>>>(a, rk);
+    if (!done) {
+      // as a programmatic dependent only while both stages' CTAs find SMs of
+      // their own (64 blocks, N = 3: 7.4 -> 6.6 us; 128 and 256 lose by it)
+      const bool otf = a.m.w_fac == nullptr, pdl = a.pdl && a.m.nblk_t == 0 && a.m.nblk_w <= kPdlBlocks;
+      StageArgs<real> b = a;
+      b.pdl = pdl;
+      cudaError_t err = cudaSuccess;
+      if (want == 1 || b2 == 1) {
+        auto kernel = otf ? k_wedge_stage<N, 1, true, true> : a.tri_far ? k_wedge_stage<N, 1, true, false> : k_wedge_stage<N, 1, false, false>;
+        err = launch_dependent(kernel, a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1>(), s, pdl, b, rk);
+      } else {
+        auto kernel = otf ? k_wedge_stage<N, b2, true, true> : k_wedge_stage<N, b2, true, false>;
+        err = launch_dependent(kernel, (a.m.nblk_w + b2 - 1) / b2, 32 * (N + 1) * b2, wedge_smem_bytes<N, b2>(), s, pdl, b, rk);
+      }
+      if (err != cudaSuccess) return int(err);
+    }
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return int(err);
   }
@@ -2773,8 +2572,8 @@ int DGW_CAT(launch_set_clock_, REALNS)(double* clock, double t, void* stream) {
   REALNS::k_set_clock<<<1, 32, 0, cudaStream_t(stream)>>>(clock, t);
   return int(cudaGetLastError());
 }
-int DGW_CAT(launch_clock_, REALNS)(double* clock, double dt, void* stream) {
-  REALNS::k_clock<<<1, 32, 0, cudaStream_t(stream)>>>(clock, dt);
+int DGW_CAT(launch_clock_, REALNS)(const double* from, double* to, double dt, void* stream) {
+  REALNS::k_clock<<<1, 32, 0, cudaStream_t(stream)>>>(from, to, dt);
   return int(cudaGetLastError());
 }
 }  // namespace dgw

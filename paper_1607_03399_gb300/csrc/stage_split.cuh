@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(64 * (N + 1), 2) k_wedge_stage_split(const Sta
   // 5. point sources (pressure, h = 0) and the fused low-storage Runge-Kutta
   //    update (or the plain right-hand side) of this half's two fields
   const real kappa = M.w_mat[0 * Kp + e], irho = M.w_mat[1 * Kp + e];
-  if (src) add_sources(M, 6, e, j * Nt, Np, *M.clock + A.c_stage * double(A.dt), W);
+  if (src) add_sources(M, 6, e, j * Nt, Np, M.clock[A.clk] + A.c_stage * double(A.dt), W);
   const real2 sab = mk2(h == 0 ? kappa : irho, irho);
   if (e < M.Kw) {
 #pragma unroll
