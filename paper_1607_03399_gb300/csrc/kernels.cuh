@@ -10,7 +10,7 @@
 //           + sum_quad M~_e F_e,j                       (lift, weak form)
 //       T_j = - sum_c t_cJ(t_j) (D_t u_c)_j  (p),  - t_cJ(t_j) (D_t p)_j  (u_c)
 //     X_j = (M^{tri,k})^{-1} W_j, M^{tri,k} = sum_a J_a M_a, by a per-element
-//       Cholesky factor computed on the fly (exact inverse of the
+//       L D L^T factor, stored or formed in the stage (exact inverse of the
 //       Jacobian-weighted wedge mass, Section 4.2);
 //     rhs = kappa (-(D_r (r.u) + D_s (s.u))_j + X_p),
 //     rhs_u_c = (1/rho) (-(r_c D_r p + s_c D_s p)_j + X_u_c);
