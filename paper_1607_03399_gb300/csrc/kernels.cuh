@@ -91,7 +91,10 @@ __device__ __forceinline__ Q4 lds4(const real* slab, int node, int lane) {
     return Q4{real(t0.x), real(t0.y), real(t1.x), real(t1.y)};
   }
 }
-// global, read-only for the kernel's lifetime (the stage input)
+// global, read-only for the whole lifetime of the kernel (the non-coherent
+// path).  Not for the stage input of a kernel that may be launched as a
+// programmatic dependent (k_wedge_stage, k_wedge_wide): the stage that writes
+// it may still run when such a kernel starts; they use ld4
 __device__ __forceinline__ Q4 ldg4(const real* __restrict__ q, int64_t idx) {
   if constexpr (sizeof(real) == 4) {
     const float4 t = __ldg(reinterpret_cast<const float4*>(q + idx));
@@ -102,7 +105,8 @@ __device__ __forceinline__ Q4 ldg4(const real* __restrict__ q, int64_t idx) {
     return Q4{real(t0.x), real(t0.y), real(t1.x), real(t1.y)};
   }
 }
-// global, coherent (the residual, rewritten by the same thread)
+// global, coherent (the residual, rewritten by the same thread; the stage
+// input of a programmatic dependent, after pdl_wait)
 __device__ __forceinline__ Q4 ld4(const real* q, int64_t idx) {
   if constexpr (sizeof(real) == 4) {
     const float4 t = *reinterpret_cast<const float4*>(q + idx);
@@ -386,7 +390,8 @@ __device__ __forceinline__ void add_sources(const DevMesh<real>& M, int type, in
 // Programmatic dependent launch (StageArgs::pdl): the stage after this one may
 // be scheduled now; what it does before its own pdl_wait reads mesh tables
 // only.  pdl_wait returns when the stage before this one has completed and its
-// writes are visible (at once in an ordinary launch).
+// writes are visible (at once in an ordinary launch); the state and residual
+// are read after it, with ordinary loads and bulk copies.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -915,7 +920,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
   real* sF = base + SM::F;  // [face][node][lane] pairs (F_p, F_u), then M^tri applied to each
   real* sG = base + SM::G;
   const DevMesh<real>& M = A.m;
-  const real* __restrict__ qin = A.q_in;
+  const real* qin = A.q_in;
   const int lane = threadIdx.x & 31;
   const int blk = blockIdx.x * BPC + sb;
   if (blk >= M.nblk_w) return;  // padding block of the last CTA
@@ -978,7 +983,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
     const int nbe = bnd ? e : qnbr[ed], sh = 5 * (bnd ? 2 * ed : qcode[ed]);
     const real* nb = qin + widx<N>(nbe >> 5, j * Nt, nbe & 31);
 #pragma unroll
-    for (int m = 0; m < Nq; ++m) t[m] = ldg4(nb, int((edge_candidates(N, m) >> sh) & 31u) * (kB * 4));
+    for (int m = 0; m < Nq; ++m) t[m] = ld4(nb, int((edge_candidates(N, m) >> sh) & 31u) * (kB * 4));
   };
   // requested here at N <= 3, after the slab has arrived at N = 4 (before it they
   // cost spills: 649 against 578 us per stage on 524,288 wedges, 600 face by
@@ -1004,7 +1009,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
     if constexpr (TF) {
       const bool ntet = !bnd && (code & kCodeTet) != 0;
       const int node = ntet ? O.tab.tet_face[nf][nk] : (nf ? N * Nt : 0) + nk;
-      return ldg4(qin, ntet ? tidx<N>(M.tet_off, nbe >> 5, node, nbe & 31) : widx<N>(nbe >> 5, node, nbe & 31));
+      return ld4(qin, ntet ? tidx<N>(M.tet_off, nbe >> 5, node, nbe & 31) : widx<N>(nbe >> 5, node, nbe & 31));
     } else {
       return lds4(sq, (nf ? N * Nt : 0) + nk, nbe & 31);
     }
@@ -1411,7 +1416,7 @@ __global__ void __launch_bounds__(128) k_wedge_wide(const StageArgs<real> A, boo
   real* sD = base + SM::D;
   real* sE = base + SM::E;
   const DevMesh<real>& M = A.m;
-  const real* __restrict__ qin = A.q_in;
+  const real* qin = A.q_in;
   const int lane = threadIdx.x & 31, f = threadIdx.x >> 5;
   const int blk = blockIdx.x / Nq, j = blockIdx.x - blk * Nq;
   const int e = blk * kB + lane, Kp = M.Kw_pad;
@@ -1471,7 +1476,7 @@ __global__ void __launch_bounds__(128) k_wedge_wide(const StageArgs<real> A, boo
     const int nbe = bnd ? e : qnbr, sh = 5 * (bnd ? 2 * ed : qcode);
     const real* nb = qin + widx<N>(nbe >> 5, j * Nt, nbe & 31);
 #pragma unroll
-    for (int m = 0; m < Nq; ++m) tv[m] = ldg4(nb, int((edge_candidates(N, m) >> sh) & 31u) * (kB * 4));
+    for (int m = 0; m < Nq; ++m) tv[m] = ld4(nb, int((edge_candidates(N, m) >> sh) & 31u) * (kB * 4));
   }
   constexpr int NTT = (2 * Nt + 3) / 4;
   Q4 tnv[NTT];
@@ -1485,7 +1490,7 @@ __global__ void __launch_bounds__(128) k_wedge_wide(const StageArgs<real> A, boo
     const int nbe = bnd ? e : nbr, nf = bnd ? fb : (code >> 4) & 3;
     const int nk = bnd ? k : O.tab.tri_perm[code & 15][k];
     const int node = ntet ? O.tab.tet_face[nf][nk] : (nf ? N * Nt : 0) + nk;
-    tnv[t] = ldg4(qin, ntet ? tidx<N>(M.tet_off, nbe >> 5, node, nbe & 31) : widx<N>(nbe >> 5, node, nbe & 31));
+    tnv[t] = ld4(qin, ntet ? tidx<N>(M.tet_off, nbe >> 5, node, nbe & 31) : widx<N>(nbe >> 5, node, nbe & 31));
   }
   if (threadIdx.x == 96) *status = (ok && mbar_wait_bounded(&bar[0], 0)) ? 1 : 0;
   if (f == 0 && !stored) factor_wedge<N>(O, M, e, lane, sL);
