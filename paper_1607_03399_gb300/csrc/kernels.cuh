@@ -2402,26 +2402,52 @@ int prepare_n() {
 template <int N>
 constexpr int kWideCtas = N <= 3 ? 256 : 160;
 constexpr int kPdlBlocks = 76;  // half the SMs
-template <int N, int OP>
-void launch_op(const StageArgs<real>& a, bool rk, cudaStream_t s) {
-  auto kernel = a.m.w_fac == nullptr ? k_wedge_stage<N, 1, true, true, OP> : k_wedge_stage<N, 1, true, false, OP>;
-  kernel<<<a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1, OP>(), s>>>(a, rk);
-}
-// One kernel launch, as a programmatic dependent of the kernel before it on the
-// stream where pdl is set (inside a capture: a programmatic edge).
+// Launch attributes of a stage kernel.  dependent: a programmatic dependent of
+// the kernel before it on the stream (inside a capture: a programmatic edge).
+// beside: it runs beside the other element type's stage.  Kernels of different
+// shared-memory carve-outs do not share an SM (its split between L1 and shared
+// memory changes only while it is idle), so both then ask for the largest: left
+// to the default, each takes what its own shared memory and registers suggest,
+// and the two stages queued behind each other on the SMs they met on.  us per
+// stage pair of a step, without / with: 100 + 150 blocks FP64 N = 1 47.1 / 24.4,
+// N = 2 115.5 / 58.8, N = 3 183.1 / 121.1; 64 + 48 blocks FP32 N = 3 10.1 / 7.8;
+// 512 + 768 blocks FP32 N = 1 11.0 / 7.6, N = 3 21.0 / 20.8.  (Of 88 pairs one
+// lost by it, whose CTAs happened to find SMs of their own: 64 + 48 blocks FP64
+// N = 2 33.0 / 38.3.)
+struct LaunchAttrs {
+  cudaLaunchAttribute at[2];
+  unsigned n = 0;
+  LaunchAttrs(bool dependent, bool beside) : at{} {
+    if (dependent) {
+      at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (beside) {
+      at[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+      at[n++].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+    }
+  }
+};
 template <typename... P>
-cudaError_t launch_dependent(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t s, bool pdl, P... args) {
+cudaError_t launch_kernel(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t s, LaunchAttrs attrs, P... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(unsigned(grid));
   cfg.blockDim = dim3(unsigned(block));
   cfg.dynamicSmemBytes = size_t(smem);
   cfg.stream = s;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = pdl ? 1 : 0;
+  cfg.attrs = attrs.at;
+  cfg.numAttrs = attrs.n;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... P>
+cudaError_t launch_dependent(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t s, bool pdl, bool beside,
+                             P... args) {
+  return launch_kernel(kernel, grid, block, smem, s, LaunchAttrs(pdl, beside), args...);
+}
+template <int N, int OP>
+cudaError_t launch_op(const StageArgs<real>& a, bool rk, cudaStream_t s, bool beside) {
+  auto kernel = a.m.w_fac == nullptr ? k_wedge_stage<N, 1, true, true, OP> : k_wedge_stage<N, 1, true, false, OP>;
+  return launch_kernel(kernel, a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1, OP>(), s, LaunchAttrs(false, beside), a, rk);
 }
 template <int N>
 int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream_t st, cudaEvent_t ev_fork,
@@ -2435,8 +2461,7 @@ int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream
     cudaError_t err = cudaEventRecord(ev_fork, s);
     if (err == cudaSuccess) err = cudaStreamWaitEvent(st, ev_fork, 0);
     if (err != cudaSuccess) return int(err);
-    k_tet_stage<N><<<a.m.nblk_t, 128, tet_smem_bytes<N>(), st>>>(a, rk);
-    err = cudaGetLastError();
+    err = launch_kernel(k_tet_stage<N>, a.m.nblk_t, 128, tet_smem_bytes<N>(), st, LaunchAttrs(false, true), a, rk);
     if (err == cudaSuccess) err = cudaEventRecord(ev_join, st);
     if (err != cudaSuccess) return int(err);
   }
@@ -2449,20 +2474,24 @@ int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream
       // factor): when the autotuner or dg_set_launch_variant chose it
       const bool split = a.op == kOpFFMA && a.m.w_fac != nullptr && a.split > 0;
       if (split) {
-        k_wedge_stage_split<N><<<a.m.nblk_w, 64 * (N + 1), split_smem_bytes<N>(), s>>>(a, rk);
+        const cudaError_t err = launch_kernel(k_wedge_stage_split<N>, a.m.nblk_w, 64 * (N + 1), split_smem_bytes<N>(), s,
+                                              LaunchAttrs(false, fork), a, rk);
+        if (err != cudaSuccess) return int(err);
         done = true;
       }
     }
     if constexpr (sizeof(real) == 4 && nt_of(N) <= 16) {
       done = done || a.op != kOpFFMA;
-      if (a.op == kOpTF32x3) launch_op<N, kOpTF32x3>(a, rk, s);
-      else if (a.op == kOpTF32) launch_op<N, kOpTF32>(a, rk, s);
-      else if (a.op == kOpBF16) launch_op<N, kOpBF16>(a, rk, s);
+      cudaError_t err = cudaSuccess;
+      if (a.op == kOpTF32x3) err = launch_op<N, kOpTF32x3>(a, rk, s, fork);
+      else if (a.op == kOpTF32) err = launch_op<N, kOpTF32>(a, rk, s, fork);
+      else if (a.op == kOpBF16) err = launch_op<N, kOpBF16>(a, rk, s, fork);
+      if (err != cudaSuccess) return int(err);
     }
     if constexpr (wide_fits<N>()) {
       if (!done && a.wedge_bpc <= 1 && a.m.nblk_w * (N + 1) <= kWideCtas<N>) {
         const cudaError_t err = launch_dependent(k_wedge_wide<N>, a.m.nblk_w * (N + 1), 128, wide_smem_bytes<N>(), s,
-                                                 a.pdl && a.m.nblk_t == 0, a, rk);
+                                                 a.pdl && a.m.nblk_t == 0, fork, a, rk);
         if (err != cudaSuccess) return int(err);
         done = true;
       }
@@ -2476,10 +2505,11 @@ int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream
       cudaError_t err = cudaSuccess;
       if (want == 1 || b2 == 1) {
         auto kernel = otf ? k_wedge_stage<N, 1, true, true> : a.tri_far ? k_wedge_stage<N, 1, true, false> : k_wedge_stage<N, 1, false, false>;
-        err = launch_dependent(kernel, a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1>(), s, pdl, b, rk);
+        err = launch_dependent(kernel, a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1>(), s, pdl, fork, b, rk);
       } else {
         auto kernel = otf ? k_wedge_stage<N, b2, true, true> : k_wedge_stage<N, b2, true, false>;
-        err = launch_dependent(kernel, (a.m.nblk_w + b2 - 1) / b2, 32 * (N + 1) * b2, wedge_smem_bytes<N, b2>(), s, pdl, b, rk);
+        err = launch_dependent(kernel, (a.m.nblk_w + b2 - 1) / b2, 32 * (N + 1) * b2, wedge_smem_bytes<N, b2>(), s, pdl, fork, b,
+                               rk);
       }
       if (err != cudaSuccess) return int(err);
     }
