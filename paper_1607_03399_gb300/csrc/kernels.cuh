@@ -1773,28 +1773,17 @@ template <int N>
 __host__ __device__ constexpr bool tet_stage_res() {
   return sizeof(real) == 4 && tet_wtab<N>();
 }
-// Whether the lift rows are copied to shared memory with the derivative
-// records: everywhere but FP64 at N = 5, where the whole image would exceed a
-// CTA's shared memory; there the warps read their lift rows (uniform
-// addresses) from global memory.
 template <int N>
 __host__ __device__ constexpr int tet_work_reals() {  // slab, flux pairs, coordinates, normals, (p, -w) table
   return 4 * npt_of(N) * kB + 8 * nt_of(N) * kB + 24 * kB + (tet_wtab<N>() ? 4 * npt_of(N) * kB : 0);
-}
-template <int N>
-__host__ __device__ constexpr bool tet_lift_smem() {
-  return 128 + (tet_ops_image_reals<N>() + tet_work_reals<N>()) * int(sizeof(real)) <= 227 * 1024;
-}
-template <int N>
-__host__ __device__ constexpr int tet_ops_reals() {  // the part of the image in shared memory
-  return tet_lift_smem<N>() ? tet_ops_image_reals<N>() : tet_drecs<N>();
 }
 // 128-byte header (4 mbarriers), operators, slab [Np][32][4], flux pairs
 // [4 faces][Nt][32][2], vertex coordinates [12][32], normals [4][3][32], (p, -w) [Np][32][4]
 template <int N>
 __host__ __device__ constexpr int tet_smem_bytes() {
-  return 128 + (tet_ops_reals<N>() + tet_work_reals<N>()) * int(sizeof(real));
+  return 128 + (tet_ops_image_reals<N>() + tet_work_reals<N>()) * int(sizeof(real));
 }
+static_assert(tet_smem_bytes<NORD>() <= 227 * 1024, "the whole operator image fits a CTA at every order and precision");
 // acc.x += a.x b, acc.y += a.y b; FP64 leaves out the second where it is padding
 template <bool PAD>
 __device__ __forceinline__ real2 fma_pair(const real2 a, real b, const real2 acc) {
@@ -1811,7 +1800,7 @@ __global__ void __launch_bounds__(128, (sizeof(REAL) == 4) ? (N >= 4 ? 3 : 5) : 
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);  // [0] operators, [1] coordinates, [2] state, [3] residual
   real* sOp = reinterpret_cast<real*>(smem_raw + 128);
   real* sL = sOp + tet_drecs<N>();  // lift [warp][4 Nt][LS]
-  real* sq = sOp + tet_ops_reals<N>();
+  real* sq = sOp + tet_ops_image_reals<N>();
   real* sF = sq + 4 * Np * kB;
   real* sX = sF + 8 * Nt * kB;
   real* sN = sX + 12 * kB;
@@ -1825,7 +1814,7 @@ __global__ void __launch_bounds__(128, (sizeof(REAL) == 4) ? (N >= 4 ? 3 : 5) : 
   const int e = blk * kB + lane;
   const int Kp = M.Kt_pad;
   constexpr uint32_t slab_bytes = uint32_t(4 * Np * kB * sizeof(real)), xyz_bytes = uint32_t(12 * kB * sizeof(real));
-  constexpr uint32_t ops_bytes = uint32_t(tet_ops_reals<N>() * sizeof(real));
+  constexpr uint32_t ops_bytes = uint32_t(tet_ops_image_reals<N>() * sizeof(real));
   if (threadIdx.x == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
@@ -2012,9 +2001,9 @@ __global__ void __launch_bounds__(128, (sizeof(REAL) == 4) ? (N >= 4 ? 3 : 5) : 
       bulk_g2s(sW, A.res + M.tet_off + int64_t(blk) * 4 * Np * kB, slab_bytes, &bar[3]);
     }
   }
-  // the lift of the four faces: this warp's records [4 Nt][LS] (shared memory, or the global image)
+  // the lift of the four faces: this warp's records [4 Nt][LS]
   {
-    const real* lw = (tet_lift_smem<N>() ? sL : M.t_ops + tet_drecs<N>()) + w * (4 * Nt) * LS;
+    const real* lw = sL + w * (4 * Nt) * LS;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       real2 lu[CH];
