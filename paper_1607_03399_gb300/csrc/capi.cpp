@@ -283,8 +283,8 @@ void fill_ops(const RefElems& R, std::vector<unsigned char>& out) {
   pairs(o.w.Mea, Nq, Nq, o.w.MeaP);
   pairs(o.w.Meb, Nq, Nq, o.w.MebP);
   for (int a = 0; a < 3; ++a) pairs(o.w.Ma[a], Nt, Nt, o.w.MaP[a]);
-  if (NN >= 4) {
-    using W = WedgeOps<NN, real>;
+  using W = WedgeOps<NN, real>;
+  if constexpr (W::by_input) {
     auto by_input = [&](const real* XP, real* XT) {
       for (int l = 0; l < Nt; ++l)
         for (int h = 0; h < W::Nh; ++h)

@@ -54,8 +54,9 @@ struct WedgeOps {
   alignas(16) real MebP[Nqh * Nq * 2];
   alignas(16) real MaP[3][Nh * Nt * 2];
   // and by input node, entry (l, h) of XT the same pair at XT[(l * Nhp + h) * 2]
-  // (N >= 4: the stage loops over the input nodes)
-  static constexpr int Nhp = (Nh + 1) / 2 * 2, Nlt = N >= 4 ? Nt : 1;
+  // (where the stage loops over the input nodes: FP32, N >= 4)
+  static constexpr bool by_input = sizeof(real) == 4 && N >= 4;
+  static constexpr int Nhp = (Nh + 1) / 2 * 2, Nlt = by_input ? Nt : 1;
   alignas(16) real MT[Nlt * Nhp * 2];
   alignas(16) real DrT[Nlt * Nhp * 2];
   alignas(16) real DsT[Nlt * Nhp * 2];

@@ -904,7 +904,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
   // N = 5, half of its constant loads: N = 4 622 -> 600 us per stage on 524,288
   // wedges, N = 5 613 -> 438 us on 131,072.  (FP64 waits on its pipe and gains
   // more from leaving out the zeros of D_s: N = 4 1,295 against 1,360 us.)
-  constexpr bool rolled = sizeof(real) == 4 && N >= 4;
+  constexpr bool rolled = WedgeOps<N, real>::by_input;
   constexpr int NHP = (NH + 1) / 2 * 2;
   static_assert(OP == kOpFFMA || (sizeof(real) == 4 && BPC == 1 && Nt <= 16), "tensor-core applies: FP32, Nt <= 16");
   using SM = WedgeSmem<N, OP>;
