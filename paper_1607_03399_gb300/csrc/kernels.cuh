@@ -45,22 +45,6 @@ __host__ __device__ constexpr int tri_idx(int N, int a, int b) { return b * (N +
 __host__ __device__ constexpr int edge_node(int N, int ed, int m) {
   return ed == 0 ? tri_idx(N, m, 0) : (ed == 1 ? tri_idx(N, N - m, m) : tri_idx(N, 0, N - m));
 }
-// k-th node of tet face f in element node order
-__host__ __device__ constexpr int tet_face_node(int N, int f, int k) {
-  int n = 0, cnt = 0;
-  for (int c = 0; c <= N; ++c)
-    for (int b = 0; b <= N - c; ++b)
-      for (int a = 0; a <= N - b - c; ++a) {
-        const bool on = (f == 0) ? (c == 0) : (f == 1) ? (b == 0) : (f == 2) ? (a + b + c == N) : (a == 0);
-        if (on) {
-          if (cnt == k) return n;
-          ++cnt;
-        }
-        ++n;
-      }
-  return -1;
-}
-
 // Packed state layout: node-major, the four fields innermost, so one thread
 // moves a node's (p, u_x, u_y, u_z) with one 16-byte (FP32) access and a warp
 // moves 512 contiguous bytes:
@@ -79,7 +63,6 @@ __device__ __forceinline__ int64_t tidx(int64_t off, int blk_e, int node, int la
 struct Q4 {
   real p, u, v, w;
 };
-__device__ __forceinline__ Q4 q4_from(const float4 t) { return Q4{real(t.x), real(t.y), real(t.z), real(t.w)}; }
 // shared-memory slab [Np][32][4]
 __device__ __forceinline__ Q4 lds4(const real* slab, int node, int lane) {
   const real* a = slab + ((node * kB + lane) << 2);
@@ -116,16 +99,6 @@ __device__ __forceinline__ Q4 ld4(const real* q, int64_t idx) {
     return Q4{real(t0.x), real(t0.y), real(t1.x), real(t1.y)};
   }
 }
-// generic address: the block's slab in shared memory or the stage input in global memory
-__device__ __forceinline__ Q4 ldx4(const real* a) {
-  if constexpr (sizeof(real) == 4) {
-    const float4 t = *reinterpret_cast<const float4*>(a);
-    return Q4{real(t.x), real(t.y), real(t.z), real(t.w)};
-  } else {
-    const double2 t0 = reinterpret_cast<const double2*>(a)[0], t1 = reinterpret_cast<const double2*>(a)[1];
-    return Q4{real(t0.x), real(t0.y), real(t1.x), real(t1.y)};
-  }
-}
 // shared-memory operator records: (a, b, c, d) in natural order -> Q4{a, b, c, d}
 __device__ __forceinline__ Q4 ldop4(const real* a) {
   if constexpr (sizeof(real) == 4) {
@@ -134,17 +107,6 @@ __device__ __forceinline__ Q4 ldop4(const real* a) {
   } else {
     const double2 t0 = reinterpret_cast<const double2*>(a)[0], t1 = reinterpret_cast<const double2*>(a)[1];
     return Q4{real(t0.x), real(t0.y), real(t1.x), real(t1.y)};
-  }
-}
-__device__ __forceinline__ void ldop2(const real* a, real& x, real& y) {
-  if constexpr (sizeof(real) == 4) {
-    const float2 t = *reinterpret_cast<const float2*>(a);
-    x = real(t.x);
-    y = real(t.y);
-  } else {
-    const double2 t = *reinterpret_cast<const double2*>(a);
-    x = real(t.x);
-    y = real(t.y);
   }
 }
 __device__ __forceinline__ void st4(real* q, int64_t idx, const Q4& v) {
@@ -416,9 +378,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) { return uint32_t(__
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
-__device__ __forceinline__ void mbar_inval(uint64_t* bar) {
-  asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 __device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
@@ -486,7 +445,7 @@ enum WGeo : int {
 // tiles (Nq x Nt x 128 reals, the size of the residual slab) share the
 // residual slab's space: the residual is copied in once the weak-form
 // accumulation has released them.
-template <int N, int OP = kOpFFMA>
+template <int N>
 __host__ __device__ constexpr bool stage_res() {
   return sizeof(real) == 4 ? N <= 4 : N <= 3;
 }
@@ -496,12 +455,12 @@ struct WedgeSmem {
   static constexpr int Nt = nt_of(N), Nq = N + 1, Np = Nt * Nq;
   static constexpr int q = 0;                                            // [4][Np][32]
   static constexpr int r = q + 4 * Np * kB;                              // [4][Np][32] (if staged)
-  static constexpr int L = r + (stage_res<N, OP>() ? 4 * Np * kB : 0);   // [NL4][32][4]
+  static constexpr int L = r + (stage_res<N>() ? 4 * Np * kB : 0);       // [NL4][32][4]
   static constexpr int F = L + nl4_of(N) * 4 * kB;                        // [4][Nt][32]
   static constexpr int G = F + 4 * Nt * kB;                              // [G_STAGE][32]
-  // per-warp operand tiles [Nt][kTP] (tensor cores): the residual slab's space where it is staged
-  static constexpr int T = stage_res<N, OP>() ? r : G + G_STAGE * kB;
-  static constexpr int reals = G + G_STAGE * kB + ((OP == kOpFFMA || stage_res<N, OP>()) ? 0 : Nq * Nt * kTP);
+  static constexpr int T = r;  // per-warp operand tiles [Nt][kTP] (tensor cores): the residual slab's space
+  static constexpr int reals = G + G_STAGE * kB;
+  static_assert(OP == kOpFFMA || (stage_res<N>() && Nq * Nt * kTP <= 4 * Np * kB), "the tiles fit the residual slab's space");
 };
 
 template <int N, int OP = kOpFFMA>
@@ -523,6 +482,7 @@ template <int N, int BPC, int OP = kOpFFMA>
 __host__ __device__ constexpr int wedge_smem_bytes() {
   return BPC * (32 + wedge_smem_reals<N, OP>() * int(sizeof(real)));
 }
+constexpr int kHalfSMs = 76;  // half of the 152 SMs
 // resident CTAs per SM the stage is compiled for
 template <int N, int BPC, int OP>
 __host__ __device__ constexpr int wedge_min_ctas() {
@@ -931,7 +891,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
   const int e = blk * kB + lane;
   const int Kp = M.Kw_pad;
   constexpr uint32_t slab_bytes = uint32_t(4 * Np * kB * sizeof(real));
-  const bool res_async = rk && stage_res<N, OP>() && A.rk_a != real(0);
+  const bool res_async = rk && stage_res<N>() && A.rk_a != real(0);
 #define GEO(item) sG[(item) * kB + lane]
   // the warps of one block synchronise among themselves (named barrier 1 + sb)
   auto block_sync = [&]() {
@@ -969,7 +929,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(A.res + int64_t(blk) * 4 * Np * kB), "r"(slab_bytes));
     }
   }
-  if (j == N) prefetch_ahead<N>(M, qin, blk + 76 * wedge_min_ctas<N, BPC, OP>() * BPC, lane, N <= 4 && stored);
+  if (j == N) prefetch_ahead<N>(M, qin, blk + kHalfSMs * wedge_min_ctas<N, BPC, OP>() * BPC, lane, N <= 4 && stored);
   // face neighbours, their impedances and the source flag, loaded while the
   // slabs are in flight; so are (N <= 3) the neighbour traces
   const real kappa = M.w_mat[0 * Kp + e], irho = M.w_mat[1 * Kp + e], zM = M.w_mat[2 * Kp + e];
@@ -1149,22 +1109,22 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
   //    + A D_t u_z) and D_t p; W_p += M^tri dd, Mdp = M^tri D_t p
   const real tj = O.w.gll[j];
   const real ntx = -fmar(tj, GEO(G_TX1), GEO(G_TX0)), nty = -fmar(tj, GEO(G_TY1), GEO(G_TY0)), nA = -GEO(G_A);
-      real dtr[Nq];
+  real dtr[Nq];
 #pragma unroll
-      for (int m = 0; m < Nq; ++m) dtr[m] = O.w.Dt[j * Nq + m];
-      // node i: D_t of the four fields as two packed pairs (p, u_x) and (u_y, u_z)
-      auto t_part = [&](int i, real& dp, real& dd) {
-        real2 dpu = dup2(real(0)), dvw = dup2(real(0));
+  for (int m = 0; m < Nq; ++m) dtr[m] = O.w.Dt[j * Nq + m];
+  // node i: D_t of the four fields as two packed pairs (p, u_x) and (u_y, u_z)
+  auto t_part = [&](int i, real& dp, real& dd) {
+    real2 dpu = dup2(real(0)), dvw = dup2(real(0));
 #pragma unroll
-        for (int m = 0; m < Nq; ++m) {
-          const Q4 v = lds4(sq, m * Nt + i, lane);
-          const real2 d2 = dup2(dtr[m]);
-          dpu = fma2(d2, mk2(v.p, v.u), dpu);
-          dvw = fma2(d2, mk2(v.v, v.w), dvw);
-        }
-        dp = dpu.x;
-        dd = fmar(ntx, dpu.y, fmar(nty, dvw.x, nA * dvw.y));
-      };
+    for (int m = 0; m < Nq; ++m) {
+      const Q4 v = lds4(sq, m * Nt + i, lane);
+      const real2 d2 = dup2(dtr[m]);
+      dpu = fma2(d2, mk2(v.p, v.u), dpu);
+      dvw = fma2(d2, mk2(v.v, v.w), dvw);
+    }
+    dp = dpu.x;
+    dd = fmar(ntx, dpu.y, fmar(nty, dvw.x, nA * dvw.y));
+  };
   real2 W01[Nt], W23[Nt];
   // the coefficients of the four right-hand sides, and node i's values from the
   // flux pairs, the pressure's (a) and D_t p's (d) part
@@ -1350,7 +1310,7 @@ __global__ void __launch_bounds__(32 * (N + 1) * BPC, wedge_min_ctas<N, BPC, OP>
     return;
   }
   if (src) add_sources(M, 6, e, j * Nt, Np, M.clock[A.clk] + A.c_stage * double(A.dt), W01);
-  wedge_update<N, stage_res<N, OP>()>(A, rk, sq, sr, blk, j, lane, e, kappa, irho, W01, W23);
+  wedge_update<N, stage_res<N>()>(A, rk, sq, sr, blk, j, lane, e, kappa, irho, W01, W23);
 #undef GEO
 }
 
@@ -2394,7 +2354,7 @@ int prepare_n() {
 // FP64 N = 3 1: 32 / 77, 64: 54 / 77, 128: 106 / 78; N = 4 32: 116 / 186.
 template <int N>
 constexpr int kWideCtas = N <= 3 ? 256 : 160;
-constexpr int kPdlBlocks = 76;  // half the SMs
+constexpr int kPdlBlocks = kHalfSMs;
 // Launch attributes of a stage kernel.  dependent: a programmatic dependent of
 // the kernel before it on the stream (inside a capture: a programmatic edge).
 // beside: it runs beside the other element type's stage.  Kernels of different
