@@ -156,9 +156,12 @@ __global__ void __launch_bounds__(32 * (N + 1), (sizeof(real) == 4) ? (N <= 3 ? 
     }
     return;
   }
-  // (by one warp: split over the warps it measured no faster, with more spills)
+  // (by one warp, its six parts interleaved: one after the other they add their
+  // latencies, 0.5 us of a small mesh's launch, us per reverse stage of 128 wedges
+  // N = 1 5.9 -> 5.4, N = 3 9.4 -> 8.9 and of 110,592 N = 3 142.2 -> 138.9; split
+  // over the warps it costs spills at N = 3, 144.8)
   if (j == 0) {
-#pragma unroll 1
+#pragma unroll
     for (int p = 0; p < kGeoParts; ++p) wedge_geometry_part<true>(p, sC, sG, lane);
   }
   __syncthreads();
