@@ -792,6 +792,7 @@ struct StageExtra {
   void* rhs_out = nullptr;
   bool no_sources = false;
   bool res_store = true;
+  bool reverse = false; // a stage of the reverse sweep: gradient kernels run beside it
   bool pdl = false;     // the stage before it on the stream is the only work it waits for
 };
 
@@ -820,6 +821,7 @@ int launch_stage(dg_ctx* c, const void* q_in, void* q_out, void* res, double a, 
     A.res_store = x.res_store ? 1 : 0;
     A.clk = c->cur;
     A.pdl = x.pdl ? 1 : 0;
+    A.reverse = x.reverse ? 1 : 0;
     A.rhs_out = static_cast<double*>(x.rhs_out);
     if (x.no_sources) A.m.nsrc = 0;
     rc = stage_f64(c->N, A, rk, s, c->tet_stream, c->ev_fork, c->ev_join);
@@ -844,6 +846,7 @@ int launch_stage(dg_ctx* c, const void* q_in, void* q_out, void* res, double a, 
     A.res_store = x.res_store ? 1 : 0;
     A.clk = c->cur;
     A.pdl = x.pdl ? 1 : 0;
+    A.reverse = x.reverse ? 1 : 0;
     A.rhs_out = static_cast<float*>(x.rhs_out);
     if (x.no_sources) A.m.nsrc = 0;
     rc = stage_f32(c->N, A, rk, s, c->tet_stream, c->ev_fork, c->ev_join);
@@ -1975,6 +1978,7 @@ int adjoint_reverse_stages(dg_ctx* c, double dt, const void* const* Q, const voi
     StageExtra x;
     x.g = kLSRK_A[st];
     x.no_sources = true;
+    x.reverse = gs != c->stream;
     rc = launch_stage(c, xin, xout, adj_field(c, kAdjMuq), 1.0, kLSRK_B[(st + 4) % 5], dt, true, c->stream, 0.0, x);
     if (gs != c->stream) {
       cudaError_t e = cudaEventRecord(c->ev_gjoin, gs);

@@ -168,6 +168,7 @@ struct StageArgs {
   int op = 0;                   // kOpFFMA, or a tensor-core variant (FP32 fields)
   int split = 0;                // wedge stage split over field pairs: 1 yes, otherwise no
   int tri_far = 0;              // some wedge's triangle-face neighbour is a tet or in another block
+  int reverse = 0;              // a stage of the reverse sweep: gradient kernels run beside it
 };
 
 enum : int { kErrTimeout = 1, kErrNonfinite = 2 };

@@ -2355,14 +2355,20 @@ int prepare_n() {
 template <int N>
 constexpr int kWideCtas = N <= 3 ? 256 : 160;
 constexpr int kPdlBlocks = kHalfSMs;
+// Whether the wedge part of a stage takes the small-mesh form.
+template <int N>
+bool small_mesh_form(int nblk_w) {
+  return wide_fits<N>() && nblk_w * (N + 1) <= kWideCtas<N>;
+}
 // Launch attributes of a stage kernel.  dependent: a programmatic dependent of
 // the kernel before it on the stream (inside a capture: a programmatic edge).
-// beside: it runs beside the other element type's stage.  Kernels of different
-// shared-memory carve-outs do not share an SM (its split between L1 and shared
-// memory changes only while it is idle), so both then ask for the largest: left
-// to the default, each takes what its own shared memory and registers suggest,
-// and the two stages queued behind each other on the SMs they met on.  us per
-// stage pair of a step, without / with: 100 + 150 blocks FP64 N = 1 47.1 / 24.4,
+// carve: the part of an SM's memory to be shared memory, in per cent, or 0 for
+// the default, which follows from the kernel's own shared memory and registers.
+// Kernels of different carve-outs do not share an SM (its split between L1 and
+// shared memory changes only while it is idle): left to the default, two that
+// run on two streams queue behind each other on the SMs they meet on, so they
+// are given the same.  The two element types' stages ask for all of it: us per
+// stage pair of a step, default / all: 100 + 150 blocks FP64 N = 1 47.1 / 24.4,
 // N = 2 115.5 / 58.8, N = 3 183.1 / 121.1; 64 + 48 blocks FP32 N = 3 10.1 / 7.8;
 // 512 + 768 blocks FP32 N = 1 11.0 / 7.6, N = 3 21.0 / 20.8.  (Of 88 pairs one
 // lost by it, whose CTAs happened to find SMs of their own: 64 + 48 blocks FP64
@@ -2370,17 +2376,36 @@ constexpr int kPdlBlocks = kHalfSMs;
 struct LaunchAttrs {
   cudaLaunchAttribute at[2];
   unsigned n = 0;
-  LaunchAttrs(bool dependent, bool beside) : at{} {
+  LaunchAttrs(bool dependent, int carve) : at{} {
     if (dependent) {
       at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
       at[n++].val.programmaticStreamSerializationAllowed = 1;
     }
-    if (beside) {
+    if (carve > 0) {
       at[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-      at[n++].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+      at[n++].val.sharedMemCarveout = unsigned(carve);
     }
   }
 };
+constexpr int kCarveAll = cudaSharedmemCarveoutMaxShared;
+// The carve-out of the reverse sweep's kernels, a stage beside its gradient
+// kernel.  us per reverse stage, default / this: FP64 N = 2, 128 wedge blocks 149.2 /
+// 54.2 and 108 tet blocks 65.2 / 39.6; FP32 N = 1, 512 wedge blocks 12.7 / 7.0.
+// FP32 without tets, no more CTAs than SMs: room for one CTA of each, as the
+// gradient kernel's gathers and spills live in the L1 that is left (N = 4, 72
+// blocks default 18.3, all 18.1, this 15.3).  FP32 with tets: the default, where
+// all costs more than it gives (N = 3, 108 tet blocks 9.4 / 11.0).  What lost: FP64
+// N = 3, 200 wedge blocks 215 / 247.
+template <int N>
+int reverse_carve(const DevMesh<real>& m) {
+  if (sizeof(real) == 8) return kCarveAll;
+  if (m.nblk_t > 0) return 0;
+  const bool small = small_mesh_form<N>(m.nblk_w);
+  if ((small ? m.nblk_w * (N + 1) : m.nblk_w) > 2 * kHalfSMs) return kCarveAll;
+  const int stage = small ? wide_smem_bytes<N>() : wedge_smem_bytes<N, 1>();
+  const int bytes = stage + grad_smem_bytes<N>() + 2 * 1024, sm = 228 * 1024;  // (1 KB per CTA is the system's)
+  return bytes < sm ? int((100ll * bytes + sm - 1) / sm) : kCarveAll;
+}
 template <typename... P>
 cudaError_t launch_kernel(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t s, LaunchAttrs attrs, P... args) {
   cudaLaunchConfig_t cfg{};
@@ -2390,17 +2415,18 @@ cudaError_t launch_kernel(void (*kernel)(P...), int grid, int block, int smem, c
   cfg.stream = s;
   cfg.attrs = attrs.at;
   cfg.numAttrs = attrs.n;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
+  cudaLaunchKernelEx(&cfg, kernel, args...);
+  return cudaGetLastError();
 }
 template <typename... P>
-cudaError_t launch_dependent(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t s, bool pdl, bool beside,
+cudaError_t launch_dependent(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t s, bool pdl, int carve,
                              P... args) {
-  return launch_kernel(kernel, grid, block, smem, s, LaunchAttrs(pdl, beside), args...);
+  return launch_kernel(kernel, grid, block, smem, s, LaunchAttrs(pdl, carve), args...);
 }
 template <int N, int OP>
-cudaError_t launch_op(const StageArgs<real>& a, bool rk, cudaStream_t s, bool beside) {
+cudaError_t launch_op(const StageArgs<real>& a, bool rk, cudaStream_t s, int carve) {
   auto kernel = a.m.w_fac == nullptr ? k_wedge_stage<N, 1, true, true, OP> : k_wedge_stage<N, 1, true, false, OP>;
-  return launch_kernel(kernel, a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1, OP>(), s, LaunchAttrs(false, beside), a, rk);
+  return launch_kernel(kernel, a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1, OP>(), s, LaunchAttrs(false, carve), a, rk);
 }
 template <int N>
 int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream_t st, cudaEvent_t ev_fork,
@@ -2410,11 +2436,12 @@ int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream
   // it, forked from and joined back into s (also inside a graph capture), so
   // the two kernels share the GPU instead of running back to back
   const bool fork = a.m.nblk_w > 0 && a.m.nblk_t > 0 && st != nullptr && ev_fork != nullptr && ev_join != nullptr;
+  const int carve = fork ? kCarveAll : (a.reverse ? reverse_carve<N>(a.m) : 0);
   if (fork) {
     cudaError_t err = cudaEventRecord(ev_fork, s);
     if (err == cudaSuccess) err = cudaStreamWaitEvent(st, ev_fork, 0);
     if (err != cudaSuccess) return int(err);
-    err = launch_kernel(k_tet_stage<N>, a.m.nblk_t, 128, tet_smem_bytes<N>(), st, LaunchAttrs(false, true), a, rk);
+    err = launch_kernel(k_tet_stage<N>, a.m.nblk_t, 128, tet_smem_bytes<N>(), st, LaunchAttrs(false, carve), a, rk);
     if (err == cudaSuccess) err = cudaEventRecord(ev_join, st);
     if (err != cudaSuccess) return int(err);
   }
@@ -2428,7 +2455,7 @@ int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream
       const bool split = a.op == kOpFFMA && a.m.w_fac != nullptr && a.split > 0;
       if (split) {
         const cudaError_t err = launch_kernel(k_wedge_stage_split<N>, a.m.nblk_w, 64 * (N + 1), split_smem_bytes<N>(), s,
-                                              LaunchAttrs(false, fork), a, rk);
+                                              LaunchAttrs(false, carve), a, rk);
         if (err != cudaSuccess) return int(err);
         done = true;
       }
@@ -2436,15 +2463,15 @@ int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream
     if constexpr (sizeof(real) == 4 && nt_of(N) <= 16) {
       done = done || a.op != kOpFFMA;
       cudaError_t err = cudaSuccess;
-      if (a.op == kOpTF32x3) err = launch_op<N, kOpTF32x3>(a, rk, s, fork);
-      else if (a.op == kOpTF32) err = launch_op<N, kOpTF32>(a, rk, s, fork);
-      else if (a.op == kOpBF16) err = launch_op<N, kOpBF16>(a, rk, s, fork);
+      if (a.op == kOpTF32x3) err = launch_op<N, kOpTF32x3>(a, rk, s, carve);
+      else if (a.op == kOpTF32) err = launch_op<N, kOpTF32>(a, rk, s, carve);
+      else if (a.op == kOpBF16) err = launch_op<N, kOpBF16>(a, rk, s, carve);
       if (err != cudaSuccess) return int(err);
     }
     if constexpr (wide_fits<N>()) {
-      if (!done && a.wedge_bpc <= 1 && a.m.nblk_w * (N + 1) <= kWideCtas<N>) {
+      if (!done && a.wedge_bpc <= 1 && small_mesh_form<N>(a.m.nblk_w)) {
         const cudaError_t err = launch_dependent(k_wedge_wide<N>, a.m.nblk_w * (N + 1), 128, wide_smem_bytes<N>(), s,
-                                                 a.pdl && a.m.nblk_t == 0, fork, a, rk);
+                                                 a.pdl && a.m.nblk_t == 0, carve, a, rk);
         if (err != cudaSuccess) return int(err);
         done = true;
       }
@@ -2458,10 +2485,10 @@ int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream
       cudaError_t err = cudaSuccess;
       if (want == 1 || b2 == 1) {
         auto kernel = otf ? k_wedge_stage<N, 1, true, true> : a.tri_far ? k_wedge_stage<N, 1, true, false> : k_wedge_stage<N, 1, false, false>;
-        err = launch_dependent(kernel, a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1>(), s, pdl, fork, b, rk);
+        err = launch_dependent(kernel, a.m.nblk_w, 32 * (N + 1), wedge_smem_bytes<N, 1>(), s, pdl, carve, b, rk);
       } else {
         auto kernel = otf ? k_wedge_stage<N, b2, true, true> : k_wedge_stage<N, b2, true, false>;
-        err = launch_dependent(kernel, (a.m.nblk_w + b2 - 1) / b2, 32 * (N + 1) * b2, wedge_smem_bytes<N, b2>(), s, pdl, fork, b,
+        err = launch_dependent(kernel, (a.m.nblk_w + b2 - 1) / b2, 32 * (N + 1) * b2, wedge_smem_bytes<N, b2>(), s, pdl, carve, b,
                                rk);
       }
       if (err != cudaSuccess) return int(err);
@@ -2470,11 +2497,8 @@ int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream
     if (err != cudaSuccess) return int(err);
   }
   if (fork) return int(cudaStreamWaitEvent(s, ev_join, 0));
-  if (a.m.nblk_t > 0) {
-    k_tet_stage<N><<<a.m.nblk_t, 128, tet_smem_bytes<N>(), s>>>(a, rk);
-    cudaError_t err = cudaGetLastError();
-    if (err != cudaSuccess) return int(err);
-  }
+  if (a.m.nblk_t > 0)
+    return int(launch_kernel(k_tet_stage<N>, a.m.nblk_t, 128, tet_smem_bytes<N>(), s, LaunchAttrs(false, carve), a, rk));
   return 0;
 }
 
@@ -2535,22 +2559,20 @@ int DGW_CAT(launch_grad_, REALNS)(const DevMesh<REAL>& m, const REAL* x, const R
   if (m.nblk_w > 0) {
     constexpr int bytes = REALNS::grad_smem_bytes<NORD>();
     if (bytes > 227 * 1024) return int(cudaErrorInvalidConfiguration);
-    if (m.nblk_t > 0)
-      REALNS::k_wedge_grad<NORD, true><<<m.nblk_w, 32 * (NORD + 1), bytes, cudaStream_t(stream)>>>(m, x, q, r, dt, flux,
-                                                                                                  bc, gk, gr, gz);
-    else
-      REALNS::k_wedge_grad<NORD, false><<<m.nblk_w, 32 * (NORD + 1), bytes, cudaStream_t(stream)>>>(m, x, q, r, dt, flux,
-                                                                                                   bc, gk, gr, gz);
+    auto kernel = m.nblk_t > 0 ? REALNS::k_wedge_grad<NORD, true> : REALNS::k_wedge_grad<NORD, false>;
+    return int(REALNS::launch_kernel(kernel, m.nblk_w, 32 * (NORD + 1), bytes, cudaStream_t(stream),
+                                     REALNS::LaunchAttrs(false, REALNS::reverse_carve<NORD>(m)), m, x, q, r, dt, flux, bc, gk, gr, gz));
   }
-  return int(cudaGetLastError());
+  return 0;
 }
 int DGW_CAT(launch_tgrad_, REALNS)(const DevMesh<REAL>& m, const REAL* x, const REAL* q, const REAL* r, double dt,
                                    int flux, int bc, double* gk, double* gr, void* stream) {
   if (m.nblk_t > 0) {
     constexpr int bytes = REALNS::tgrad_smem_bytes<NORD>();
-    REALNS::k_tet_grad<NORD><<<m.nblk_t, 128, bytes, cudaStream_t(stream)>>>(m, x, q, r, dt, flux, bc, gk, gr);
+    return int(REALNS::launch_kernel(REALNS::k_tet_grad<NORD>, m.nblk_t, 128, bytes, cudaStream_t(stream),
+                                     REALNS::LaunchAttrs(false, REALNS::reverse_carve<NORD>(m)), m, x, q, r, dt, flux, bc, gk, gr));
   }
-  return int(cudaGetLastError());
+  return 0;
 }
 int DGW_CAT(launch_wait_expire_, REALNS)(int* err, void* stream) {
   REALNS::k_wait_expire<<<1, 32, 0, cudaStream_t(stream)>>>(err);

@@ -38,3 +38,35 @@ def test_stage_pair_takes_no_longer_than_its_stages(N):
         pair.append(1e3 * e0.elapsed_time(e1) / 40)
     S.close()
     assert min(pair) <= 1.15 * alone, (min(pair), alone)
+
+
+def _reverse_step_us(side, layers, N):
+    """Device microseconds of a recorded reverse step, FP64."""
+    m = I.bumpy_layered_mesh(side, layers)
+    S = Solver(m.VX, m.EToV, m.etype, N, precision="f64")
+    S.set_fields(I.random_fields(S.total_nodes, 1))
+    dt = S.stable_dt(0.3)
+    S.adjoint_bind()
+    S.adjoint_reset()
+    rec = S.new_record()
+    S.step_record(dt, rec)
+    times = []
+    for _ in range(6):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record(S.stream)
+        for _ in range(4):
+            S.adjoint_step_recorded(dt, rec)
+        e1.record(S.stream)
+        e1.synchronize()
+        times.append(1e3 * e0.elapsed_time(e1) / 4)
+    S.close()
+    return min(times)
+
+
+def test_reverse_stages_share_the_gpu_with_their_gradient_kernels():
+    """A reverse step of 128 blocks takes no longer, per block, than one of 72:
+    on neither mesh do the gradient kernels and the stages fill the GPU.  (Where
+    they queue behind each other, the 128 blocks take 3 times as long as the 72
+    instead of 1.2 times.)"""
+    small, large = _reverse_step_us(12, 8, 2), _reverse_step_us(16, 8, 2)
+    assert large <= small * 128 / 72, (small, large)
