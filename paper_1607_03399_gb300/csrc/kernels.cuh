@@ -2355,10 +2355,16 @@ int prepare_n() {
 template <int N>
 constexpr int kWideCtas = N <= 3 ? 256 : 160;
 constexpr int kPdlBlocks = kHalfSMs;
-// Whether the wedge part of a stage takes the small-mesh form.
+// Whether the wedge part of a stage takes the small-mesh form.  In FP32 at
+// N >= 3 a stage that runs beside other kernels (beside) takes it only up to one
+// CTA per SM: past that it gains little by itself, and its N + 1 times as many
+// CTAs hold the SMs that the other kernels need.  us, up to kWideCtas / so: reverse
+// stage N = 3, 64 blocks 11.3 / 9.7, N = 4, 32 blocks 18.1 / 14.2, 64 + 96 blocks N = 3
+// 26.6 / 23.2; stage pair N = 4, 32 + 192 blocks 15.5 / 14.2, N = 3, 64 + 192 9.4 / 8.8.
 template <int N>
-bool small_mesh_form(int nblk_w) {
-  return wide_fits<N>() && nblk_w * (N + 1) <= kWideCtas<N>;
+bool small_mesh_form(int nblk_w, bool beside) {
+  const int limit = sizeof(real) == 4 && N >= 3 && beside ? 2 * kHalfSMs : kWideCtas<N>;
+  return wide_fits<N>() && nblk_w * (N + 1) <= limit;
 }
 // Launch attributes of a stage kernel.  dependent: a programmatic dependent of
 // the kernel before it on the stream (inside a capture: a programmatic edge).
@@ -2400,7 +2406,7 @@ template <int N>
 int reverse_carve(const DevMesh<real>& m) {
   if (sizeof(real) == 8) return kCarveAll;
   if (m.nblk_t > 0) return 0;
-  const bool small = small_mesh_form<N>(m.nblk_w);
+  const bool small = small_mesh_form<N>(m.nblk_w, true);
   if ((small ? m.nblk_w * (N + 1) : m.nblk_w) > 2 * kHalfSMs) return kCarveAll;
   const int stage = small ? wide_smem_bytes<N>() : wedge_smem_bytes<N, 1>();
   const int bytes = stage + grad_smem_bytes<N>() + 2 * 1024, sm = 228 * 1024;  // (1 KB per CTA is the system's)
@@ -2469,7 +2475,7 @@ int launch_stage_n(const StageArgs<real>& a, bool rk, cudaStream_t s, cudaStream
       if (err != cudaSuccess) return int(err);
     }
     if constexpr (wide_fits<N>()) {
-      if (!done && a.wedge_bpc <= 1 && small_mesh_form<N>(a.m.nblk_w)) {
+      if (!done && a.wedge_bpc <= 1 && small_mesh_form<N>(a.m.nblk_w, fork || a.reverse)) {
         const cudaError_t err = launch_dependent(k_wedge_wide<N>, a.m.nblk_w * (N + 1), 128, wide_smem_bytes<N>(), s,
                                                  a.pdl && a.m.nblk_t == 0, carve, a, rk);
         if (err != cudaSuccess) return int(err);
