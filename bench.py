@@ -85,6 +85,18 @@ def _alg_bytes_per_stage(K, total_nodes, real_bytes=4):
     return 4 * real_bytes * (4 * total_nodes) + 64 * K
 
 
+def _skipped_bytes_per_step(total_nodes, real_bytes=4):
+    """What a five-stage step leaves out of five full stages: its first stage
+    (a = 0) reads no residual and its last one stores none, 4 reals per node
+    each."""
+    return 2 * real_bytes * 4 * total_nodes
+
+
+def _mean_stage_bytes(stage_bytes, total_nodes, real_bytes=4):
+    """Mean bytes of a step's five stages, from those of a full stage."""
+    return stage_bytes - _skipped_bytes_per_step(total_nodes, real_bytes) / 5
+
+
 def _kernel_bytes_per_stage(K, nverts, total_nodes, real_bytes=4, N=3, mass="stored"):
     """What this kernel design reads and writes at least (above the method's
     minimum: its own choices): the state as above; per wedge 12 vertex
@@ -101,22 +113,27 @@ def _kernel_bytes_per_stage(K, nverts, total_nodes, real_bytes=4, N=3, mass="sto
 
 
 def _flops_per_wedge(N, mass="stored"):
-    """Arithmetic of one wedge in one stage as the stage kernel performs it
-    (an FMA counts 2), per slice j of the N + 1 slices: D_t on 4 fields
-    (8 Nt Nq), the t-part and triangle-lift assembly (28 Nt), M^tri on 4
-    vectors (8 Nt^2), the two triangular solves with 4 right-hand sides
-    (8 Nt (Nt - 1) + 16 Nt), the strong D_r / D_s part (8 Nt^2 + 16 Nt), the
-    three quadrilateral faces (fluxes 18 Nq, edge masses 8 Nq^2 each), the
-    triangle-face fluxes (15 per node, 2 Nt / Nq nodes per slice) and the
-    fused update (24 Nt); plus about 150 flops of geometry per wedge and, with
-    the factor computed in the stage, the Cholesky factorisation
-    (Nt^3 / 3 + 3 Nt^2 per wedge)."""
+    """Arithmetic of one wedge in one stage as the FP32 stage kernel performs it
+    (an FMA counts 2; operator rows in packed pairs, padded to pr rows), per
+    slice j of the N + 1 slices: D_t on 4 fields (8 Nt Nq) and the t-divergence
+    (5 Nt); M^tri on 2 vectors per slice and on the wedge's 4 triangle-face flux
+    vectors ((4 + 8 / Nq) Nt pr); the lifts into the four right-hand sides
+    (19 Nt + 15 Nq); the three quadrilateral faces (fluxes 13 Nq, edge masses 7
+    per entry); the two triangular sweeps and the diagonal with 4 right-hand
+    sides (8 Nt (Nt - 1) + 4 Nt); the strong part (velocity transform 6 Nt, D_r
+    and D_s on two vectors each without the pairs of zero rows of D_r, sums
+    9 Nt); the triangle-face fluxes (17 per node, 2 Nt / Nq nodes per slice) and
+    the fused update (28 Nt); plus about 150 flops of geometry per wedge and,
+    with the factor computed in the stage, its L D L^T (5 per entry of
+    M^{tri,k}, then Nt^3 / 3 + 3 Nt^2 / 2)."""
     nt, nq = (N + 1) * (N + 2) // 2, N + 1
-    per_slice = (8 * nt * nq + 28 * nt + 8 * nt * nt + 8 * nt * (nt - 1) + 16 * nt + 8 * nt * nt + 16 * nt
-                 + 3 * (18 * nq + 8 * nq * nq) + 15 * 2 * nt / nq + 24 * nt)
+    pr, qr = nt + nt % 2, nq + nq % 2
+    dr = nq * pr + (nt - nq) * (pr - 2 * (nq // 2))  # entries of D_r: past the edge b = 0 its first row pairs are zero
+    per_slice = (8 * nt * nq + 5 * nt + 4 * nt * pr + 8 * nt * pr / nq + 19 * nt + 15 * nq + 3 * (13 * nq + 7 * nq * qr)
+                 + 8 * nt * (nt - 1) + 4 * nt + 6 * nt + 4 * (dr + nt * pr) + 9 * nt + 17 * 2 * nt / nq + 28 * nt)
     f = nq * per_slice + 150
     if mass != "stored":
-        f += nt ** 3 / 3 + 3 * nt * nt
+        f += 5 * nt * (nt + 1) / 2 + nt ** 3 / 3 + 1.5 * nt * nt
     return f
 
 
@@ -772,8 +789,8 @@ def run_ours(args, rank, world):
     ms_step = r3["ms_max"] / args.steps
     value = _gdofs(r3["dof"], 5 * args.steps, r3["ms_max"] / 1e3, world)
     stage_s = r3["ms"] / 1e3 / (5 * args.steps)
-    alg = _alg_bytes_per_stage(K, r3["dof"] // 4)
-    kbytes = _kernel_bytes_per_stage(K, nverts, r3["dof"] // 4, N=orders[0], mass=args.mass)
+    alg = _mean_stage_bytes(_alg_bytes_per_stage(K, r3["dof"] // 4), r3["dof"] // 4)
+    kbytes = _mean_stage_bytes(_kernel_bytes_per_stage(K, nverts, r3["dof"] // 4, N=orders[0], mass=args.mass), r3["dof"] // 4)
     achieved = alg / stage_s / 1e9
 
     def flop_rate(N, mode, st):
@@ -784,8 +801,8 @@ def run_ours(args, rank, world):
     by_order = {}
     for N, r in out.items():
         st = r["ms"] / 1e3 / (5 * args.steps)
-        a = _alg_bytes_per_stage(K, r["dof"] // 4)
-        kb = _kernel_bytes_per_stage(K, nverts, r["dof"] // 4, N=N, mass=args.mass)
+        a = _mean_stage_bytes(_alg_bytes_per_stage(K, r["dof"] // 4), r["dof"] // 4)
+        kb = _mean_stage_bytes(_kernel_bytes_per_stage(K, nverts, r["dof"] // 4, N=N, mass=args.mass), r["dof"] // 4)
         by_order[str(N)] = {"autotune": r["autotune"],
                             "value": _gdofs(r["dof"], 5 * args.steps, r["ms_max"] / 1e3, world),
                             "ms_per_step": r["ms_max"] / args.steps, "stage_us": st * 1e6,
@@ -797,8 +814,8 @@ def run_ours(args, rank, world):
     if alt is not None:
         for mode, r in ((args.mass, r3), (other, alt)):
             st = r["ms"] / 1e3 / (5 * args.steps)
-            a = _alg_bytes_per_stage(K, r["dof"] // 4)
-            kb = _kernel_bytes_per_stage(K, nverts, r["dof"] // 4, N=orders[0], mass=mode)
+            a = _mean_stage_bytes(_alg_bytes_per_stage(K, r["dof"] // 4), r["dof"] // 4)
+            kb = _mean_stage_bytes(_kernel_bytes_per_stage(K, nverts, r["dof"] // 4, N=orders[0], mass=mode), r["dof"] // 4)
             by_mass[mode] = {"value": _gdofs(r["dof"], 5 * args.steps, r["ms_max"] / 1e3, world), "stage_us": st * 1e6,
                              "alg_bytes_per_stage": a, "frac": a / st / 1e9 / peak,
                              "kernel_bytes_per_stage": kb, "kernel_bytes_frac": kb / st / 1e9 / peak,
@@ -818,9 +835,11 @@ def run_ours(args, rank, world):
                      "traffic": _traffic_per_launch(args.mass) if (args.workload == "full" and orders[0] == 3
                                                                    and args.element_order == "column") else None,
                      "alg_bytes_per_launch": alg,
-                     "alg_bytes": "the method's minimum: 16 B per field-DOF (read q and res, write res and q) "
-                                  "+ 64 B per wedge of mesh data",
+                     "alg_bytes": "the method's minimum, mean of a step's five stages: 16 B per field-DOF (read q "
+                                  "and res, write res and q) less the residual that the first stage does not read "
+                                  "and the last does not store, + 64 B per wedge of mesh data",
                      "kernel_bytes_per_launch": kbytes,
+                     "traffic_of": "an inner stage (ncu), which reads and writes the residual",
                      "kernel_bytes": "what this kernel must move: the state as above, 100 B of mesh tables per "
                                      "wedge and the stored mass factor (overhead above the method's minimum)",
                      "alu": by_order[str(orders[0])]["alu"]},
