@@ -19,7 +19,7 @@ __device__ __forceinline__ int64_t pidx(const DevMesh<real>& M, int type, int e,
 // Bound by latency (a few hundred receivers, scattered 4-byte reads), so a
 // warp takes one receiver and its lanes the nodes: one exposed memory latency
 // instead of a chain of Np dependent adds on one thread's loads (256
-// receivers, N = 3: 14.3 -> 4.7 us).
+// receivers, N = 3: 14.3 -> 4.6 us).
 template <int N>
 __global__ void __launch_bounds__(128) k_sample(const DevMesh<real> M, const real* __restrict__ q, real* __restrict__ out,
                                                 int nshots) {
@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(128) k_sample(const DevMesh<real> M, const rea
 // the next stage input x += b5 times the same.  A warp takes one (shot, element
 // group), its lanes the nodes, receivers of a group in list order:
 // deterministic.  Latency bound like the sampling (256 receivers, N = 3, one
-// thread per group: 82.7 -> 8.8 us).
+// thread per group: 82.7 -> 8.2 us).
 template <int N>
 __global__ void __launch_bounds__(128) k_inject(const DevMesh<real> M, real* __restrict__ muq, real* __restrict__ x,
                                                 const real* __restrict__ resid, int nshots, real b5) {

@@ -838,10 +838,10 @@ __device__ __forceinline__ void quad_edge(const AllOps<N, real>& O, const real* 
 // neighbours from global memory, also those in its own block (no per-lane
 // choice between two address spaces), and a boundary face reads its own trace.
 // Bound by memory latency and traffic at N <= 3 (a copy of the slabs and the
-// traces alone takes 218 us of the 240 at N = 3), by issue and registers at
+// traces alone takes 218 us of the 243 at N = 3), by issue and registers at
 // N >= 4.  Instructions per warp, N = 3: 2,769 -> 2,240.  us per stage of a step
 // on 524,288 wedges, with the skipped residual traffic and the prefetch: N = 3
-// 298 -> 239, N = 4 769 -> 578; 30,118 wedges N = 5 326 -> 125.
+// 301 -> 243, N = 4 774 -> 583; 30,118 wedges N = 5 326 -> 125.
 // TF: the neighbour nodes of the triangle-face fluxes come from global memory
 // and are requested before the slab arrives (meshes where some of them are
 // tets or lie in another block, StageArgs::tri_far; two blocks per CTA:

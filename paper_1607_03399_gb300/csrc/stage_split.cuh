@@ -8,11 +8,11 @@
 // record, so the update moves 8-byte pairs).  Each thread keeps the
 // weak-form accumulators of two fields only (2 Nt instead of 4 Nt), so twice
 // the warps can be resident where the one-thread-per-slice kernel is limited
-// by registers (N = 4).  A launch variant of dg_autotune: at N = 4 on the
-// 524,288-wedge workload, both on packed pairs, it measured 1248 us per stage
-// against 1061 us for the one-thread form (96 registers with spills, duplicated
-// face gathers; the one-thread form has since come to 585 us), so it is not the
-// default.  Work split:
+// by registers (N = 4).  A launch variant of dg_autotune and never the faster
+// one as measured (96 registers with spills, duplicated face gathers, M^tri on
+// four vectors per slice): us per stage, this against the one-thread form, 199,712
+// wedges N = 2 133 / 51, N = 3 283 / 103, N = 4 485 / 235, 131,072 wedges N = 5
+// 1,311 / 431, 8,192 wedges N = 1 7.3 / 6.2.  Work split:
 //   fluxes: both halves form the quadrilateral-face jumps of their slice
 //     (the same neighbour traces); h = 0 lifts F_p and n_x F_u, h = 1 n_y F_u;
 //     the triangle-face node fluxes are spread over all warps;
