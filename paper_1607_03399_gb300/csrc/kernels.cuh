@@ -2565,9 +2565,14 @@ int DGW_CAT(launch_grad_, REALNS)(const DevMesh<REAL>& m, const REAL* x, const R
   if (m.nblk_w > 0) {
     constexpr int bytes = REALNS::grad_smem_bytes<NORD>();
     if (bytes > 227 * 1024) return int(cudaErrorInvalidConfiguration);
-    auto kernel = m.nblk_t > 0 ? REALNS::k_wedge_grad<NORD, true> : REALNS::k_wedge_grad<NORD, false>;
-    return int(REALNS::launch_kernel(kernel, m.nblk_w, 32 * (NORD + 1), bytes, cudaStream_t(stream),
-                                     REALNS::LaunchAttrs(false, REALNS::reverse_carve<NORD>(m)), m, x, q, r, dt, flux, bc, gk, gr, gz));
+    constexpr int threads = 32 * (NORD + 1);
+    const REALNS::LaunchAttrs attrs(false, REALNS::reverse_carve<NORD>(m));
+    const cudaStream_t s = cudaStream_t(stream);
+    if (m.nblk_t > 0)
+      return int(REALNS::launch_kernel(REALNS::k_wedge_grad<NORD, true>, m.nblk_w, threads, bytes, s, attrs, m, x, q, r, dt, flux,
+                                       bc, gk, gr, gz));
+    return int(REALNS::launch_kernel(REALNS::k_wedge_grad<NORD, false>, m.nblk_w, threads, bytes, s, attrs, m, x, q, r, dt, flux,
+                                     bc, gk, gr, gz));
   }
   return 0;
 }
